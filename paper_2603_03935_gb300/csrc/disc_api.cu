@@ -422,6 +422,7 @@ disc_status runner_init(Runner& r, int device, cudaStream_t stream, int D, int P
         bs.sMMD = (long long)MM * D;
         bs.sS = 5LL * MM;
         bs.scap = (long long)scap;
+        bs.spx = (long long)npx;
         bs.sK = r.Kpad;
         Scratch& sc = bs.base;
         sc.sumF = a.get<long long>((size_t)B * D);
@@ -451,15 +452,16 @@ disc_status runner_init(Runner& r, int device, cudaStream_t stream, int D, int P
         sc.ang = a.get<long long>((size_t)B * MM);
         sc.nvox = a.get<int32_t>((size_t)B * MM);
         sc.segrep = a.get<int32_t>((size_t)B * MM);
-        sc.sslot = a.get<SegSlot>((size_t)B * scap);
-        sc.sent = a.get<unsigned long long>((size_t)B * scap);
-        sc.slist = a.get<int32_t>((size_t)B * scap);
-        sc.elab = a.get<int32_t>((size_t)B * scap);
+        sc.sparts = seg_parts((long long)npx);
+        sc.srec = a.get<SegRec>((size_t)B * ((size_t)sc.sparts * SEG_REGION + npx));
+        sc.scur = a.get<int32_t>((size_t)B * (sc.sparts + 1) * SEG_CUR);
+        sc.sent = a.get<unsigned long long>((size_t)B * npx);
+        sc.elab = a.get<int32_t>((size_t)B * npx);
         sc.smask = scap - 1;
         sc.pkey = a.get<unsigned long long>((size_t)B * scap);
         sc.pcnt = a.get<int32_t>((size_t)B * scap);
         sc.plist = a.get<int32_t>((size_t)B * scap);
-        sc.aent = a.get<int32_t>((size_t)B * 2 * scap);  // per slot: aent [scap], aslot [scap]
+        sc.aent = a.get<int32_t>((size_t)B * 2 * npx);  // per slot: aent [px], aslot [px]
         sc.newcnt = a.get<int32_t>((size_t)B * MM);
         sc.ctr = a.get<FrameCounters>(B);
     }
@@ -548,7 +550,7 @@ disc_status runner_init(Runner& r, int device, cudaStream_t stream, int D, int P
         CK(cudaMemsetAsync(sc.qmul, 0, sizeof(float) * (size_t)B * r.Kpad, s));
         CK(cudaMemsetAsync(sc.qexpm, 0, sizeof(int32_t) * (size_t)B * MM, s));
         CK(cudaMemsetAsync(sc.cov, 0, sizeof(int32_t) * (size_t)B * MM * P, s));
-        CK(cudaMemsetAsync(sc.sslot, 0, sizeof(SegSlot) * B * scap, s));
+        CK(cudaMemsetAsync(sc.scur, 0, sizeof(int32_t) * (size_t)B * (sc.sparts + 1) * SEG_CUR, s));
         CK(cudaMemsetAsync(sc.pkey, 0xff, sizeof(unsigned long long) * B * scap, s));
         CK(cudaMemsetAsync(sc.pcnt, 0, sizeof(int32_t) * B * scap, s));
         CK(cudaMemsetAsync(sc.newcnt, 0, sizeof(int32_t) * B * MM, s));
@@ -658,7 +660,6 @@ disc_status ensure_dbscan(Runner& r)
         sc.dflag = a.get<unsigned char>(B * px);
         sc.dsp = a.get<float4>(B * px);
         sc.dund = a.get<int32_t>(B * px);
-        r.bs[k].spx = (long long)px;
     }
     if (a.failed) {
         a.failed = false;
@@ -1023,7 +1024,7 @@ int enqueue_stateless(Runner& r, int k, int S, int combos, cudaStream_t st, int 
                 run_phase(r, PH_DBSCAN, st, [&] { return launch_dbscan(dfp, bs, f0, nb, r.Hmax, r.Wmax, st); });
             run_phase(r, PH_BACKPROJECT, st, [&] { return launch_backproject(dfp, bs, f0, nb, r.Hmax, r.Wmax, st); });
             run_phase(r, PH_ENTRIES, st,
-                      [&] { return launch_entries(dfp, bs, refs, f0, nb, Mmax, (combos & COMBO_DILATE) != 0, st); });
+                      [&] { return launch_entries(dfp, bs, refs, f0, nb, (combos & COMBO_DILATE) != 0, st); });
         }
         run_phase(r, PH_ENTRIES, st, [&] { return launch_quality(dfp, bs, S, st); });
     }

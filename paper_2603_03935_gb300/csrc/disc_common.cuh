@@ -51,9 +51,38 @@ __device__ __forceinline__ long long fix32f(float x, int S)
     const long long v = (long long)((b & 0x7fffffu) | 0x800000u) << e;
     return (b >> 31) ? -v : v;
 }
+// The same for |x| <= 2 and S = 32, without divergence: y = x * 2^32 splits
+// exactly into hi * 2^24 + rem, hi = y / 2^24 rounded to an integer (adding
+// 1.5 * 2^23 leaves it in the low bits of the sum) and |rem| <= 2^23, whose
+// conversion rounds to nearest, ties to even (hi * 2^24 is even, so a tie of
+// rem is a tie of y).
+__device__ __forceinline__ long long fix32_unit(float x)
+{
+    const float t = __fmaf_rn(x, 256.0f, 12582912.0f);
+    const float rem = __fmaf_rn(__fsub_rn(12582912.0f, t), 16777216.0f, __fmul_rn(x, 4294967296.0f));
+    return (long long)(__float_as_int(t) - 0x4b400000) * 16777216 + (long long)__float2int_rn(rem);
+}
 __device__ __forceinline__ double unfix(long long n, int S)
 {
     return __dmul_rn(__ll2double_rn(n), __longlong_as_double((long long)(1023 - S) << 52));
+}
+
+// fp32 of n * 2^-S, rounded as double first and then as float.  Below 2^53
+// in magnitude the double is exact, so the value rounds once: its 32 leading
+// bits, the dropped ones gathered in the last of them, convert to fp32 (8
+// bits below the significand, so the gathered one decides ties only), then
+// an exact power of two.  Conversions from 64-bit integers run on the fp64
+// pipe, which this keeps idle.
+__device__ __forceinline__ float unfix32f(long long n, int S)
+{
+    const unsigned long long u = n < 0 ? 0ull - (unsigned long long)n : (unsigned long long)n;
+    if (u >> 53) return __double2float_rn(unfix(n, S));
+    if (u == 0) return 0.0f;
+    const int lz = __clzll((long long)u);
+    const unsigned long long m = u << lz;
+    const unsigned top = (unsigned)(m >> 32) | ((unsigned)m != 0u ? 1u : 0u);
+    const float f = __fmul_rn(__uint2float_rn(top), __int_as_float((127 + 32 - lz - S) << 23));
+    return n < 0 ? -f : f;
 }
 
 __device__ __forceinline__ unsigned long long mix64(unsigned long long z)
@@ -149,11 +178,20 @@ struct FrameCounters {
     int32_t n_copies;            // embeddings written (new instances and fusion winners)
 };
 
-// One slot of the per-frame (segment, voxel) hash: one 32-byte sector.
-struct __align__(32) SegSlot {
-    unsigned long long key;     // (mask << 54 | voxel key); 0 = empty
-    long long n[3];             // exact sums of the pixel normals (2^-32 fixed point)
+// One record of a frame's back-projection: pixels of one (segment, voxel),
+// one 32-byte sector.
+struct __align__(32) SegRec {
+    unsigned long long key;     // (mask << 54 | voxel key), never 0
+    long long n[3];             // exact sum of their normals (2^-32 fixed point)
 };
+// A frame's records are spread by their key's hash over one partition per
+// SEG_PART_PX pixels; k_entries gathers each in shared memory.  A region
+// holds SEG_REGION records (every pixel valid and its own record: 512 +- 23
+// of them); records past it go to the frame's overflow list, which holds one
+// per pixel, so no frame runs out of room.
+constexpr int SEG_PART_PX = 512, SEG_REGION = 768;
+constexpr int SEG_CUR = 32;  // ints from one partition counter to the next: each on a cache line of its own
+__host__ __device__ __forceinline__ int seg_parts(long long px) { return (int)((px + SEG_PART_PX - 1) / SEG_PART_PX); }
 
 // Per-frame scratch of one frame slot (pointers already offset to the slot).
 struct Scratch {
@@ -187,11 +225,12 @@ struct Scratch {
     long long* ang;     // [MM]
     int32_t* nvox;      // [MM]
     int32_t* segrep;    // [MM]
-    // per-frame (segment, voxel) hash, cleared slot by slot before reuse
-    SegSlot* sslot;             // [scap] key (mask << 54 | voxel key; EMPTY = 0) + normal sums
-    int32_t* slist;             // [scap] used slots, in claim order (entry i -> slot)
-    unsigned long long* sent;   // [scap] key of entry i (dense copy of the slot key)
-    int32_t* elab;              // [scap] per entry: label at batch start, -1 absent
+    // per-frame (segment, voxel) records by partition (SegRec)
+    SegRec* srec;               // [sparts][SEG_REGION], then the overflow list [px]
+    int32_t* scur;              // [sparts] records of each partition, then [1] of the overflow list
+    int32_t sparts;             // partitions of the largest frame
+    unsigned long long* sent;   // [px] key of entry i, (mask << 54 | voxel key), each once
+    int32_t* elab;              // [px] per entry: label at batch start, -1 absent
     unsigned long long smask;
     // per-frame overlap items, counted over the whole batch before the frames
     // run in order (one hash per slot, capacity scap, cleared slot by slot):
@@ -201,8 +240,8 @@ struct Scratch {
     unsigned long long* pkey;   // [scap] EMPTY = ~0
     int32_t* pcnt;              // [scap] voxels of the item
     int32_t* plist;             // [scap] used slots, in claim order
-    int32_t* aent;              // [scap] entries absent at the batch start
-    int32_t* aslot;             // [scap] and their slot in the batch's absent-voxel hash (aent + scap)
+    int32_t* aent;              // [px] entries absent at the batch start
+    int32_t* aslot;             // [px] and their slot in the batch's absent-voxel hash (aent + px)
     // the items again, dense (k_items, once k_absent is done with aent and
     // aslot): ikey over aent | aslot, icnt over plist
     unsigned long long* ikey;   // [n_pre] item keys
@@ -259,16 +298,16 @@ struct BatchScratch {
         s.ang += f * sMM;
         s.nvox += f * sMM;
         s.segrep += f * sMM;
-        s.sslot += f * scap;
-        s.slist += f * scap;
-        s.sent += f * scap;
-        s.elab += f * scap;
+        s.srec += f * ((long long)s.sparts * SEG_REGION + spx);
+        s.scur += f * ((long long)s.sparts + 1) * SEG_CUR;
+        s.sent += f * spx;
+        s.elab += f * spx;
         if (s.pkey) {
             s.pkey += f * scap;
             s.pcnt += f * scap;
             s.plist += f * scap;
-            s.aent += f * 2 * scap;
-            s.aslot = s.aent + scap;
+            s.aent += f * 2 * spx;
+            s.aslot = s.aent + spx;
             s.ikey = (unsigned long long*)s.aent;
             s.icnt = s.plist;
             s.newcnt += f * sMM;

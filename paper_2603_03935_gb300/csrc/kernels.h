@@ -54,11 +54,11 @@ int launch_pool_gemm(const FrameParams* fps, const BatchScratch& bs, int B, int 
 int launch_backproject(const FrameParams* fps, const BatchScratch& bs, int f0, int nb, int H, int W, cudaStream_t st);
 // DBSCAN noise flags of frames [f0, f0 + nb) (frames without DBSCAN return at once)
 int launch_dbscan(const FrameParams* fps, const BatchScratch& bs, int f0, int nb, int H, int W, cudaStream_t st);
-int launch_entries(const FrameParams* fps, const BatchScratch& bs, const MapRefs* refs, int f0, int nb, int Mmax,
-                   bool lookup, cudaStream_t st);
+int launch_entries(const FrameParams* fps, const BatchScratch& bs, const MapRefs* refs, int f0, int nb, bool lookup,
+                   cudaStream_t st);
 int launch_quality(const FrameParams* fps, const BatchScratch& bs, int B, cudaStream_t st);
-// default frames per back-projection/entries/DBSCAN launch (their per-frame
-// hashes stay in L2); the runner's tuning may pick another
+// default frames per back-projection/entries/DBSCAN launch (their records
+// stay in L2); the runner's tuning may pick another
 constexpr int GEOMETRY_CHUNK = 8;
 
 // start of a batch's serial part: every map's edge and copy counters to zero

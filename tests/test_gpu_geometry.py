@@ -1,0 +1,92 @@
+"""Back-projection records and their gathering into (segment, voxel) entries,
+at the edges of the partitions: every frame's voxel sets, normals (S_angle)
+and counters equal the oracle's bit for bit."""
+import numpy as np
+import pytest
+
+import oracle
+from tests import common
+
+pytestmark = pytest.mark.gpu
+
+W, H, GRID, DIM = 64, 48, (6, 8), 32
+MASK64 = (1 << 64) - 1
+
+
+def _mix64(z):
+    z = (z + 0x9E3779B97F4A7C15) & MASK64
+    z = ((z ^ (z >> 30)) * 0xBF58476D1CE4E5B9) & MASK64
+    z = ((z ^ (z >> 27)) * 0x94D049BB133111EB) & MASK64
+    return z ^ (z >> 31)
+
+
+def _wall(width, height, z, tilt, voxel, f=50.0):
+    """Depth of a tilted wall and the voxel key of every pixel (fp32, as the library computes it)."""
+    u, v = np.meshgrid(np.arange(width, dtype=np.float32), np.arange(height, dtype=np.float32))
+    depth = (z + tilt * (u + 0.37 * v)).astype(np.float32)
+    inv_f, inv_s = np.float32(1) / np.float32(f), np.float32(1) / np.float32(voxel)
+    x = ((u + np.float32(0.5) - np.float32(width / 2)) * depth) * inv_f
+    y = ((v + np.float32(0.5) - np.float32(height / 2)) * depth) * inv_f
+    k = [np.floor(a * inv_s).astype(np.int64) + (1 << 17) for a in (x, y, depth)]
+    return depth, (k[0] << 36) | (k[1] << 18) | k[2]
+
+
+def _one_partition(keys, parts, masks):
+    """Labels that send every pixel's record to partition 0 (the key's top hash bits), so that it holds the whole
+    frame: more records than its region and more distinct keys than one walk takes."""
+    labels = np.zeros(keys.shape, np.uint16)
+    for i, key in enumerate(keys.reshape(-1).tolist()):
+        for m in range(1, masks + 1):
+            m = (m + 7 * i) % masks + 1
+            if ((_mix64((m << 54) | key) >> 32) * parts) >> 32 == 0:
+                labels.reshape(-1)[i] = m
+                break
+    assert (labels > 0).mean() > 0.99
+    return labels
+
+
+@pytest.mark.parametrize("case", ["one_voxel", "few_voxels", "rows", "distinct", "one_partition", "ragged", "smallest"])
+def test_records_at_the_partition_edges(case):
+    import torch
+    from paper_2603_03935_gb300 import DiscMap, device_frame
+    dev = torch.device("cuda:0")
+    rng = np.random.default_rng(3)
+    width, height, masks, voxel, z, tilt = W, H, 8, 0.02, 2.0, 0.004
+    if case == "one_voxel":      # every pixel of a tile in a voxel or two: tiles merge
+        voxel, z, tilt = 0.8, 0.3, 0.0
+    elif case == "few_voxels":   # merged tiles, voxels crossing tiles
+        voxel, z = 0.2, 1.0
+    elif case == "rows":         # half the pixels share their row neighbour's voxel: the merge rule's line
+        voxel, z, tilt = 0.08, 2.0, 0.0
+    elif case == "ragged":
+        width, height = 61, 35
+    elif case == "smallest":
+        width, height, masks = 3, 2, 2
+    elif case == "one_partition":
+        masks = 60
+    depth, keys = _wall(width, height, z, tilt, voxel)
+    if case == "one_partition":
+        labels = _one_partition(keys, -(-width * height // 512), masks)
+    else:
+        labels = ((np.arange(height)[:, None] // 6 + np.arange(width)[None, :] // 9) % masks + 1).astype(np.uint16)
+        depth[rng.uniform(size=depth.shape) < 0.03] = 0.0  # holes
+    tokens = rng.normal(size=(GRID[0] * GRID[1], DIM)).astype(np.float32)
+    cfg = dict(voxel_size=voxel, embed_dim=DIM, patch_h=GRID[0], patch_w=GRID[1], max_width=width, max_height=height,
+               max_masks=masks, min_mask_pixels=1, voxel_capacity=1 << 14, max_load=0.5, instance_capacity=256,
+               z_min=0.1, z_max=10.0, eps=1e-6, tau_cos=0.75, lambda_size=3.3, ov_num=1, ov_den=5)
+    gmap, omap = DiscMap(**cfg), oracle.OracleMap(**common.to_oracle_cfg(cfg))
+    intr = (50.0, 50.0, width / 2.0, height / 2.0)
+    for i in range(2):  # the second frame reuses the slot
+        pose = np.eye(4)
+        pose[0, 3] = 0.013 * i
+        fr = device_frame(torch.from_numpy(depth).to(dev), torch.from_numpy(labels.view(np.int16)).to(dev),
+                          torch.from_numpy(tokens).to(dev), pose, intr, masks)
+        st = gmap.integrate(fr)
+        o = omap.integrate(depth, labels, tokens, pose, intr, masks)
+        common.compare_frame(st, gmap.last_frame(), o, ctx=f"{case} frame {i}")
+    common.compare_maps(gmap, omap, ctx=case)
+    if case == "distinct":
+        assert st["unique_seg_voxels"] > 0.9 * st["valid_pixels"]
+    if case in ("one_voxel", "few_voxels"):
+        assert st["unique_seg_voxels"] < 0.2 * st["valid_pixels"]
+    gmap.close()
