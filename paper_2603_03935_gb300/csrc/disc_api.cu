@@ -430,8 +430,7 @@ disc_status runner_init(Runner& r, int device, cudaStream_t stream, int D, int P
         sc.gvec = a.get<float>((size_t)B * D);
         sc.gg = a.get<long long>(B);
         sc.nsum = a.get<long long>(B);
-        sc.dotg = a.get<long long>((size_t)B * P);
-        sc.ffp = a.get<long long>((size_t)B * P);
+        sc.tick = a.get<int32_t>((size_t)B * TOK_GROUPS);
         sc.nrm = a.get<float>((size_t)B * P);
         sc.Dp = a.get<float>((size_t)B * P);
         sc.cosg = a.get<float>((size_t)B * P);
@@ -492,8 +491,7 @@ disc_status runner_init(Runner& r, int device, cudaStream_t stream, int D, int P
             sc.gvec = a.get<float>((size_t)B * Da_);
             sc.gg = a.get<long long>(B);
             sc.nsum = a.get<long long>(B);
-            sc.dotg = a.get<long long>((size_t)B * Pa);
-            sc.ffp = a.get<long long>((size_t)B * Pa);
+            sc.tick = a.get<int32_t>((size_t)B * TOK_GROUPS);
             sc.nrm = a.get<float>((size_t)B * Pa);
             sc.Dp = a.get<float>((size_t)B * Pa);
             sc.cosg = a.get<float>((size_t)B * Pa);
@@ -999,7 +997,7 @@ int enqueue_stateless(Runner& r, int k, int S, int combos, cudaStream_t st, int 
     const int64_t before = r.launches;
     run_phase(r, PH_CLEAR, st, [&] { return launch_slot_clear(bs, S, D, r.MM, st); });
     run_phase(r, PH_TOKENS, st, [&] { return launch_token_stats(dfp, bs, S, P, D, any_bf16, any_f32, st); });
-    run_phase(r, PH_COVERAGE, st, [&] { return launch_coverage(dfp, bs, S, r.Ph, r.Pw, Mmax, st); });
+    run_phase(r, PH_COVERAGE, st, [&] { return launch_coverage(dfp, bs, S, r.Ph, r.Pw, r.Wmax, Mmax, st); });
     run_phase(r, PH_WEIGHTS, st, [&] { return launch_weights(dfp, bs, S, Mmax, st); });
     run_phase(r, PH_POOL_EXACT, st, [&] { return launch_pool_exact(dfp, bs, S, P, D, Mmax, any_bf16, any_f32, st); });
     run_phase(r, PH_POOL_GEMM, st, [&] { return launch_pool_gemm(dfp, bs, S, D, Mmax, any, st); });
@@ -1011,7 +1009,7 @@ int enqueue_stateless(Runner& r, int k, int S, int combos, cudaStream_t st, int 
         const FrameParams* dfa = r.fpa(k) + base;
         run_phase(r, PH_CLEAR, st, [&] { return launch_view_clear(va, S, r.Da, r.MM, st); });
         run_phase(r, PH_TOKENS, st, [&] { return launch_token_stats(dfa, va, S, r.Pa, r.Da, any_bf16, any_f32, st); });
-        run_phase(r, PH_COVERAGE, st, [&] { return launch_coverage(dfa, va, S, r.Pha, r.Pwa, Mmax, st); });
+        run_phase(r, PH_COVERAGE, st, [&] { return launch_coverage(dfa, va, S, r.Pha, r.Pwa, r.Wmax, Mmax, st); });
         run_phase(r, PH_WEIGHTS, st, [&] { return launch_weights(dfa, va, S, Mmax, st); });
         run_phase(r, PH_POOL_EXACT, st,
                   [&] { return launch_pool_exact(dfa, va, S, r.Pa, r.Da, Mmax, any_bf16, any_f32, st); });

@@ -34,6 +34,8 @@ constexpr int KEY_BITS = 18;
 constexpr int32_t KEY_BIAS = 1 << (KEY_BITS - 1);
 constexpr unsigned long long EMPTY_KEY = ~0ull;
 constexpr int MAX_MASKS = 256;
+constexpr int TOK_COLS = 256;   // columns of a column-sum block
+constexpr int TOK_GROUPS = 16;  // column groups (D <= 4096)
 constexpr int GEMM_MT = 128;    // token-dimension rows per GEMM tile
 constexpr int GEMM_KC = 32;     // patches per GEMM pipeline chunk
 
@@ -51,16 +53,19 @@ __device__ __forceinline__ long long fix32f(float x, int S)
     const long long v = (long long)((b & 0x7fffffu) | 0x800000u) << e;
     return (b >> 31) ? -v : v;
 }
-// The same for |x| <= 2 and S = 32, without divergence: y = x * 2^32 splits
-// exactly into hi * 2^24 + rem, hi = y / 2^24 rounded to an integer (adding
-// 1.5 * 2^23 leaves it in the low bits of the sum) and |rem| <= 2^23, whose
-// conversion rounds to nearest, ties to even (hi * 2^24 is even, so a tie of
-// rem is a tie of y).
-__device__ __forceinline__ long long fix32_unit(float x)
+// The same for |x| < 2^(52 - S), without divergence (values around 2^(31 - S)
+// run both sides of the above in most warps): y = x * 2^S splits exactly
+// into hi * 2^30 + rem, hi = y / 2^30 rounded to an integer (adding 1.5 * 2^23
+// leaves it in the low bits of the sum) and |rem| <= 2^29, whose conversion
+// rounds to nearest, ties to even (hi * 2^30 is even, so a tie of rem is a
+// tie of y).
+template <int S>
+__device__ __forceinline__ long long fix_split(float x)
 {
-    const float t = __fmaf_rn(x, 256.0f, 12582912.0f);
-    const float rem = __fmaf_rn(__fsub_rn(12582912.0f, t), 16777216.0f, __fmul_rn(x, 4294967296.0f));
-    return (long long)(__float_as_int(t) - 0x4b400000) * 16777216 + (long long)__float2int_rn(rem);
+    const float t = __fmaf_rn(x, __int_as_float((127 + S - 30) << 23), 12582912.0f);
+    const float y = __fmul_rn(x, __int_as_float((127 + S) << 23));
+    const float rem = __fmaf_rn(__fsub_rn(12582912.0f, t), 1073741824.0f, y);
+    return (long long)(__float_as_int(t) - 0x4b400000) * 1073741824 + (long long)__float2int_rn(rem);
 }
 __device__ __forceinline__ double unfix(long long n, int S)
 {
@@ -201,8 +206,7 @@ struct Scratch {
     float* gvec;        // [D]
     long long* gg;      // [1]
     long long* nsum;    // [1]
-    long long* dotg;    // [P]
-    long long* ffp;     // [P]
+    int32_t* tick;      // [TOK_GROUPS] column-sum blocks done, per group of TOK_COLS columns
     float* nrm;         // [P]
     float* Dp;          // [P]
     float* cosg;        // [P]
@@ -276,8 +280,7 @@ struct BatchScratch {
         s.gvec += f * sD;
         s.gg += f;
         s.nsum += f;
-        s.dotg += f * sP;
-        s.ffp += f * sP;
+        s.tick += f * TOK_GROUPS;
         s.nrm += f * sP;
         s.Dp += f * sP;
         s.cosg += f * sP;

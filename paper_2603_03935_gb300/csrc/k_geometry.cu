@@ -72,6 +72,7 @@ __global__ void k_slot_reset(BatchScratch bs, int B)
     const Scratch sc = bs.frame(b);
     *sc.gg = 0;
     *sc.nsum = 0;
+    for (int i = 0; i < TOK_GROUPS; i++) sc.tick[i] = 0;
     FrameCounters z = {};
     *sc.ctr = z;
 }
@@ -137,7 +138,7 @@ __device__ __forceinline__ void pixel_normal(const FrameParams& fp, const TilePo
                                          __fmul_rn(__fsub_rn(me.p[1], fp.t[1]), n[1])),
                                __fmul_rn(__fsub_rn(me.p[2], fp.t[2]), n[2]));
 #pragma unroll
-    for (int r = 0; r < 3; r++) nfix[r] = fix32_unit(vd > 0.0f ? -n[r] : n[r]);
+    for (int r = 0; r < 3; r++) nfix[r] = fix_split<S_VEC>(vd > 0.0f ? -n[r] : n[r]);
 }
 
 __global__ void __launch_bounds__(BP_THREADS) k_backproject(const FrameParams* fps, BatchScratch bs, int f0)
@@ -443,7 +444,7 @@ __global__ void __launch_bounds__(SEG_THREADS) k_entries(const FrameParams* fps,
                     if (!(term > 0.0f)) term = 0.0f;
                 }
             }
-            const long long tf = fix32_unit(term);
+            const long long tf = fix_split<S_VEC>(term);
             const unsigned hi = (unsigned)(tf >> 16), lo = (unsigned)(tf & 0xffff);
             if (hi) atomicAdd(&s_hi[m - 1], hi);
             if (lo) atomicAdd(&s_lo[m - 1], lo);

@@ -42,7 +42,8 @@ int launch_slot_clear(const BatchScratch& bs, int B, int D, int MM, cudaStream_t
 int launch_view_clear(const BatchScratch& bs, int B, int D, int MM, cudaStream_t st);
 int launch_token_stats(const FrameParams* fps, const BatchScratch& bs, int B, int P, int D, bool any_bf16,
                        bool any_f32, cudaStream_t st);
-int launch_coverage(const FrameParams* fps, const BatchScratch& bs, int B, int Ph, int Pw, int Mmax, cudaStream_t st);
+int launch_coverage(const FrameParams* fps, const BatchScratch& bs, int B, int Ph, int Pw, int Wmax, int Mmax,
+                    cudaStream_t st);
 int launch_weights(const FrameParams* fps, const BatchScratch& bs, int B, int Mmax, cudaStream_t st);
 int launch_pool_exact(const FrameParams* fps, const BatchScratch& bs, int B, int P, int D, int Mmax, bool any_bf16,
                       bool any_f32, cudaStream_t st);
