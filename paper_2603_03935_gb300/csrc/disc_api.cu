@@ -1000,7 +1000,7 @@ int enqueue_stateless(Runner& r, int k, int S, int combos, cudaStream_t st, int 
     run_phase(r, PH_COVERAGE, st, [&] { return launch_coverage(dfp, bs, S, r.Ph, r.Pw, r.Wmax, Mmax, st); });
     run_phase(r, PH_WEIGHTS, st, [&] { return launch_weights(dfp, bs, S, Mmax, st); });
     run_phase(r, PH_POOL_EXACT, st, [&] { return launch_pool_exact(dfp, bs, S, P, D, Mmax, any_bf16, any_f32, st); });
-    run_phase(r, PH_POOL_GEMM, st, [&] { return launch_pool_gemm(dfp, bs, S, D, Mmax, any, st); });
+    run_phase(r, PH_POOL_GEMM, st, [&] { return launch_pool_gemm(dfp, bs, S, P, D, Mmax, any, st); });
     if ((combos & COMBO_ASSOC) && r.Da) {
         // the association features: the same kernels on the second grid's
         // view (pixel-mean weights; frames of maps without it are inert)
@@ -1013,7 +1013,7 @@ int enqueue_stateless(Runner& r, int k, int S, int combos, cudaStream_t st, int 
         run_phase(r, PH_WEIGHTS, st, [&] { return launch_weights(dfa, va, S, Mmax, st); });
         run_phase(r, PH_POOL_EXACT, st,
                   [&] { return launch_pool_exact(dfa, va, S, r.Pa, r.Da, Mmax, any_bf16, any_f32, st); });
-        run_phase(r, PH_POOL_GEMM, st, [&] { return launch_pool_gemm(dfa, va, S, r.Da, Mmax, any, st); });
+        run_phase(r, PH_POOL_GEMM, st, [&] { return launch_pool_gemm(dfa, va, S, r.Pa, r.Da, Mmax, any, st); });
     }
     if (Mmax > 0) {
         for (int f0 = 0; f0 < S; f0 += r.geo_chunk) {

@@ -1345,75 +1345,6 @@ constexpr size_t ASSOC_SMEM = (size_t)APH * 16 + union_region_bytes(2 * APH, ASS
 constexpr int ASSOC_CLUSTER_MAX = 8;
 static_assert(ASSOC_EDGES >= 2 * ASSOC_ROOTS, "the fusion step overlays the edge arrays");
 
-// ---- distributed shared memory of a thread-block cluster (inline PTX) ------------
-// Addresses are 32-bit shared::cluster addresses: a CTA's own shared-memory
-// offset mapped to the CTA of the given rank (mapa).
-__device__ __forceinline__ unsigned dsm_map(const void* local, unsigned rank)
-{
-    unsigned out;
-    const unsigned a = (unsigned)__cvta_generic_to_shared(local);
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(out) : "r"(a), "r"(rank));
-    return out;
-}
-__device__ __forceinline__ unsigned long long dsm_cas64(unsigned a, unsigned long long cmp, unsigned long long v)
-{
-    unsigned long long old;
-    asm volatile("atom.shared::cluster.cas.b64 %0, [%1], %2, %3;" : "=l"(old) : "r"(a), "l"(cmp), "l"(v) : "memory");
-    return old;
-}
-__device__ __forceinline__ int dsm_add(unsigned a, int v)
-{
-    int old;
-    asm volatile("atom.shared::cluster.add.u32 %0, [%1], %2;" : "=r"(old) : "r"(a), "r"(v) : "memory");
-    return old;
-}
-__device__ __forceinline__ void dsm_red_add(unsigned a, int v)
-{
-    asm volatile("red.shared::cluster.add.u32 [%0], %1;" ::"r"(a), "r"(v) : "memory");
-}
-__device__ __forceinline__ unsigned long long dsm_ld64(unsigned a)
-{
-    unsigned long long v;
-    asm volatile("ld.shared::cluster.u64 %0, [%1];" : "=l"(v) : "r"(a) : "memory");
-    return v;
-}
-__device__ __forceinline__ int dsm_ld32(unsigned a)
-{
-    int v;
-    asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(a) : "memory");
-    return v;
-}
-__device__ __forceinline__ void dsm_st32(unsigned a, int v)
-{
-    asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(a), "r"(v) : "memory");
-}
-__device__ __forceinline__ void dsm_st64(unsigned a, unsigned long long v)
-{
-    asm volatile("st.shared::cluster.u64 [%0], %1;" ::"r"(a), "l"(v) : "memory");
-}
-__device__ __forceinline__ unsigned cluster_rank()
-{
-    unsigned r;
-    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-    return r;
-}
-__device__ __forceinline__ unsigned cluster_size()
-{
-    unsigned n;
-    asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(n));
-    return n;
-}
-// every thread of every CTA of the cluster; shared-memory and global writes
-// before it are visible to the cluster after it (release / acquire)
-__device__ __forceinline__ void cluster_sync()
-{
-    asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
-}
-// the two halves of cluster_sync: between them a thread may read what no
-// other thread of the cluster writes in this phase
-__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
-__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
-
 // A cluster of C CTAs per map of the batch (C = cluster size, 1 to 8)
 // walks the map's frames in order.  The leader CTA (rank 0) holds the
 // frame's pair hash, scored-pair list, edge list and union state in its

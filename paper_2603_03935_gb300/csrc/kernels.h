@@ -48,7 +48,7 @@ int launch_weights(const FrameParams* fps, const BatchScratch& bs, int B, int Mm
 int launch_pool_exact(const FrameParams* fps, const BatchScratch& bs, int B, int P, int D, int Mmax, bool any_bf16,
                       bool any_f32, cudaStream_t st);
 // one launch per (token dtype, precision) present: any[tok_bf16][prec_bf16]
-int launch_pool_gemm(const FrameParams* fps, const BatchScratch& bs, int B, int D, int Mmax, const bool any[2][3],
+int launch_pool_gemm(const FrameParams* fps, const BatchScratch& bs, int B, int P, int D, int Mmax, const bool any[2][3],
                      cudaStream_t st);
 // back-projection and the per-entry pass (S_angle terms, |V_m|, labels at
 // batch start) on frames [f0, f0 + nb); then Q of every segment
@@ -89,7 +89,6 @@ int launch_commit(const BatchScratch& bs, const SerialStep& st, const AbsentHash
 size_t union_region_bytes_full();
 
 size_t coverage_smem_bytes(int max_masks, int Pw);
-size_t gemm_smem_bytes(int NT);
 cudaError_t set_feature_kernel_attrs(int max_dyn_smem);
 cudaError_t set_gemm_kernel_attrs();
 cudaError_t set_gemm_stall(bool on);
