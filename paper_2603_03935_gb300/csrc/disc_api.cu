@@ -134,6 +134,9 @@ struct Runner {
     cudaStream_t stream = nullptr;   // the caller's stream (everything when not pipelined)
     cudaStream_t stream2 = nullptr;  // stateless part of pipelined batches, lowest priority
     cudaStream_t stream3 = nullptr;  // serial part of pipelined batches, highest priority
+    // branches of the stateless part: back-projection, entries, the second grid
+    cudaStream_t branch[3] = {};
+    cudaEvent_t ev_clear = nullptr, ev_cover = nullptr, ev_geo = nullptr, ev_branch[2] = {};
     cudaEvent_t ev_join = nullptr;   // call start on the caller's stream, call end on stream3
     CUgreenCtx green[2] = {};        // SM partitions of stream3 / stream2 (when the driver offers them)
     int serial_sms = -1;             // SMs of the serial partition; < 0: no pipelining
@@ -524,6 +527,17 @@ disc_status runner_init(Runner& r, int device, cudaStream_t stream, int D, int P
         CK(cudaStreamCreateWithPriority(&r.stream2, cudaStreamNonBlocking, prio_lo));
         CK(cudaStreamCreateWithPriority(&r.stream3, cudaStreamNonBlocking, prio_hi));
     }
+    if (!r.green[0]) {  // (an SM partition keeps its stateless part on its own stream)
+        int prio_lo = 0, prio_hi = 0;
+        CK(cudaDeviceGetStreamPriorityRange(&prio_lo, &prio_hi));
+        for (int i = 0; i < 3; i++) {
+            CK(cudaStreamCreateWithPriority(&r.branch[i], cudaStreamNonBlocking, prio_lo));
+            if (i < 2) CK(cudaEventCreateWithFlags(&r.ev_branch[i], cudaEventDisableTiming));
+        }
+        CK(cudaEventCreateWithFlags(&r.ev_clear, cudaEventDisableTiming));
+        CK(cudaEventCreateWithFlags(&r.ev_cover, cudaEventDisableTiming));
+        CK(cudaEventCreateWithFlags(&r.ev_geo, cudaEventDisableTiming));
+    }
     CK(cudaEventCreateWithFlags(&r.ev_join, cudaEventDisableTiming));
     CK(cudaStreamCreateWithFlags(&r.stream_in, cudaStreamNonBlocking));
     CK(cudaHostAlloc(&r.h_room, sizeof(unsigned long long) * 2 * Gmax, cudaHostAllocDefault));
@@ -570,15 +584,17 @@ disc_status runner_init(Runner& r, int device, cudaStream_t stream, int D, int P
 void runner_release(Runner& r)
 {
     cudaStreamSynchronize(r.stream);
-    for (cudaStream_t* sp : {&r.stream2, &r.stream3, &r.stream_in}) {
+    for (cudaStream_t* sp : {&r.stream2, &r.stream3, &r.stream_in, &r.branch[0], &r.branch[1], &r.branch[2]}) {
         if (*sp) {
             cudaStreamSynchronize(*sp);
             cudaStreamDestroy(*sp);
             *sp = nullptr;
         }
     }
-    if (r.ev_join) cudaEventDestroy(r.ev_join);
-    r.ev_join = nullptr;
+    for (cudaEvent_t* ep : {&r.ev_join, &r.ev_clear, &r.ev_cover, &r.ev_geo, &r.ev_branch[0], &r.ev_branch[1]}) {
+        if (*ep) cudaEventDestroy(*ep);
+        *ep = nullptr;
+    }
     if (r.ev_room) cudaEventDestroy(r.ev_room);
     r.ev_room = nullptr;
     if (r.h_room) cudaFreeHost(r.h_room);
@@ -982,7 +998,13 @@ constexpr int COMBO_DILATE = 1 << 8;  // some frame's map takes the neighbourhoo
                                       // frames run as four kernels each (overlap, score, union, apply)
 
 // slots [base, base + S) of set k (base > 0: the second half of a batch whose
-// halves wait for their own input copies)
+// halves wait for their own input copies).  The token kernels (st) and the
+// geometry kernels (branch 0; the entries of a chunk on branch 1, beside the
+// next chunk's back-projection) need nothing of each other but the coverage,
+// and the second grid (branch 2) only shares the frames: they run side by
+// side, which hides a small batch's launches (a single Room frame: 18 in a
+// row) and fills the SMs that a large one's last blocks leave.  With phase
+// timing everything runs in a row on st.
 int enqueue_stateless(Runner& r, int k, int S, int combos, cudaStream_t st, int base = 0)
 {
     const bool any_bf16 = (combos & 070) != 0, any_f32 = (combos & 07) != 0;  // bits 0-5
@@ -995,37 +1017,52 @@ int enqueue_stateless(Runner& r, int k, int S, int combos, cudaStream_t st, int 
     const FrameParams* dfp = r.fps(k) + base;
     const MapRefs* refs = r.refs(k);
     const int64_t before = r.launches;
+    const bool side = !r.timing && r.branch[0];
+    const bool geo = Mmax > 0, grid2 = (combos & COMBO_ASSOC) && r.Da;
+    cudaStream_t sg = side ? r.branch[0] : st, se = side ? r.branch[1] : st, sv = side ? r.branch[2] : st;
+    // b starts after what a holds now
+    auto after = [&](cudaStream_t b, cudaStream_t a, cudaEvent_t ev) {
+        if (a == b) return;
+        cudaEventRecord(ev, a);
+        cudaStreamWaitEvent(b, ev, 0);
+    };
     run_phase(r, PH_CLEAR, st, [&] { return launch_slot_clear(bs, S, D, r.MM, st); });
+    if (geo) after(sg, st, r.ev_clear);
+    if (grid2) after(sv, st, r.ev_clear);
     run_phase(r, PH_TOKENS, st, [&] { return launch_token_stats(dfp, bs, S, P, D, any_bf16, any_f32, st); });
-    run_phase(r, PH_COVERAGE, st, [&] { return launch_coverage(dfp, bs, S, r.Ph, r.Pw, r.Wmax, Mmax, st); });
+    run_phase(r, PH_COVERAGE, sg, [&] { return launch_coverage(dfp, bs, S, r.Ph, r.Pw, r.Wmax, Mmax, sg); });
+    if (geo) after(st, sg, r.ev_cover);
     run_phase(r, PH_WEIGHTS, st, [&] { return launch_weights(dfp, bs, S, Mmax, st); });
     run_phase(r, PH_POOL_EXACT, st, [&] { return launch_pool_exact(dfp, bs, S, P, D, Mmax, any_bf16, any_f32, st); });
     run_phase(r, PH_POOL_GEMM, st, [&] { return launch_pool_gemm(dfp, bs, S, P, D, Mmax, any, st); });
-    if ((combos & COMBO_ASSOC) && r.Da) {
+    if (grid2) {
         // the association features: the same kernels on the second grid's
         // view (pixel-mean weights; frames of maps without it are inert)
         BatchScratch va = r.bsa[k];
         va.base = r.bsa[k].frame(base);
         const FrameParams* dfa = r.fpa(k) + base;
-        run_phase(r, PH_CLEAR, st, [&] { return launch_view_clear(va, S, r.Da, r.MM, st); });
-        run_phase(r, PH_TOKENS, st, [&] { return launch_token_stats(dfa, va, S, r.Pa, r.Da, any_bf16, any_f32, st); });
-        run_phase(r, PH_COVERAGE, st, [&] { return launch_coverage(dfa, va, S, r.Pha, r.Pwa, r.Wmax, Mmax, st); });
-        run_phase(r, PH_WEIGHTS, st, [&] { return launch_weights(dfa, va, S, Mmax, st); });
-        run_phase(r, PH_POOL_EXACT, st,
-                  [&] { return launch_pool_exact(dfa, va, S, r.Pa, r.Da, Mmax, any_bf16, any_f32, st); });
-        run_phase(r, PH_POOL_GEMM, st, [&] { return launch_pool_gemm(dfa, va, S, r.Pa, r.Da, Mmax, any, st); });
+        run_phase(r, PH_CLEAR, sv, [&] { return launch_view_clear(va, S, r.Da, r.MM, sv); });
+        run_phase(r, PH_TOKENS, sv, [&] { return launch_token_stats(dfa, va, S, r.Pa, r.Da, any_bf16, any_f32, sv); });
+        run_phase(r, PH_COVERAGE, sv, [&] { return launch_coverage(dfa, va, S, r.Pha, r.Pwa, r.Wmax, Mmax, sv); });
+        run_phase(r, PH_WEIGHTS, sv, [&] { return launch_weights(dfa, va, S, Mmax, sv); });
+        run_phase(r, PH_POOL_EXACT, sv,
+                  [&] { return launch_pool_exact(dfa, va, S, r.Pa, r.Da, Mmax, any_bf16, any_f32, sv); });
+        run_phase(r, PH_POOL_GEMM, sv, [&] { return launch_pool_gemm(dfa, va, S, r.Pa, r.Da, Mmax, any, sv); });
     }
-    if (Mmax > 0) {
+    if (geo) {
         for (int f0 = 0; f0 < S; f0 += r.geo_chunk) {
             const int nb = std::min(r.geo_chunk, S - f0);
             if (combos & COMBO_DBSCAN)
-                run_phase(r, PH_DBSCAN, st, [&] { return launch_dbscan(dfp, bs, f0, nb, r.Hmax, r.Wmax, st); });
-            run_phase(r, PH_BACKPROJECT, st, [&] { return launch_backproject(dfp, bs, f0, nb, r.Hmax, r.Wmax, st); });
-            run_phase(r, PH_ENTRIES, st,
-                      [&] { return launch_entries(dfp, bs, refs, f0, nb, (combos & COMBO_DILATE) != 0, st); });
+                run_phase(r, PH_DBSCAN, sg, [&] { return launch_dbscan(dfp, bs, f0, nb, r.Hmax, r.Wmax, sg); });
+            run_phase(r, PH_BACKPROJECT, sg, [&] { return launch_backproject(dfp, bs, f0, nb, r.Hmax, r.Wmax, sg); });
+            after(se, sg, r.ev_geo);
+            run_phase(r, PH_ENTRIES, se,
+                      [&] { return launch_entries(dfp, bs, refs, f0, nb, (combos & COMBO_DILATE) != 0, se); });
         }
-        run_phase(r, PH_ENTRIES, st, [&] { return launch_quality(dfp, bs, S, st); });
+        after(st, se, r.ev_branch[0]);  // (the entries follow every back-projection)
     }
+    if (grid2) after(st, sv, r.ev_branch[1]);
+    if (geo) run_phase(r, PH_ENTRIES, st, [&] { return launch_quality(dfp, bs, S, st); });
     return (int)(r.launches - before);
 }
 

@@ -172,7 +172,7 @@ struct FrameCounters {
     int32_t err;                 // disc_status of the frame (0 = ok)
     int32_t next_id;             // instance ids handed out so far
     int32_t num_masks;           // of the frame
-    int32_t n_edges;
+    int32_t geo_err;             // first error of the geometry kernels (into err by k_quality)
     int32_t n_cells;             // DBSCAN grid cells of the frame
     int32_t denoised;            // pixels DBSCAN marked as noise
     int32_t db_left[2];          // DBSCAN points left to the warp-wide core / noise search

@@ -32,7 +32,7 @@ namespace disc {
 
 namespace {
 
-__device__ __forceinline__ void db_err(const Scratch& sc, int code) { atomicCAS(&sc.ctr->err, 0, code); }
+__device__ __forceinline__ void db_err(const Scratch& sc, int code) { atomicCAS(&sc.ctr->geo_err, 0, code); }
 
 __device__ __forceinline__ unsigned long long cell_key(int lab, int cx, int cy, int cz)
 {
@@ -155,7 +155,7 @@ __global__ void k_db_points(const FrameParams* fps, BatchScratch bs, int f0)
 {
     const FrameParams& fp = fps[f0 + blockIdx.y];
     const Scratch sc = bs.frame(f0 + blockIdx.y);
-    if (fp.db_min_pts <= 0 || fp.M <= 0 || sc.ctr->err) return;  // uniform per block
+    if (fp.db_min_pts <= 0 || fp.M <= 0 || sc.ctr->geo_err) return;  // uniform per block
     const int npx = fp.W * fp.H;
     const int idx = blockIdx.x * blockDim.x + threadIdx.x;
     const int lane = threadIdx.x & 31;
@@ -220,7 +220,7 @@ __global__ void k_db_ranges(const FrameParams* fps, BatchScratch bs, int f0)
 {
     const FrameParams& fp = fps[f0 + blockIdx.y];
     const Scratch sc = bs.frame(f0 + blockIdx.y);
-    if (fp.db_min_pts <= 0 || fp.M <= 0 || sc.ctr->err) return;
+    if (fp.db_min_pts <= 0 || fp.M <= 0 || sc.ctr->geo_err) return;
     const int n = sc.ctr->n_cells;
     const int lane = threadIdx.x & 31;
     for (int i0 = blockIdx.x * blockDim.x; i0 < n; i0 += gridDim.x * blockDim.x) {  // uniform per block
@@ -246,7 +246,7 @@ __global__ void k_db_scatter(const FrameParams* fps, BatchScratch bs, int f0)
 {
     const FrameParams& fp = fps[f0 + blockIdx.y];
     const Scratch sc = bs.frame(f0 + blockIdx.y);
-    if (fp.db_min_pts <= 0 || fp.M <= 0 || sc.ctr->err) return;
+    if (fp.db_min_pts <= 0 || fp.M <= 0 || sc.ctr->geo_err) return;
     const int npx = fp.W * fp.H;
     const int idx = blockIdx.x * blockDim.x + threadIdx.x;
     const int lane = threadIdx.x & 31;
@@ -267,7 +267,7 @@ __global__ void k_db_core(const FrameParams* fps, BatchScratch bs, int f0)
 {
     const FrameParams& fp = fps[f0 + blockIdx.y];
     const Scratch sc = bs.frame(f0 + blockIdx.y);
-    if (fp.db_min_pts <= 0 || fp.M <= 0 || sc.ctr->err) return;
+    if (fp.db_min_pts <= 0 || fp.M <= 0 || sc.ctr->geo_err) return;
     const int npx = fp.W * fp.H;
     const int idx = blockIdx.x * blockDim.x + threadIdx.x;
     bool left = false;
@@ -288,7 +288,7 @@ __global__ void k_db_core_full(const FrameParams* fps, BatchScratch bs, int f0)
 {
     const FrameParams& fp = fps[f0 + blockIdx.y];
     const Scratch sc = bs.frame(f0 + blockIdx.y);
-    if (fp.db_min_pts <= 0 || fp.M <= 0 || sc.ctr->err) return;
+    if (fp.db_min_pts <= 0 || fp.M <= 0 || sc.ctr->geo_err) return;
     const int n = sc.ctr->db_left[0], need = fp.db_min_pts;
     const int wpb = blockDim.x >> 5;
     for (int i = blockIdx.x * wpb + (threadIdx.x >> 5); i < n; i += gridDim.x * wpb) {  // uniform per warp
@@ -306,7 +306,7 @@ __global__ void k_db_noise(const FrameParams* fps, BatchScratch bs, int f0)
 {
     const FrameParams& fp = fps[f0 + blockIdx.y];
     const Scratch sc = bs.frame(f0 + blockIdx.y);
-    if (fp.db_min_pts <= 0 || fp.M <= 0 || sc.ctr->err) return;
+    if (fp.db_min_pts <= 0 || fp.M <= 0 || sc.ctr->geo_err) return;
     const int npx = fp.W * fp.H;
     const int idx = blockIdx.x * blockDim.x + threadIdx.x;
     bool left = false;
@@ -326,7 +326,7 @@ __global__ void k_db_noise_full(const FrameParams* fps, BatchScratch bs, int f0)
 {
     const FrameParams& fp = fps[f0 + blockIdx.y];
     const Scratch sc = bs.frame(f0 + blockIdx.y);
-    if (fp.db_min_pts <= 0 || fp.M <= 0 || sc.ctr->err) return;
+    if (fp.db_min_pts <= 0 || fp.M <= 0 || sc.ctr->geo_err) return;
     const int n = sc.ctr->db_left[1];
     const int wpb = blockDim.x >> 5;
     for (int i = blockIdx.x * wpb + (threadIdx.x >> 5); i < n; i += gridDim.x * wpb) {  // uniform per warp

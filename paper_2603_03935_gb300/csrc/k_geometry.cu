@@ -15,7 +15,9 @@
 
 namespace disc {
 
-__device__ __forceinline__ void set_err(FrameCounters* c, int code) { atomicCAS(&c->err, 0, code); }
+// The geometry kernels run beside the token kernels: they neither read nor set
+// the frame's err (which those may set meanwhile) but their own geo_err.
+__device__ __forceinline__ void set_err(FrameCounters* c, int code) { atomicCAS(&c->geo_err, 0, code); }
 
 // partition of a (mask, voxel) key with hash h (its top bits; the shared
 // hash of a partition and its splits take the low ones)
@@ -159,7 +161,7 @@ __global__ void __launch_bounds__(BP_THREADS) k_backproject(const FrameParams* f
     const int tid = threadIdx.y * BP_TX + threadIdx.x, lane = threadIdx.x;
     if (tid == 0) {
         s_valid = s_runs = s_dropped = s_listed = 0;
-        s_err = sc.ctr->err;
+        s_err = sc.ctr->geo_err;
     }
     {
         const unsigned act = __ballot_sync(0xffffffffu, tid < M && sc.npix[tid] >= fp.min_px);
@@ -507,10 +509,22 @@ __global__ void __launch_bounds__(SEG_THREADS) k_entries(const FrameParams* fps,
 }
 
 // ---- Eq. 2-3: S_angle = mean of the voxel terms; Q per segment -------------------
+// Runs after both the token and the geometry kernels: a frame that either
+// failed takes its error here, and its geometry counters read zero.
 __global__ void k_quality(const FrameParams* fps, BatchScratch bs)
 {
     const FrameParams& fp = fps[blockIdx.x];
     const Scratch sc = bs.frame(blockIdx.x);
+    const int err = sc.ctr->err ? sc.ctr->err : sc.ctr->geo_err;
+    if (err) {
+        __syncthreads();  // every thread has read both
+        if (threadIdx.x == 0) {
+            FrameCounters* c = sc.ctr;
+            c->err = err;
+            c->n_entries = c->valid_pixels = c->dropped_pixels = c->max_probe = c->denoised = 0;
+        }
+        return;
+    }
     int live = 0;
     for (int m = threadIdx.x; m < fp.M; m += blockDim.x) {
         float* S = sc.S + 5 * m;

@@ -849,7 +849,6 @@ __device__ bool union_frame(const FrameParams& fp, const Scratch& sc, const Seri
         ctr->active_instances = s_nroots;
         ctr->new_instances = s_new;
         ctr->merges = s_merges;
-        ctr->n_edges = nedge;
         ctr->next_id = s_next;
         ctr->n_copies = s_ncopy;
     }
