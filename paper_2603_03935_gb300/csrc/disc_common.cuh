@@ -122,6 +122,36 @@ __device__ __forceinline__ void unpack_key(unsigned long long key, int k[3])
     k[2] = (int)(key & mask) - KEY_BIAS;
 }
 
+// Slots of a voxel in a table of mask + 1 (a power of two).  The 2 x 2 x 2
+// voxels of a block have eight consecutive home slots (64 bytes of keys, 32 of
+// labels), so a surface's lookups read a fraction of the sectors that slots
+// hashed voxel by voxel do, and a voxel's neighbours lie in at most eight
+// places.  The probe sequence keeps the place within the eight and moves on
+// by whole groups: two blocks hashed to one group (half full, as surfaces
+// are) collide only where both hold a voxel, and the sequence's length is that
+// of plain hashing at the same load.  (Moving on slot by slot chained the
+// groups: a commit of 1,700 voxels at load 0.25 took 29 us in the place of
+// 15.)  After a whole round at one place it moves to the next, so every slot
+// is reached.
+__device__ __forceinline__ unsigned long long vt_home(unsigned long long key, unsigned long long mask)
+{
+    const unsigned long long low = (1ull << (2 * KEY_BITS)) | (1ull << KEY_BITS) | 1ull;
+    const unsigned long long local = ((key >> (2 * KEY_BITS - 2)) & 4) | ((key >> (KEY_BITS - 1)) & 2) | (key & 1);
+    return ((mix64(key & ~low) << 3) | local) & mask;
+}
+// the slot after h, the n-th of the sequence (n = 1 for the home slot)
+__device__ __forceinline__ unsigned long long vt_next(unsigned long long h, unsigned long long n,
+                                                      unsigned long long mask)
+{
+    return (h + ((n & (mask >> 3)) == 0 ? 9 : 8)) & mask;
+}
+// slot i of the sequence (i = 0: the home slot)
+__device__ __forceinline__ unsigned long long vt_slot(unsigned long long home, unsigned long long i,
+                                                      unsigned long long mask)
+{
+    return (home + 8 * i + (i >> __popcll(mask >> 3))) & mask;
+}
+
 template <typename T>
 __device__ __forceinline__ T warp_sum(T v)
 {

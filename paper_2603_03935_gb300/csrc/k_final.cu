@@ -29,12 +29,12 @@ __device__ __forceinline__ void fin_err(FinalizeScratch fs, int code) { atomicCA
 // label of a key in the table, or -2 when absent
 __device__ __forceinline__ int table_label(const VoxelTable& vt, unsigned long long key)
 {
-    unsigned long long h = mix64(key) & vt.mask;
+    unsigned long long h = vt_home(key, vt.mask);
     for (unsigned long long pr = 0; pr <= vt.mask; pr++) {
         const unsigned long long kk = vt.keys[h];
         if (kk == key) return vt.labels[h];
         if (kk == EMPTY_KEY) return -2;
-        h = (h + 1) & vt.mask;
+        h = vt_next(h, pr + 1, vt.mask);
     }
     return -2;
 }

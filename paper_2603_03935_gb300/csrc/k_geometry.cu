@@ -323,7 +323,7 @@ __global__ void __launch_bounds__(BP_THREADS) k_backproject(const FrameParams* f
 // per part.  Per-segment sums gather in shared memory first (one global
 // atomic per block and segment): each term t (0 <= t <= 2^32 in 2^-32 fixed
 // point) adds as its two 16-bit halves, whose block sums stay below 2^31.
-// lookup = 0: the labels are left to k_lookup, which runs once the previous
+// Without LOOKUP the labels are left to k_lookup, which runs once the previous
 // batch's voxels are in (this kernel then reads no map state).
 constexpr int SEG_THREADS = 256;
 constexpr int SEG_SLOTS = 1024;
@@ -331,8 +331,9 @@ constexpr int SEG_MAX = 760;  // distinct keys per walk; every thread may claim 
 static_assert(SEG_MAX + SEG_THREADS <= SEG_SLOTS - 1, "a probe always finds an empty slot");
 static_assert(SEG_THREADS >= MAX_MASKS, "one thread per mask in the prefix sum");
 
+template <bool LOOKUP>
 __global__ void __launch_bounds__(SEG_THREADS) k_entries(const FrameParams* fps, BatchScratch bs,
-                                                         const MapRefs* refs, int f0, int lookup)
+                                                         const MapRefs* refs, int f0)
 {
     __shared__ __align__(16) unsigned long long tkey[SEG_SLOTS];
     __shared__ __align__(16) int thead[SEG_SLOTS];         // last record of the slot's chain
@@ -474,16 +475,16 @@ __global__ void __launch_bounds__(SEG_THREADS) k_entries(const FrameParams* fps,
             const unsigned long long hk = tkey[tlist[i]];
             const int at = s_off[(int)(hk >> 54) - 1] + trank[i];
             sc.sent[at] = hk;
-            if (lookup) {  // label in the map at the start of the batch (-1: absent then)
+            if constexpr (LOOKUP) {  // label in the map at the start of the batch (-1: absent then)
                 const VoxelTable& vt = refs[fp.map].vt;
                 const unsigned long long key = hk & ((1ull << 54) - 1);
-                unsigned long long h = mix64(key) & vt.mask;
+                unsigned long long h = vt_home(key, vt.mask);
                 int lab = -1, probes = 0;
                 while (true) {
                     const unsigned long long kk = vt.keys[h];
                     if (kk == key) { lab = vt.labels[h]; break; }
                     if (kk == EMPTY_KEY) break;
-                    h = (h + 1) & vt.mask;
+                    h = vt_next(h, probes + 1, vt.mask);
                     if (++probes > (int)vt.mask) { set_err(sc.ctr, DISC_ERR_TABLE_FULL); break; }
                 }
                 maxp = max(maxp, probes);
@@ -560,7 +561,9 @@ int launch_backproject(const FrameParams* fps, const BatchScratch& bs, int f0, i
 int launch_entries(const FrameParams* fps, const BatchScratch& bs, const MapRefs* refs, int f0, int nb, bool lookup,
                    cudaStream_t st)
 {
-    k_entries<<<dim3(bs.base.sparts, nb), SEG_THREADS, 0, st>>>(fps, bs, refs, f0, lookup ? 1 : 0);
+    const dim3 g(bs.base.sparts, nb);
+    if (lookup) k_entries<true><<<g, SEG_THREADS, 0, st>>>(fps, bs, refs, f0);
+    else k_entries<false><<<g, SEG_THREADS, 0, st>>>(fps, bs, refs, f0);
     return 1;
 }
 

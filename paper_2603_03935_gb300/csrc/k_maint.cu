@@ -15,12 +15,12 @@ __global__ void k_rehash(VoxelTable from, VoxelTable to, int* err)
          i += (unsigned long long)gridDim.x * blockDim.x) {
         const unsigned long long key = from.keys[i];
         if (key == EMPTY_KEY) continue;
-        unsigned long long h = mix64(key) & to.mask;
+        unsigned long long h = vt_home(key, to.mask);
         unsigned long long probes = 0;
         while (true) {
             unsigned long long prev = atomicCAS(&to.keys[h], EMPTY_KEY, key);
             if (prev == EMPTY_KEY) { to.labels[h] = from.labels[i]; break; }
-            h = (h + 1) & to.mask;
+            h = vt_next(h, probes + 1, to.mask);
             if (++probes > to.mask) { atomicExch(err, DISC_ERR_TABLE_FULL); return; }
         }
     }
@@ -92,7 +92,7 @@ __global__ void k_query_points(const float* xyz, long long n, float voxel, Voxel
         unsigned long long key;
         int out = -1;
         if (voxel_key(xyz[3 * i], xyz[3 * i + 1], xyz[3 * i + 2], __fdiv_rn(1.0f, voxel), &key)) {
-            unsigned long long h = mix64(key) & vt.mask;
+            unsigned long long h = vt_home(key, vt.mask);
             for (unsigned long long pr = 0; pr <= vt.mask; pr++) {
                 unsigned long long kk = vt.keys[h];
                 if (kk == key) {
@@ -101,7 +101,7 @@ __global__ void k_query_points(const float* xyz, long long n, float voxel, Voxel
                     break;
                 }
                 if (kk == EMPTY_KEY) break;
-                h = (h + 1) & vt.mask;
+                h = vt_next(h, pr + 1, vt.mask);
             }
         }
         ids[i] = out;
@@ -113,12 +113,12 @@ __global__ void k_load_voxels(const unsigned long long* keys, const int* labels,
 {
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
         const unsigned long long key = keys[i];
-        unsigned long long h = mix64(key) & vt.mask;
+        unsigned long long h = vt_home(key, vt.mask);
         unsigned long long probes = 0;
         while (true) {
             unsigned long long prev = atomicCAS(&vt.keys[h], EMPTY_KEY, key);
             if (prev == EMPTY_KEY || prev == key) { vt.labels[h] = labels[i]; break; }
-            h = (h + 1) & vt.mask;
+            h = vt_next(h, probes + 1, vt.mask);
             if (++probes > vt.mask) { atomicExch(err, DISC_ERR_TABLE_FULL); return; }
         }
     }

@@ -34,12 +34,12 @@ constexpr int OV_SLOTS = 2 * SER_THREADS;
 // label of a key in the voxel table, -1 if absent
 __device__ __forceinline__ int vt_label(const VoxelTable& vt, unsigned long long key)
 {
-    unsigned long long h = mix64(key) & vt.mask;
+    unsigned long long h = vt_home(key, vt.mask);
     for (unsigned long long pr = 0; pr <= vt.mask; pr++) {
         const unsigned long long kk = vt.keys[h];
         if (kk == key) return vt.labels[h];
         if (kk == EMPTY_KEY) return -1;
-        h = (h + 1) & vt.mask;
+        h = vt_next(h, pr + 1, vt.mask);
     }
     return -1;
 }
@@ -93,7 +93,7 @@ __device__ void dilated_pairs(const Scratch& sc, const SerialScratch& ss, const 
                     q[1] <= KEY_BIAS - 1 && q[2] >= -KEY_BIAS && q[2] <= KEY_BIAS - 1;
             nk[j] = ((unsigned long long)(q[0] + KEY_BIAS) << (2 * KEY_BITS)) |
                     ((unsigned long long)(q[1] + KEY_BIAS) << KEY_BITS) | (unsigned long long)(q[2] + KEY_BIAS);
-            h[j] = mix64(nk[j]) & vt.mask;
+            h[j] = vt_home(nk[j], vt.mask);
             cur[j] = in[j] ? vt.keys[h[j]] : EMPTY_KEY;
         }
 #pragma unroll
@@ -134,12 +134,12 @@ __device__ void phase_overlap(const Scratch& sc, const SerialScratch& ss, const 
             int lab = sc.elab[i];
             if (lab < 0) {
                 // absent when the batch started: an earlier frame may have added it
-                unsigned long long h = mix64(key) & vt.mask;
+                unsigned long long h = vt_home(key, vt.mask);
                 for (int pr = 0;; pr++) {
                     const unsigned long long kk = vt.keys[h];
                     if (kk == key) { lab = vt.labels[h]; break; }
                     if (kk == EMPTY_KEY || pr > (int)vt.mask) break;
-                    h = (h + 1) & vt.mask;
+                    h = vt_next(h, pr + 1, vt.mask);
                 }
             }
             if (dilate) dilated_pairs(sc, ss, vt, inst, m, key, lab);
@@ -937,11 +937,11 @@ __device__ void phase_apply(const FrameParams& fp, const Scratch& sc, const Scra
             const int t = ss.nlist[i];
             const unsigned long long key = ss.nkeys[t];
             const int lab = sc.segrep[ss.nown[t] - 1];
-            unsigned long long h = mix64(key) & vt.mask;
+            unsigned long long h = vt_home(key, vt.mask);
             for (int pr = 0;; pr++) {
                 const unsigned long long prev = atomicCAS(&vt.keys[h], EMPTY_KEY, key);
                 if (prev == EMPTY_KEY) { vt.labels[h] = lab; break; }
-                h = (h + 1) & vt.mask;
+                h = vt_next(h, pr + 1, vt.mask);
                 if (pr > (int)vt.mask) { set_err(sc.ctr, DISC_ERR_TABLE_FULL); break; }
             }
             // one count update per distinct instance of the warp
@@ -1105,15 +1105,9 @@ __global__ void k_serial_begin(const MapRefs* refs, int G)
 
 constexpr unsigned long long KEY54 = (1ull << 54) - 1;
 
-// The warp's lanes with `want` set add one voxel each to overlap item `key`
-// of the frame: lanes with the same key add together (one atomic per
-// distinct key of the warp).  All 32 lanes call.
-__device__ __forceinline__ void add_item_warp(const Scratch& sc, unsigned long long key, bool want)
+// `cnt` more voxels of overlap item `key` of the frame
+__device__ __forceinline__ void add_item(const Scratch& sc, unsigned long long key, int cnt)
 {
-    const unsigned act = __ballot_sync(0xffffffffu, want);
-    if (!want) return;
-    const unsigned grp = __match_any_sync(act, key);
-    if ((int)(threadIdx.x & 31) != __ffs(grp) - 1) return;
     unsigned long long t = mix64(key) & sc.smask;
     for (unsigned long long pr = 0;; pr++) {
         const unsigned long long cur = sc.pkey[t];
@@ -1132,7 +1126,19 @@ __device__ __forceinline__ void add_item_warp(const Scratch& sc, unsigned long l
             return;
         }
     }
-    atomicAdd(&sc.pcnt[t], __popc(grp));
+    atomicAdd(&sc.pcnt[t], cnt);
+}
+
+// The warp's lanes with `want` set add one voxel each to overlap item `key`
+// of the frame: lanes with the same key add together (one atomic per
+// distinct key of the warp).  All 32 lanes call.
+__device__ __forceinline__ void add_item_warp(const Scratch& sc, unsigned long long key, bool want)
+{
+    const unsigned act = __ballot_sync(0xffffffffu, want);
+    if (!want) return;
+    const unsigned grp = __match_any_sync(act, key);
+    if ((int)(threadIdx.x & 31) != __ffs(grp) - 1) return;
+    add_item(sc, key, __popc(grp));
 }
 
 // Warp-aggregated append: each lane with `want` gets a distinct index from
@@ -1162,9 +1168,9 @@ __device__ __forceinline__ int probe_label(const VoxelTable& vt, unsigned long l
     if (!active) return -1;
     const int lane = threadIdx.x & 31, base = lane & ~(PW - 1), sub = lane - base;
     const unsigned gmask = (PW == 32 ? 0xffffffffu : ((1u << PW) - 1u)) << base;
-    const unsigned long long h = mix64(key) & vt.mask;
+    const unsigned long long h = vt_home(key, vt.mask);
     for (unsigned long long pr = 0; pr <= vt.mask; pr += PW) {
-        const unsigned long long slot = (h + pr + sub) & vt.mask;
+        const unsigned long long slot = vt_slot(h, pr + sub, vt.mask);
         const unsigned long long kk = vt.keys[slot];
         const unsigned hit = (__ballot_sync(gmask, kk == key || kk == EMPTY_KEY) & gmask) >> base;
         if (hit) {
@@ -1180,11 +1186,133 @@ __device__ __forceinline__ int probe_label(const VoxelTable& vt, unsigned long l
     return -1;
 }
 
+// Absent voxel `key` of segment m of frame fp, into the batch's absent-voxel
+// hash: its slot (-1 on failure); *claimed: the first to name the voxel.
+__device__ __forceinline__ int add_absent(const FrameParams& fp, const Scratch& sc, const AbsentHash& ah, int m,
+                                          unsigned long long key, bool* claimed)
+{
+    const unsigned long long ak = ((unsigned long long)(fp.map + 1) << 54) | key;
+    unsigned long long t = mix64(ak) & ah.mask;
+    for (unsigned long long pr = 0;; pr++) {
+        const unsigned long long cur = ah.key[t];
+        if (cur == ak) break;
+        if (cur == 0ull) {
+            const unsigned long long prev = atomicCAS(&ah.key[t], 0ull, ak);
+            if (prev == 0ull) { *claimed = true; break; }
+            if (prev == ak) break;
+        }
+        t = (t + 1) & ah.mask;
+        if (pr > ah.mask) { set_err(sc.ctr, DISC_ERR_TABLE_FULL); return -1; }
+    }
+    atomicMin(&ah.val[t], (fp.jpos << 9) | m);
+    return (int)t;
+}
+
+// Every entry of every frame slot of the batch (block row = slot), one lane
+// per entry: as k_lookup below.  A thread takes four entries, whose keys,
+// table slots and labels are each loaded together: the kernel waits for
+// random table sectors, and one entry per thread kept too few of them in
+// flight.  A block's 1024 entries (sorted by mask within their partitions)
+// meet in a shared hash of items, so that only its distinct ones reach the
+// frame's.
+// Bound by the latency of random table sectors.  Room frames, 32 per launch,
+// with k_absent and k_items: 4.8 us per frame with one entry per thread and a
+// warp match, 4.0 so, 3.2 with a block's voxels in one place of the table
+// (vt_home).
+constexpr int LK_PER = 4, LK_THREADS = 256, LK_TILE = LK_PER * LK_THREADS, LK_SLOTS = 2 * LK_TILE;
+
+__global__ void __launch_bounds__(LK_THREADS) k_lookup1(const FrameParams* fps, BatchScratch bs, const MapRefs* refs,
+                                                        AbsentHash ah)
+{
+    __shared__ __align__(16) unsigned long long tkey[LK_SLOTS];
+    __shared__ __align__(16) int tcnt[LK_SLOTS];
+    __shared__ unsigned short tlist[LK_TILE];
+    __shared__ int s_n, s_err;
+    const int f = blockIdx.y;
+    const FrameParams& fp = fps[f];
+    const Scratch sc = bs.frame(f);
+    const int ne = sc.ctr->n_entries, tid = threadIdx.x;
+    if (tid == 0) s_err = *(volatile int32_t*)&sc.ctr->err;  // blocks of this launch may set it
+    __syncthreads();
+    if (fp.M <= 0 || s_err) return;  // a failed frame's items are never read
+    const VoxelTable vt = refs[fp.map].vt;
+    int maxp = 0;
+    for (int i0 = blockIdx.x * LK_TILE; i0 < ne; i0 += gridDim.x * LK_TILE) {  // uniform per block
+        unsigned long long hk[LK_PER], h[LK_PER], cur[LK_PER];
+        int lab[LK_PER];
+#pragma unroll
+        for (int j = 0; j < LK_PER; j++) {
+            const int i = i0 + j * LK_THREADS + tid;
+            hk[j] = i < ne ? sc.sent[i] : 0ull;
+        }
+        for (int i = tid; i < LK_SLOTS / 2; i += LK_THREADS) ((uint4*)tkey)[i] = make_uint4(~0u, ~0u, ~0u, ~0u);
+        for (int i = tid; i < LK_SLOTS / 4; i += LK_THREADS) ((int4*)tcnt)[i] = make_int4(0, 0, 0, 0);
+        if (tid == 0) s_n = 0;
+#pragma unroll
+        for (int j = 0; j < LK_PER; j++) {
+            h[j] = vt_home(hk[j] & KEY54, vt.mask);
+            cur[j] = hk[j] ? vt.keys[h[j]] : EMPTY_KEY;
+        }
+        // the first slot decides most entries; the others walk on
+#pragma unroll
+        for (int j = 0; j < LK_PER; j++) {
+            int pr = 0;
+            while (cur[j] != EMPTY_KEY && cur[j] != (hk[j] & KEY54)) {
+                if ((unsigned long long)++pr > vt.mask) {
+                    set_err(sc.ctr, DISC_ERR_TABLE_FULL);
+                    hk[j] = 0ull;
+                    break;
+                }
+                h[j] = vt_next(h[j], pr, vt.mask);
+                cur[j] = vt.keys[h[j]];
+            }
+            maxp = max(maxp, pr);
+        }
+#pragma unroll
+        for (int j = 0; j < LK_PER; j++) lab[j] = hk[j] && cur[j] != EMPTY_KEY ? vt.labels[h[j]] : -1;
+        __syncthreads();
+#pragma unroll
+        for (int j = 0; j < LK_PER; j++) {
+            if (lab[j] >= 0) {
+                const unsigned long long key = ((hk[j] >> 54) << 33) | (unsigned)lab[j];
+                unsigned t = (unsigned)mix64(key) & (LK_SLOTS - 1);
+                while (true) {  // at most LK_TILE distinct keys in LK_SLOTS slots
+                    const unsigned long long prev = atomicCAS(&tkey[t], EMPTY_KEY, key);
+                    if (prev == EMPTY_KEY) {
+                        tlist[atomicAdd(&s_n, 1)] = (unsigned short)t;
+                        break;
+                    }
+                    if (prev == key) break;
+                    t = (t + 1) & (LK_SLOTS - 1);
+                }
+                atomicAdd(&tcnt[t], 1);
+            }
+            const bool absent = hk[j] && lab[j] < 0;
+            if (!__any_sync(0xffffffffu, absent)) continue;
+            bool claimed = false;
+            int at = -1;
+            if (absent) at = add_absent(fp, sc, ah, (int)(hk[j] >> 54), hk[j] & KEY54, &claimed);
+            const int li = warp_append(ah.n, claimed);
+            if (claimed) ah.list[li] = at;
+            const int ai = warp_append(&sc.ctr->n_absent, at >= 0);
+            if (at >= 0) {
+                sc.aent[ai] = i0 + j * LK_THREADS + tid;
+                sc.aslot[ai] = at;
+            }
+        }
+        __syncthreads();
+        for (int i = tid; i < s_n; i += LK_THREADS) add_item(sc, tkey[tlist[i]], tcnt[tlist[i]]);
+        __syncthreads();
+    }
+    const int pm = __reduce_max_sync(0xffffffffu, maxp);
+    if ((tid & 31) == 0 && pm > 0) atomicMax(&sc.ctr->max_probe, pm);
+}
+
 // Every entry of every frame slot of the batch (block row = slot): its label
 // in the map at the batch start (tag-0 item), or, when absent, its slot in
 // the batch's absent-voxel hash, where the least (frame position, segment)
-// containing it is kept.  PW lanes look each entry up together (PW = 1: one
-// lane per entry); the group's first lane carries the entry afterwards.
+// containing it is kept.  PW lanes (2, 4 or 8) look each entry up together;
+// the group's first lane carries the entry afterwards.
 template <int PW>
 __global__ void __launch_bounds__(256) k_lookup(const FrameParams* fps, BatchScratch bs, const MapRefs* refs,
                                                AbsentHash ah)
@@ -1195,7 +1323,6 @@ __global__ void __launch_bounds__(256) k_lookup(const FrameParams* fps, BatchScr
     const int ne = sc.ctr->n_entries;
     if (fp.M <= 0 || sc.ctr->err) return;  // a failed frame's items are never read
     const VoxelTable vt = refs[fp.map].vt;
-    const unsigned long long gtag = (unsigned long long)(fp.map + 1) << 54;
     const int lane = threadIdx.x & 31;
     constexpr int PER = 32 / PW;  // entries of a warp per round
     const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nwarps = (gridDim.x * blockDim.x) >> 5;
@@ -1215,23 +1342,7 @@ __global__ void __launch_bounds__(256) k_lookup(const FrameParams* fps, BatchScr
         int at = -1;
         bool claimed = false;
         if (lead && !full && lab < 0) {
-            const unsigned long long ak = gtag | key;
-            unsigned long long t = mix64(ak) & ah.mask;
-            for (unsigned long long pr = 0;; pr++) {
-                const unsigned long long cur = ah.key[t];
-                if (cur == ak) break;
-                if (cur == 0ull) {
-                    const unsigned long long prev = atomicCAS(&ah.key[t], 0ull, ak);
-                    if (prev == 0ull) { claimed = true; break; }
-                    if (prev == ak) break;
-                }
-                t = (t + 1) & ah.mask;
-                if (pr > ah.mask) { set_err(sc.ctr, DISC_ERR_TABLE_FULL); t = ~0ull; break; }
-            }
-            if (t != ~0ull) {
-                atomicMin(&ah.val[t], (fp.jpos << 9) | m);
-                at = (int)t;
-            }
+            at = add_absent(fp, sc, ah, m, key, &claimed);
         }
         add_item_warp(sc, ((unsigned long long)m << 33) | (unsigned)lab, lead && lab >= 0);
         const int li = warp_append(ah.n, claimed);
@@ -1683,14 +1794,14 @@ __global__ void k_commit(BatchScratch bs, SerialStep st, AbsentHash ah, int G)
         const bool ins = lab >= 0;
         if (ins) {
             const VoxelTable vt = st.refs[g].vt;
-            unsigned long long h = mix64(key) & vt.mask;
+            unsigned long long h = vt_home(key, vt.mask);
             for (unsigned long long pr = 0;; pr++) {
                 const unsigned long long prev = atomicCAS(&vt.keys[h], EMPTY_KEY, key);
                 if (prev == EMPTY_KEY) {
                     vt.labels[h] = lab;
                     break;
                 }
-                h = (h + 1) & vt.mask;
+                h = vt_next(h, pr + 1, vt.mask);
                 if (pr > vt.mask) break;  // not reached: the batch's room was checked before it ran
             }
         }
@@ -1792,7 +1903,7 @@ int launch_lookup(const FrameParams* fps, const BatchScratch& bs, const MapRefs*
         case 2: k_lookup<2><<<grid, 256, 0, st>>>(fps, bs, refs, ah); break;
         case 4: k_lookup<4><<<grid, 256, 0, st>>>(fps, bs, refs, ah); break;
         case 8: k_lookup<8><<<grid, 256, 0, st>>>(fps, bs, refs, ah); break;
-        default: k_lookup<1><<<grid, 256, 0, st>>>(fps, bs, refs, ah); break;
+        default: k_lookup1<<<grid, LK_THREADS, 0, st>>>(fps, bs, refs, ah); break;
     }
     k_absent<<<dim3(38, S), 256, 0, st>>>(fps, bs, ah);
     k_items<<<dim3(16, S), 256, 0, st>>>(bs);

@@ -90,3 +90,38 @@ def test_records_at_the_partition_edges(case):
     if case in ("one_voxel", "few_voxels"):
         assert st["unique_seg_voxels"] < 0.2 * st["valid_pixels"]
     gmap.close()
+
+
+@pytest.mark.parametrize("probe_width", [1, 2, 8])
+def test_skewed_voxel_tables_use_every_slot(probe_width):
+    """Voxels two apart share one place of their blocks' eight slots: a table at 3/4 load has to place most of them
+    in the other places, and every lookup has to find them there."""
+    import torch
+    from paper_2603_03935_gb300 import DiscMap, device_frame
+    dev = torch.device("cuda:0")
+    rng = np.random.default_rng(5)
+    cfg = dict(voxel_size=0.02, embed_dim=DIM, patch_h=GRID[0], patch_w=GRID[1], max_width=W, max_height=H, max_masks=8,
+               min_mask_pixels=1, voxel_capacity=1 << 12, max_load=0.9, instance_capacity=64, z_min=0.1, z_max=10.0,
+               eps=1e-6, tau_cos=0.75, lambda_size=3.3, ov_num=1, ov_den=5)
+    gmap, omap = DiscMap(**cfg), oracle.OracleMap(**common.to_oracle_cfg(cfg))
+    gmap.set_schedule(probe_width=probe_width)
+    depth = np.full((H, W), 2.0, np.float32)
+    labels = ((np.arange(H)[:, None] // 12 + np.arange(W)[None, :] // 16) % 8 + 1).astype(np.uint16)
+    tokens = rng.normal(size=(GRID[0] * GRID[1], DIM)).astype(np.float32)
+    intr = (50.0, 50.0, W / 2 - 0.25, H / 2 - 0.25)  # 0.04 m from pixel to pixel, each in the middle of its voxel
+    for i in range(3):
+        pose = np.eye(4)
+        pose[2, 3] = 0.01
+        pose[0, 3] = (0.0, 0.64, 0.0)[i]  # the second frame covers half of the first and new voxels
+        st = gmap.integrate(device_frame(torch.from_numpy(depth).to(dev), torch.from_numpy(labels.view(np.int16)).to(dev),
+                                         torch.from_numpy(tokens).to(dev), pose, intr, 8))
+        o = omap.integrate(depth, labels, tokens, pose, intr, 8)
+        common.compare_frame(st, gmap.last_frame(), o, ctx=f"frame {i}")
+        if i == 0:
+            assert st["unique_seg_voxels"] == W * H and gmap.cfg["voxel_capacity"] == 1 << 12
+    common.compare_maps(gmap, omap, ctx="skewed")
+    keys, ids = gmap.voxels()
+    k = [((keys >> np.uint64(s)).astype(np.int64) & 0x3ffff) - (1 << 17) for s in (36, 18, 0)]
+    xyz = (np.stack(k, 1) + 0.5) * 0.02
+    assert np.array_equal(gmap.query_points(xyz.astype(np.float32)), ids)
+    gmap.close()
