@@ -186,7 +186,7 @@ struct Runner {
     int geo_chunk = GEOMETRY_CHUNK;   // frames per back-projection / entries / DBSCAN launch
     int cta_scale = 4;                // serial kernels' CTAs in quarters of the default count
     int probe_width = 1;              // lanes per key of the batch's voxel-table lookup
-    int assoc_cluster = 0;            // CTAs per map of the association kernel (0: automatic)
+    int assoc_cluster = 0;            // accepted, without effect (one CTA per map associates)
     int batch_split = 0;              // smaller batches per call that fits one (0: automatic)
     bool graphs_off = false;
     std::map<long long, BatchGraph> graphs;
@@ -1087,11 +1087,9 @@ int enqueue_serial(Runner& r, int k, int S, int G, int J, int combos, cudaStream
     step.merged = r.d_merged;
     if (!(combos & COMBO_DILATE)) {
         step.j = 0;
-        run_phase(r, PH_LOOKUP, st, [&] { return launch_lookup(dfp, bs, step.refs, r.ah, S, r.probe_width, st); });
-        // on an SM partition (serial_sms) the chain runs one CTA per map: a
-        // cluster's CTAs must fit the partition's SMs together
-        const int cluster = r.green[0] ? 1 : r.assoc_cluster;
-        run_phase(r, PH_ASSOCIATE, st, [&] { return launch_associate(dfp, bs, step, G, cluster, st); });
+        run_phase(r, PH_LOOKUP, st,
+                  [&] { return launch_lookup(dfp, bs, step.view, step.refs, r.ah, S, r.probe_width, st); });
+        run_phase(r, PH_ASSOCIATE, st, [&] { return launch_associate(dfp, bs, step, G, st); });
         run_phase(r, PH_COMMIT, st, [&] {
             const int n = launch_commit(bs, step, r.ah, G, st);
             cudaMemsetAsync(r.ah.n, 0, sizeof(int32_t), st);  // the hash is empty again

@@ -551,53 +551,11 @@ __device__ __forceinline__ unsigned dsm_map(const void* local, unsigned rank)
     asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(out) : "r"(a), "r"(rank));
     return out;
 }
-__device__ __forceinline__ unsigned long long dsm_cas64(unsigned a, unsigned long long cmp, unsigned long long v)
-{
-    unsigned long long old;
-    asm volatile("atom.shared::cluster.cas.b64 %0, [%1], %2, %3;" : "=l"(old) : "r"(a), "l"(cmp), "l"(v) : "memory");
-    return old;
-}
-__device__ __forceinline__ int dsm_add(unsigned a, int v)
-{
-    int old;
-    asm volatile("atom.shared::cluster.add.u32 %0, [%1], %2;" : "=r"(old) : "r"(a), "r"(v) : "memory");
-    return old;
-}
-__device__ __forceinline__ void dsm_red_add(unsigned a, int v)
-{
-    asm volatile("red.shared::cluster.add.u32 [%0], %1;" ::"r"(a), "r"(v) : "memory");
-}
-__device__ __forceinline__ unsigned long long dsm_ld64(unsigned a)
-{
-    unsigned long long v;
-    asm volatile("ld.shared::cluster.u64 %0, [%1];" : "=l"(v) : "r"(a) : "memory");
-    return v;
-}
 __device__ __forceinline__ int dsm_ld32(unsigned a)
 {
     int v;
     asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(a) : "memory");
     return v;
-}
-__device__ __forceinline__ void dsm_st32(unsigned a, int v)
-{
-    asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(a), "r"(v) : "memory");
-}
-__device__ __forceinline__ void dsm_st64(unsigned a, unsigned long long v)
-{
-    asm volatile("st.shared::cluster.u64 [%0], %1;" ::"r"(a), "l"(v) : "memory");
-}
-__device__ __forceinline__ unsigned cluster_rank()
-{
-    unsigned r;
-    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-    return r;
-}
-__device__ __forceinline__ unsigned cluster_size()
-{
-    unsigned n;
-    asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(n));
-    return n;
 }
 // every thread of every CTA of the cluster; shared-memory and global writes
 // before it are visible to the cluster after it (release / acquire)
@@ -605,9 +563,4 @@ __device__ __forceinline__ void cluster_sync()
 {
     asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
 }
-// the two halves of cluster_sync: between them a thread may read what no
-// other thread of the cluster writes in this phase
-__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
-__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
-
 }  // namespace disc

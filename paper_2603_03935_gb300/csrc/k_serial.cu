@@ -480,7 +480,6 @@ constexpr unsigned UH_EMPTY = 0xffffffffu;
 constexpr unsigned UH_UNUSED = 0xffffffffu;
 constexpr unsigned UH_LOCAL = 0x80000000u;
 constexpr size_t UNION_SMEM = (size_t)UHASH * 8 + (size_t)EDGE_ROOT_CAP * 24 + (size_t)EDGE_CAP * 8;
-static_assert(UNION_SMEM == (size_t)UHASH * 8 + (size_t)EDGE_ROOT_CAP * 24 + (size_t)EDGE_CAP * 8, "union layout");
 
 // slot of root id k in the union's root hash (32-bit multiplicative mix)
 __device__ __forceinline__ unsigned uhash(unsigned k, unsigned mask)
@@ -517,85 +516,43 @@ __device__ __forceinline__ int local_of(const unsigned* hkey, const unsigned* hv
     return (int)(hval[h] & ~UH_LOCAL);
 }
 
-// Bytes of a union region with the given capacities (layout in
-// UnionRegion); pre: with the arrays of values gathered before the union.
-__host__ __device__ constexpr size_t union_region_bytes(unsigned uhash_cap, int root_cap, int edge_cap,
-                                                        bool pre = false)
-{
-    return (size_t)uhash_cap * 8 + (size_t)root_cap * (pre ? 32 : 24) + (size_t)edge_cap * (pre ? 24 : 8);
-}
-
-// The arrays of a union region: the root hash, the per-local-root arrays
-// and the edge arrays; with `pre` also each local root's voxel count (cloc)
-// and, per edge, its instance's count, Q and observations as the gates read
-// them (ec, eq, eo), so the union issues no global load for them.
+// The arrays of a union region (UNION_SMEM bytes): the root hash, the
+// per-local-root arrays and the edge arrays.
 struct UnionRegion {
-    unsigned* hkey;      // [uhash_cap] root id
-    unsigned* hval;      // [uhash_cap] claimant edge, then UH_LOCAL | local index
-    long long* cloc;     // [root_cap] voxel count of the local roots (pre)
-    int* gid;            // [root_cap] local -> instance id
+    unsigned* hkey;      // [UHASH] root id
+    unsigned* hval;      // [UHASH] claimant edge, then UH_LOCAL | local index
+    int* gid;            // [EDGE_ROOT_CAP] local -> instance id
     int* uf;             // union-find over local indices
     int* best_src;       // fusion winner per component
     float* best_q;
     float* qloc;         // Q of the local roots
     int* oloc;           // observations of the local roots
-    long long* ec;       // [edge_cap] count of the edge's instance (pre)
-    int* em;             // [edge_cap] edge segment
-    int* ek;             // [edge_cap] edge instance id
-    float* eq;           // [edge_cap] Q of the edge's instance (pre)
-    int* eo;             // [edge_cap] observations of the edge's instance (pre)
-    __device__ __forceinline__ UnionRegion(unsigned char* base, unsigned uhash_cap, int root_cap, int edge_cap,
-                                           bool pre)
+    int* em;             // [EDGE_CAP] edge segment
+    int* ek;             // [EDGE_CAP] edge instance id
+    __device__ __forceinline__ explicit UnionRegion(unsigned char* base)
     {
         hkey = (unsigned*)base;
-        hval = hkey + uhash_cap;
-        cloc = pre ? (long long*)(hval + uhash_cap) : nullptr;
-        gid = pre ? (int*)(cloc + root_cap) : (int*)(hval + uhash_cap);
-        uf = gid + root_cap;
-        best_src = uf + root_cap;
-        best_q = (float*)(best_src + root_cap);
-        qloc = best_q + root_cap;
-        oloc = (int*)(qloc + root_cap);
-        ec = pre ? (long long*)(oloc + root_cap) : nullptr;
-        em = pre ? (int*)(ec + edge_cap) : oloc + root_cap;
-        ek = em + edge_cap;
-        eq = pre ? (float*)(ek + edge_cap) : nullptr;
-        eo = pre ? (int*)(eq + edge_cap) : nullptr;
+        hval = hkey + UHASH;
+        gid = (int*)(hval + UHASH);
+        uf = gid + EDGE_ROOT_CAP;
+        best_src = uf + EDGE_ROOT_CAP;
+        best_q = (float*)(best_src + EDGE_ROOT_CAP);
+        qloc = best_q + EDGE_ROOT_CAP;
+        oloc = (int*)(qloc + EDGE_ROOT_CAP);
+        em = oloc + EDGE_ROOT_CAP;
+        ek = em + EDGE_CAP;
     }
 };
 
-// Per-segment inputs of the union read by the calling thread before the
-// union starts (thread t for segment t; the frame's M <= block size), and
-// what the union hands back to every thread when it completes.
-struct UnionPre {
-    int nv;       // nvox[t]
-    float q;      // the segment's Q
-    int nnew;     // voxels the frame inserts with segment t as their lowest segment
-    int next;     // the map's next instance id
-    int ok;       // out: the union completed without error
-    int ncopy;    // out: embedding copies it listed
-    int merges;   // out: instances it merged
-};
-
 // The frame's npairs overlap pairs give their roots through pair_root(i);
-// its nedge accepted edges are in ss.edge_m/k, or (edges_in_place) already in
-// the region's em/ek arrays (and, with pre, their instances' values in
-// ec/eq/eo).  The region (shared memory, or global memory for frames beyond
-// the shared capacities) is laid out as UnionRegion: hkey, hval [uhash_cap
-// >= 2 * npairs], the per-root arrays [root_cap], the edge arrays [edge_cap
-// >= 2 * root_cap: the fusion step lays root_cap 64-bit words over em].
-// pre: the calling thread's per-segment values, read before the union; the
-// union then also adds the frame's new voxels to their instances' counts.
-// Past a capacity the frame fails with DISC_ERR_CAPACITY, or, soft, the
-// call returns false before anything outside the region changed (the caller
-// then retries with larger capacities); otherwise it returns true.
+// its nedge accepted edges are in ss.edge_m/k.  union_smem: a union region in
+// shared or global memory (the fusion step lays EDGE_ROOT_CAP 64-bit words
+// over em).  Past a capacity the frame fails with DISC_ERR_CAPACITY.
 template <class PairRoot>
-__device__ bool union_frame(const FrameParams& fp, const Scratch& sc, const SerialScratch& ss, const Instances& inst,
-                            int* next_id, unsigned char* union_smem, unsigned uhash_cap, int root_cap, int edge_cap,
-                            bool soft, int npairs, int nedge, bool edges_in_place, PairRoot pair_root,
-                            UnionPre* pre = nullptr)
+__device__ void union_frame(const FrameParams& fp, const Scratch& sc, const SerialScratch& ss, const Instances& inst,
+                            int* next_id, unsigned char* union_smem, int npairs, int nedge, PairRoot pair_root)
 {
-    const UnionRegion U(union_smem, uhash_cap, root_cap, edge_cap, pre != nullptr);
+    const UnionRegion U(union_smem);
     unsigned* hkey = U.hkey;
     unsigned* hval = U.hval;
     int* gid = U.gid;
@@ -614,16 +571,15 @@ __device__ bool union_frame(const FrameParams& fp, const Scratch& sc, const Seri
     const int tid = threadIdx.x, NT = blockDim.x;
     FrameCounters* ctr = sc.ctr;
     const int M = fp.M;
-    if (2u * (unsigned)npairs > uhash_cap || nedge > edge_cap) {
-        if (soft) return false;
+    if (2u * (unsigned)npairs > (unsigned)UHASH || nedge > EDGE_CAP) {
         if (tid == 0) set_err(ctr, DISC_ERR_CAPACITY);
-        return true;
+        return;
     }
     unsigned hsize = 64;
     while (hsize < 2u * (unsigned)npairs) hsize <<= 1;
     const unsigned hm = hsize - 1;
     // the edges, once, into shared memory (segment, root)
-    for (int e = tid; e < nedge && !edges_in_place; e += NT) {
+    for (int e = tid; e < nedge; e += NT) {
         em[e] = ss.edge_m[e];
         ek[e] = ss.edge_k[e];
     }
@@ -631,18 +587,10 @@ __device__ bool union_frame(const FrameParams& fp, const Scratch& sc, const Seri
         hkey[i] = UH_EMPTY;
         hval[i] = UH_UNUSED;
     }
-    if (pre) {
-        if (tid < M) {
-            anchor[tid] = INT_MAX;
-            snv[tid] = pre->nv;
-            sq[tid] = pre->q;
-        }
-    } else {
-        for (int m = tid; m < M; m += NT) {
-            anchor[m] = INT_MAX;
-            snv[m] = sc.nvox[m];
-            sq[m] = sc.S[5 * m + 4];
-        }
+    for (int m = tid; m < M; m += NT) {
+        anchor[m] = INT_MAX;
+        snv[m] = sc.nvox[m];
+        sq[m] = sc.S[5 * m + 4];
     }
     if (tid == 0) {
         s_nroots = 0;
@@ -650,7 +598,7 @@ __device__ bool union_frame(const FrameParams& fp, const Scratch& sc, const Seri
         s_merges = 0;
         s_new = 0;
         s_ncopy = 0;
-        s_next = pre ? pre->next : *next_id;
+        s_next = *next_id;
     }
     __syncthreads();
     // (1) active set: distinct roots of all overlap pairs (counted per warp)
@@ -689,27 +637,20 @@ __device__ bool union_frame(const FrameParams& fp, const Scratch& sc, const Seri
         while (hkey[h] != k) h = (h + 1) & hm;
         if (hval[h] == (unsigned)e) {
             const int x = atomicAdd(&s_nloc, 1);
-            if (x < root_cap) {
+            if (x < EDGE_ROOT_CAP) {
                 gid[x] = (int)k;
                 uf[x] = x;
-                if (pre) {
-                    qloc[x] = U.eq[e];
-                    oloc[x] = U.eo[e];
-                    U.cloc[x] = U.ec[e];
-                } else {
-                    qloc[x] = inst.Q[k];
-                    oloc[x] = inst.n_obs[k];
-                }
+                qloc[x] = inst.Q[k];
+                oloc[x] = inst.n_obs[k];
             }
             hval[h] = UH_LOCAL | (unsigned)x;
         }
     }
     __syncthreads();
     const int nloc = s_nloc;
-    if (nloc > root_cap) {
-        if (soft) return false;
+    if (nloc > EDGE_ROOT_CAP) {
         if (tid == 0) set_err(ctr, DISC_ERR_CAPACITY);
-        return true;
+        return;
     }
     // (3) union of the instances one segment joins: every edge hooks its
     //     root onto the segment's anchor; a hook always links the root with
@@ -751,7 +692,7 @@ __device__ bool union_frame(const FrameParams& fp, const Scratch& sc, const Seri
         const int base = s_next;
         if (base + total > inst.cap) {  // uniform: every thread summed the same counts
             if (tid == 0) set_err(ctr, DISC_ERR_CAPACITY);
-            return true;
+            return;
         }
         if (want) {
             const int id = base + before, m = tid;
@@ -829,19 +770,16 @@ __device__ bool union_frame(const FrameParams& fp, const Scratch& sc, const Seri
         ss.copy_src[c] = src;
         inst.Q[rep] = q;
     }
-    // (6) merge members into their representative (then, with pre, the
-    //     frame's new voxels into their segment's instance)
+    // (6) merge members into their representative
     for (int x = tid; x < nloc; x += NT) {
         const int r = uf[x];
         if (r == x) continue;
         const int k = gid[x], rep = gid[r];
         inst.parent[k] = rep;
-        atomicAdd((unsigned long long*)&inst.count[rep], (unsigned long long)(pre ? U.cloc[x] : inst.count[k]));
+        atomicAdd((unsigned long long*)&inst.count[rep], (unsigned long long)inst.count[k]);
         inst.count[k] = 0;
         atomicAdd(&s_merges, 1);
     }
-    if (pre && tid < M && pre->nnew && srep[tid] >= 0)
-        atomicAdd((unsigned long long*)&inst.count[srep[tid]], (unsigned long long)pre->nnew);
     __syncthreads();
     if (tid == 0) {
         *ss.copy_n = s_ncopy;
@@ -852,12 +790,6 @@ __device__ bool union_frame(const FrameParams& fp, const Scratch& sc, const Seri
         ctr->next_id = s_next;
         ctr->n_copies = s_ncopy;
     }
-    if (pre) {
-        pre->ok = 1;
-        pre->ncopy = s_ncopy;
-        pre->merges = s_merges;
-    }
-    return true;
 }
 
 // The frame's pairs in the map's global pair hash, its edges in ss.edge_m/k;
@@ -867,7 +799,7 @@ __device__ void phase_union(const FrameParams& fp, const Scratch& sc, const Seri
 {
     const int npairs = sc.ctr->n_pairs;
     const int nedge = min(*ss.edge_n, ss.edge_cap);
-    union_frame(fp, sc, ss, inst, next_id, union_smem, UHASH, EDGE_ROOT_CAP, EDGE_CAP, false, npairs, nedge, false,
+    union_frame(fp, sc, ss, inst, next_id, union_smem, npairs, nedge,
                 [&](int i) { return (unsigned)(ss.okeys[ss.olist[i]] & 0xffffffffu); });
 }
 
@@ -1398,18 +1330,21 @@ __global__ void __launch_bounds__(256) k_absent(const FrameParams* fps, BatchScr
 // Every slot's overlap items, once k_absent is done: the hash slots listed
 // in plist become dense (key, count) arrays in claim order (ikey over the
 // free aent | aslot, icnt over plist itself: each thread reads plist[i]
-// before it writes icnt[i]), and the hash is emptied for the slot's next
-// batch.  Items of a failed frame are emptied as well.
-__global__ void __launch_bounds__(256) k_items(BatchScratch bs)
+// before it writes icnt[i]), tag-0 items under their label's root as the
+// batch starts, and the hash is emptied for the slot's next batch.  Items of
+// a failed frame are emptied as well.
+__global__ void __launch_bounds__(256) k_items(const FrameParams* fps, BatchScratch bs, const MapRefs* refs)
 {
     const Scratch sc = bs.frame(blockIdx.y);
     const int n = sc.ctr->n_pre;
+    const int32_t* parent = refs[fps[blockIdx.y].map].inst.parent;  // flat between batches
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
         const int t = sc.plist[i];
-        const unsigned long long key = sc.pkey[t];
+        unsigned long long key = sc.pkey[t];
         const int cnt = sc.pcnt[t];
         sc.pkey[t] = EMPTY_KEY;
         sc.pcnt[t] = 0;
+        if (!((key >> 32) & 1ull)) key = (key & ~0xffffffffull) | (unsigned)parent[(unsigned)key];
         sc.ikey[i] = key;
         sc.icnt[i] = cnt;
     }
@@ -1444,297 +1379,492 @@ __device__ __forceinline__ int block_read(const int32_t* w)
 }
 
 constexpr int ASSOC_THREADS = 512;
-constexpr int APH = 2048;         // slots of the leader CTA's pair hash (shared memory)
+constexpr int APH = 2048;         // slots of the pair hash (shared memory)
 constexpr int APH_MAX = 1536;     // pairs it takes (load <= 3/4)
+constexpr int APH_PROBES = 64;    // longest probe of the pair hash
+constexpr int ARH = 2048;         // slots of the hash of active roots
 constexpr int ASSOC_ROOTS = 256;  // instances with an accepted edge, in shared memory
 constexpr int ASSOC_EDGES = 512;  // accepted edges, in shared memory
-// A frame past one of these shared capacities runs steps (1)-(3) on the
-// leader alone with the map's global pair hash and union region.  The small
-// footprint lets the CTAs share SMs with the next batch's stateless kernels.
-constexpr size_t ASSOC_SMEM = (size_t)APH * 16 + union_region_bytes(2 * APH, ASSOC_ROOTS, ASSOC_EDGES, true);
-constexpr int ASSOC_CLUSTER_MAX = 8;
-static_assert(ASSOC_EDGES >= 2 * ASSOC_ROOTS, "the fusion step overlays the edge arrays");
+constexpr int ASSOC_CHG = 512;    // words of the bitmap of instances whose embedding changed in the batch
+// A frame past one of these shared capacities runs steps (1)-(3) with the
+// map's global pair hash and union region.
+constexpr int ASSOC_FRAMES = 64;  // frames whose slot, items and masks are read once, at the start
 
-// A cluster of C CTAs per map of the batch (C = cluster size, 1 to 8)
-// walks the map's frames in order.  The leader CTA (rank 0) holds the
-// frame's pair hash, scored-pair list, edge list and union state in its
-// shared memory; the other CTAs reach them through distributed shared
-// memory.  Per frame:
-//   (1) every CTA resolves a share of the frame's items to (segment, root)
-//       pairs and counts them in the leader's pair hash;
-//   (2) every thread of the cluster checks the overlap gate of one pair and
-//       appends a passing pair to the scored list; then every warp takes the
-//       cosine gate of one scored pair (so no warp scores several while
-//       others idle); accepted edges go to the leader's edge list;
-//   (3) the leader alone: union, new ids, merges and fusion winners; then it
-//       stages the frame's status and copy count and empties its pair hash;
-//   (4) every warp a share of the embedding copies; the leader the voxel
-//       counts of the frame's new voxels;
-// with a cluster barrier after (1), after each half of (2) and after (3).
-// Step (4) needs no barrier before the next frame's step (1): that step
-// touches only the leader's emptied hash, and the next barrier orders the
-// copies before the next gates read the embeddings.  The status and copy
-// count alternate between two words by frame parity, so the leader may
-// stage the next frame's while a slower CTA still reads this frame's.  A
-// frame with more pairs than the leader's hash takes (APH_MAX), or more
-// edges or edge roots than its union region holds, runs steps (1)-(3) on the
-// leader alone with the map's global pair hash.  Every branch that skips a
-// cluster barrier is taken by the whole cluster (its condition is read from
-// global memory written before the launch, or from the leader after a
-// barrier), so every CTA passes the same barriers.
+// an overlap item's icnt word: its voxels, and what k_gates found of its
+// segment against its instance as the batch starts
+constexpr int ITEM_COUNT = (1 << 26) - 1;
+constexpr int ITEM_KNOWN = 1 << 28, ITEM_EDGE = 1 << 29, ITEM_BORDER = 1 << 30;
+
+// The state of the frame a CTA works on.
+struct __align__(16) AssocShared {
+    unsigned long long pk[APH];             // (segment + 1) << 32 | root
+    unsigned long long best[ASSOC_ROOTS];   // per local root: best candidate of its component (cand_key)
+    long long cloc[ASSOC_ROOTS];            // voxel count
+    int pc[APH];                            // voxels of the pair
+    int pd[APH];                            // its ITEM_* flags
+    unsigned short pl[APH_MAX];             // used slots
+    unsigned rkey[ARH];                     // active roots
+    int rval[ARH];                          // local index of a root with an edge
+    int2 live[APH_MAX];                     // pairs to score now: (segment | root slot << 9, instance)
+    int gid[ASSOC_ROOTS];                   // local root -> instance id
+    int uf[ASSOC_ROOTS];                    // union-find over local roots
+    int obs[ASSOC_ROOTS];                   // observations of its component
+    int oloc[ASSOC_ROOTS];                  // observations
+    int em[ASSOC_EDGES];                    // accepted edges: segment and root slot
+    int eh[ASSOC_EDGES];
+    int anchor[MAX_MASKS];                  // smallest local root of a segment's edges
+    unsigned chg[ASSOC_CHG];                // bit hash(id): id's embedding changed in this batch
+    unsigned want[MAX_MASKS / 32];          // segments that open an instance
+    int err, ncopies;                       // the frame's status and embedding copies
+    int4 meta[ASSOC_FRAMES];                // the first frames' slot, n_pre, own error and masks
+    int ne, nlive, nloc, nroots, np, nsc, border, ovf, multi, ncopy, merges, next, merged_any, all_changed;
+};
+constexpr size_t ASSOC_SMEM = sizeof(AssocShared);
+constexpr size_t ASSOC_SMEM_ALONE = 216 * 1024;
+constexpr int RV_FREE = -1, RV_TAKEN = -2;
+
+// A fusion candidate as a number: the higher Q first, then the smaller order
+// (an instance id, or 2^31 + mask: members by id, then segments by mask).
+__device__ __forceinline__ unsigned long long cand_key(float q, unsigned order)
+{
+    return ((unsigned long long)f2key(q) << 32) | (unsigned)~order;
+}
+
+__device__ __forceinline__ unsigned chg_bit(int id) { return ((unsigned)id * 0x9E3779B1u) >> 18; }  // 14 bits
+static_assert(ASSOC_CHG * 32 == 1 << 14, "one bit per hash value");
+
+// Accepted edge (segment m, root slot h) number e: the first edge of a root
+// opens its local index with the instance's values.
+__device__ __forceinline__ void claim_root(AssocShared& A, int h, int k, long long cnt, float q, int obs)
+{
+    if (atomicCAS(&A.rval[h], RV_FREE, RV_TAKEN) != RV_FREE) return;
+    const int x = atomicAdd(&A.nloc, 1);
+    if (x < ASSOC_ROOTS) {
+        A.gid[x] = k;
+        A.uf[x] = x;
+        A.cloc[x] = cnt;
+        A.oloc[x] = A.obs[x] = obs;
+        A.best[x] = cand_key(q, (unsigned)k);
+    }
+    A.rval[h] = x;
+}
+
+// The cosine gate of every tag-0 item's segment against its instance as the
+// batch starts, one warp per item, all frames of the batch at once: most
+// instances keep their embedding through a batch, and k_associate then finds
+// the decision beside the item.  (Also for one frame per map: a Room frame's
+// 43 passing pairs, three rounds of k_associate's warps, cost it 8 us and the
+// launch 5.)
+__global__ void __launch_bounds__(256) k_gates(const FrameParams* fps, BatchScratch bs, BatchScratch view,
+                                               const MapRefs* refs)
+{
+    const int f = blockIdx.y;
+    const FrameParams& fp = fps[f];
+    const Scratch sc = bs.frame(f);
+    if (fp.M <= 0 || sc.ctr->err) return;  // a failed frame's items are never read
+    const int n = sc.ctr->n_pre, nw = (gridDim.x * blockDim.x) >> 5;
+    const Instances inst = refs[fp.map].inst;
+    const GateFeatures gf = gate_features(fp, sc, view.frame(f), inst);
+    for (int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < n; i += nw) {
+        const unsigned long long key = sc.ikey[i];
+        if ((key >> 32) & 1ull) continue;
+        int border = 0;
+        const bool edge = warp_cosine_gate(fp, gf, inst, (int)(key >> 33) - 1, (int)(unsigned)key, &border);
+        if ((threadIdx.x & 31) == 0)
+            sc.icnt[i] |= ITEM_KNOWN | (edge ? ITEM_EDGE : 0) | (border ? ITEM_BORDER : 0);
+    }
+}
+
+// One CTA per map of the batch walks the map's frames in order.  Per frame:
+//   (1) every item (its label resolved to the root as of now) adds to its
+//       (segment, root) pair in the shared pair hash;
+//   (2) a thread per pair: the overlap gate, the active roots, and the cosine
+//       gate where k_gates took it for the instance's embedding at the batch
+//       start and no frame has changed that since; the pairs left are scored
+//       now, a warp each;
+//   (3) components, new ids, merges and fusion winners, and the frame's new
+//       voxels into the counts;
+//   (4) a warp per embedding copy.
+// with a block barrier after each; step (4) runs beside the next frame's
+// step (1), which reads no embedding.  The next frame's items and segment
+// values are loaded while this one is united.  A frame past the shared
+// capacities runs steps (1)-(3) with the map's global pair hash and union
+// region.
+//
+// Bound by latency: a row of dependent steps per frame.  Room frames, 32 per
+// launch: 9.5 us per frame.  A cluster of 8 CTAs per map, whose leader's state
+// the others reached through distributed shared memory, took 15.2 us (every
+// passing pair scored between two cluster barriers, the union in fourteen
+// block barriers) and 11.8 with k_gates and this union: a cluster barrier that
+// orders global memory costs 1.2 us and empties the L1, a block barrier 0.03
+// us, and with the gates taken beforehand few pairs are left to share.
 __global__ void __launch_bounds__(ASSOC_THREADS, 1) k_associate(const FrameParams* fps, BatchScratch bs,
                                                                 SerialStep st)
 {
-    extern __shared__ __align__(16) unsigned char union_smem[];
-    __shared__ int s_np, s_ovf, s_ne, s_nsc, s_merged;
-    __shared__ int s_err[2], s_nc[2];  // by frame parity
-    const unsigned rank = cluster_rank(), C = cluster_size();
-    const bool leader = rank == 0;
-    const int g = blockIdx.x / C;
-    const int tid = threadIdx.x, lane = tid & 31, NT = blockDim.x;
+    extern __shared__ __align__(16) unsigned char assoc_smem[];
+    AssocShared& A = *(AssocShared*)assoc_smem;
+    const int g = blockIdx.x;
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    constexpr int NT = ASSOC_THREADS;
     // the map's table pointers, in shared memory: read there, they are never
     // reloaded from global memory after the kernel's own global stores
     __shared__ MapRefs s_refs;
     static_assert(sizeof(MapRefs) % 8 == 0, "copied in 8-byte words");
     for (int i = tid; i < (int)(sizeof(MapRefs) / 8); i += NT)
         ((unsigned long long*)&s_refs)[i] = ((const unsigned long long*)&st.refs[g])[i];
-    __syncthreads();
-    const MapRefs& R = s_refs;
-    const int ct = (int)rank * NT + tid, CT = (int)C * NT;               // thread within the cluster
-    const int cw = (int)rank * (NT >> 5) + (tid >> 5), CW = (int)C * (NT >> 5);  // warp within the cluster
-    // the leader's step (1)-(3) state, laid out as in its union_smem:
-    // pair hash, then the union's region (root hash of 2 * APH slots,
-    // per-root arrays, edges); the scored pairs (segment, instance) sit over
-    // the root hash, which the union fills only after the gates
-    unsigned long long* pk = (unsigned long long*)union_smem;  // [APH] (segment + 1) << 32 | root
-    int* pc = (int*)(pk + APH);                                 // [APH] voxels of the pair
-    int* pl = pc + APH;                                         // [APH] used slots
-    unsigned char* ureg = union_smem + (size_t)APH * 16;
-    int2* sp = (int2*)ureg;                                     // [APH_MAX] scored pairs
-    const UnionRegion U(ureg, 2 * APH, ASSOC_ROOTS, ASSOC_EDGES, true);
-    static_assert((size_t)APH_MAX * 8 <= (size_t)(2 * APH) * 8, "scored pairs fit over the root hash");
-    const unsigned r_pk = dsm_map(pk, 0), r_pc = dsm_map(pc, 0), r_pl = dsm_map(pl, 0), r_sp = dsm_map(sp, 0);
-    const unsigned r_em = dsm_map(U.em, 0), r_ek = dsm_map(U.ek, 0), r_ec = dsm_map(U.ec, 0);
-    const unsigned r_eq = dsm_map(U.eq, 0), r_eo = dsm_map(U.eo, 0);
-    const unsigned r_np = dsm_map(&s_np, 0), r_ovf = dsm_map(&s_ovf, 0), r_ne = dsm_map(&s_ne, 0);
-    const unsigned r_nsc = dsm_map(&s_nsc, 0), r_err = dsm_map(&s_err[0], 0), r_nc = dsm_map(&s_nc[0], 0);
-    if (leader) {
-        for (int i = tid; i < APH; i += NT) {
-            pk[i] = EMPTY_KEY;
-            pc[i] = 0;
-        }
-        if (tid == 0) {
-            *R.ss.edge_n = 0;
-            *R.ss.copy_n = 0;
-            s_merged = 0;
-            s_np = s_ovf = s_ne = s_nsc = 0;
-            s_err[0] = s_err[1] = 0;
-            s_nc[0] = s_nc[1] = 0;
-        }
+    for (int j = tid; j < min(st.J, ASSOC_FRAMES); j += NT) {
+        const int slot = st.slot_of[g * st.J + j];
+        A.meta[j] = slot < 0 ? make_int4(-1, 0, 0, 0)
+                             : make_int4(slot, bs.frame(slot).ctr->n_pre,
+                                         *(volatile const int32_t*)&bs.frame(slot).ctr->err, fps[slot].M);
     }
-    cluster_sync();
+    __syncthreads();
+    auto meta = [&](int j) -> int4 {
+        if (j < ASSOC_FRAMES) return A.meta[j];
+        const int slot = st.slot_of[g * st.J + j];
+        return slot < 0 ? make_int4(-1, 0, 0, 0)
+                        : make_int4(slot, bs.frame(slot).ctr->n_pre,
+                                    *(volatile const int32_t*)&bs.frame(slot).ctr->err, fps[slot].M);
+    };
+    const MapRefs& R = s_refs;
+    const Instances& inst = R.inst;
+    for (int i = tid; i < APH; i += NT) {
+        A.pk[i] = EMPTY_KEY;
+        A.pc[i] = A.pd[i] = 0;
+    }
+    for (int i = tid; i < ARH; i += NT) {
+        A.rkey[i] = UH_EMPTY;
+        A.rval[i] = RV_FREE;
+    }
+    for (int i = tid; i < MAX_MASKS; i += NT) A.anchor[i] = INT_MAX;
+    for (int i = tid; i < ASSOC_CHG; i += NT) A.chg[i] = 0u;
+    if (tid == 0) {
+        *R.ss.edge_n = 0;
+        *R.ss.copy_n = 0;
+        A.ne = A.nlive = A.nloc = A.nroots = A.np = A.nsc = A.border = A.ovf = A.multi = A.ncopy = A.merges = 0;
+        A.merged_any = A.all_changed = A.err = A.ncopies = 0;
+        A.next = *(volatile const int*)R.next_id;
+    }
+    // an item's (segment, root) pair: tag-1 items through the segment their
+    // voxel's first frame gave it to; known: the root is the one k_gates took
+    auto label_of = [&](unsigned long long key) -> int {
+        const unsigned x = (unsigned)key;
+        return ((key >> 32) & 1ull) ? bs.frame(st.slot_of[g * st.J + (int)(x >> 9)]).segrep[(x & 511u) - 1] : (int)x;
+    };
+    // the thread's first item of a frame and its segment's values, loaded ahead
+    unsigned long long pre_key = EMPTY_KEY;
+    int pre_cnt = 0, pre_nv = 0, pre_new = 0;
+    float pre_q = 0.0f;
+    auto prefetch = [&](int j) {
+        if (j >= st.J) return;
+        const int4 mt = meta(j);
+        if (mt.x < 0) return;
+        const Scratch sc = bs.frame(mt.x);
+        if (tid < mt.w) {
+            pre_nv = sc.nvox[tid];
+            pre_q = sc.S[5 * tid + 4];
+            pre_new = sc.newcnt[tid];
+        }
+        if (tid < mt.y) {
+            pre_key = sc.ikey[tid];
+            pre_cnt = sc.icnt[tid];
+        }
+    };
+    prefetch(0);
+    const int4 meta0 = meta(0);
+    const int ov_num = meta0.x < 0 ? 0 : fps[meta0.x].ov_num, ov_den = meta0.x < 0 ? 1 : fps[meta0.x].ov_den;
+    __syncthreads();
     for (int j = 0; j < st.J; j++) {
-        const int slot = st.slot_of[g * st.J + j];  // the same for the whole cluster
+        const int4 mt = meta(j);
+        const int slot = mt.x;
         if (slot < 0) break;
-        const int par = j & 1;
         const FrameParams& fp = fps[slot];
         const Scratch sc = bs.frame(slot);
+        const int M = mt.w;
         // blocked: the frame's own error (set before the launch), or its
-        // predecessor's status (staged by the leader before the last barrier)
-        const int prev = j > 0 ? dsm_ld32(r_err + 4u * (par ^ 1))
-                               : (st.prev_hist[g] >= 0 ? st.hist[st.prev_hist[g]].err : 0);
-        const int own = *(volatile const int32_t*)&sc.ctr->err;
+        // predecessor's status (staged before the last barrier)
+        const int prev = j > 0 ? A.err : (st.prev_hist[g] >= 0 ? st.hist[st.prev_hist[g]].err : 0);
+        const int own = mt.z;
         const bool blocked = own || prev;
-        if (leader && tid == 0 && !own && prev) set_err(sc.ctr, prev);
-        bool global_pairs = false;
-        // the leader's per-segment union inputs; up.ok: the union completed
-        // (and added the frame's new voxels to the counts)
-        UnionPre up{};
+        if (tid == 0 && !own && prev) set_err(sc.ctr, prev);
+        bool global_pairs = false, united = false;
         if (!blocked) {
-            const int npre = sc.ctr->n_pre;
-            // (1) overlap pairs: each item's label resolved to its root now
-            //     (four items per thread in flight)
-            for (int i0 = ct; i0 < npre; i0 += 4 * CT) {
-                unsigned long long key[4];
-                int cnt[4], lab[4];
-#pragma unroll
-                for (int u = 0; u < 4; u++) {
-                    const int i = i0 + u * CT;
-                    key[u] = i < npre ? sc.ikey[i] : EMPTY_KEY;
-                    cnt[u] = i < npre ? sc.icnt[i] : 0;
-                }
-#pragma unroll
-                for (int u = 0; u < 4; u++) {
-                    const unsigned x = (unsigned)key[u];
-                    lab[u] = -1;
-                    if (key[u] != EMPTY_KEY)
-                        lab[u] = ((key[u] >> 32) & 1ull)
-                                     ? bs.frame(st.slot_of[g * st.J + (int)(x >> 9)]).segrep[(x & 511u) - 1]
-                                     : (int)x;
-                }
-#pragma unroll
-                for (int u = 0; u < 4; u++) {
-                    if (lab[u] < 0) continue;
-                    const unsigned long long okey = ((key[u] >> 33) << 32) | (unsigned)find_root(R.inst.parent, lab[u]);
-                    unsigned h = (unsigned)(mix64(okey) & (APH - 1));
-                    for (int pr = 0;; pr++) {  // claim or find in one round trip per slot
-                        const unsigned long long prv = dsm_cas64(r_pk + 8u * h, EMPTY_KEY, okey);
-                        if (prv == EMPTY_KEY) {
-                            const int at = dsm_add(r_np, 1);
-                            if (at < APH_MAX) dsm_st32(r_pl + 4u * at, (int)h);
-                            else dsm_st32(r_ovf, 1);
-                            break;
-                        }
-                        if (prv == okey) break;
-                        h = (h + 1) & (APH - 1);
-                        if (pr >= APH) {
-                            dsm_st32(r_ovf, 1);
-                            break;
-                        }
+            const int nv = pre_nv, nnew = pre_new;
+            const float sq = pre_q;
+            // (1) overlap pairs
+            for (int i = tid; i < mt.y; i += NT) {
+                const unsigned long long key = i == tid ? pre_key : sc.ikey[i];
+                const int cnt = i == tid ? pre_cnt : sc.icnt[i];
+                const int lab = label_of(key);
+                if (lab < 0) continue;
+                const int root = find_root(inst.parent, lab);
+                const unsigned long long okey = ((key >> 33) << 32) | (unsigned)root;
+                unsigned h = (unsigned)(mix64(okey) & (APH - 1));
+                int pr = 0;
+                for (; pr < APH_PROBES; pr++) {
+                    const unsigned long long prv = atomicCAS(&A.pk[h], EMPTY_KEY, okey);
+                    if (prv == EMPTY_KEY) {
+                        const int at = atomicAdd(&A.np, 1);
+                        if (at < APH_MAX) A.pl[at] = (unsigned short)h;
                     }
-                    dsm_red_add(r_pc + 4u * h, cnt[u]);
+                    if (prv == EMPTY_KEY || prv == okey) break;
+                    h = (h + 1) & (APH - 1);
                 }
+                if (pr == APH_PROBES) {
+                    A.ovf = 1;
+                    continue;
+                }
+                atomicAdd(&A.pc[h], cnt & ITEM_COUNT);
+                // k_gates' decision holds for the root it saw
+                if ((cnt & ITEM_KNOWN) && root == lab) atomicOr(&A.pd[h], cnt & ~ITEM_COUNT);
             }
-            cluster_sync();
-            global_pairs = dsm_ld32(r_ovf) != 0;  // the whole cluster
+            __syncthreads();
+            const int np = A.np;
+            global_pairs = A.ovf || np > APH_MAX;  // uniform
             if (!global_pairs) {
-                const int np = dsm_ld32(r_np);
-                // (2a) overlap gate of pair i by thread i of the cluster:
-                //      |V_m & V_k| / min(|V_m|, |V_k|) >= ov_num / ov_den;
-                //      passing pairs to the scored list (one slot claim per warp)
-                for (int w0 = ct & ~31; w0 < np; w0 += CT) {  // whole warps iterate together
-                    const int i = w0 + lane;
-                    int m = 0, k = 0;
-                    bool pass = false;
-                    if (i < np) {
-                        const unsigned h = (unsigned)dsm_ld32(r_pl + 4u * i);
-                        const unsigned long long okey = dsm_ld64(r_pk + 8u * h);
-                        const long long ov = dsm_ld32(r_pc + 4u * h);
-                        m = (int)(okey >> 32) - 1;
-                        k = (int)(okey & 0xffffffffu);
-                        const long long denom = min((long long)sc.nvox[m], R.inst.count[k]);
-                        pass = ov * (long long)fp.ov_den >= (long long)fp.ov_num * denom;
+                // (2) |V_m & V_k| / min(|V_m|, |V_k|) >= ov_num / ov_den; the
+                //     hash is emptied on the way
+                int nsc = 0, nroot = 0, border = 0;
+                for (int i = tid; i < np; i += NT) {
+                    const int t = A.pl[i];
+                    const unsigned long long okey = A.pk[t];
+                    const int ov = A.pc[t], fl = A.pd[t];
+                    const int m = (int)(okey >> 32) - 1, k = (int)(okey & 0xffffffffu);
+                    const int nvm = sc.nvox[m], obs = inst.n_obs[k];
+                    const long long count = inst.count[k];
+                    const float q = inst.Q[k];
+                    A.pk[t] = EMPTY_KEY;
+                    A.pc[t] = A.pd[t] = 0;
+                    // active set: the distinct roots of all overlap pairs
+                    unsigned h = uhash((unsigned)k, ARH - 1);
+                    while (true) {  // at most APH_MAX roots in ARH slots
+                        const unsigned prv = atomicCAS(&A.rkey[h], UH_EMPTY, (unsigned)k);
+                        if (prv == UH_EMPTY) nroot++;
+                        if (prv == UH_EMPTY || prv == (unsigned)k) break;
+                        h = (h + 1) & (ARH - 1);
                     }
-                    const unsigned b = __ballot_sync(0xffffffffu, pass);
-                    int base = 0;
-                    if (lane == 0 && b) base = dsm_add(r_nsc, __popc(b));
-                    base = __shfl_sync(0xffffffffu, base, 0);
-                    if (pass) {
-                        const unsigned at = (unsigned)(base + __popc(b & ((1u << lane) - 1)));
-                        dsm_st32(r_sp + 8u * at, m);
-                        dsm_st32(r_sp + 8u * at + 4u, k);
+                    if ((long long)ov * ov_den < (long long)ov_num * min((long long)nvm, count)) continue;
+                    nsc++;
+                    const unsigned bit = chg_bit(k);
+                    if (!(fl & ITEM_KNOWN) || A.all_changed || ((A.chg[bit >> 5] >> (bit & 31)) & 1u)) {
+                        A.live[atomicAdd(&A.nlive, 1)] = make_int2(m | ((int)h << 9), k);
+                        continue;
                     }
+                    if (fl & ITEM_BORDER) border++;
+                    if (!(fl & ITEM_EDGE)) continue;
+                    const int e = atomicAdd(&A.ne, 1);
+                    if (e < ASSOC_EDGES) {
+                        A.em[e] = m;
+                        A.eh[e] = (int)h;
+                    }
+                    claim_root(A, (int)h, k, count, q, obs);
                 }
-                cluster_sync();
-                const int nsc = dsm_ld32(r_nsc);
-                if (leader && tid == 0) {
-                    sc.ctr->n_pairs = np;
-                    sc.ctr->n_scored = nsc;
+                const int sums = warp_sum(nroot | (nsc << 16));  // each at most APH_MAX / 16
+                border = warp_sum(border);
+                if (lane == 0 && sums) {
+                    atomicAdd(&A.nroots, sums & 0xffff);
+                    atomicAdd(&A.nsc, sums >> 16);
+                    if (border) atomicAdd(&A.border, border);
                 }
-                // (2b) cosine gate of scored pair s by warp s of the cluster
-                const GateFeatures gf = gate_features(fp, sc, st.view.frame(slot), R.inst);
-                int border = 0;
-                for (int q = cw; q < nsc; q += CW) {
-                    const int mm = dsm_ld32(r_sp + 8u * q), kk = dsm_ld32(r_sp + 8u * q + 4u);
-                    // the instance's values the union needs, read beside the gate
-                    const long long ck = lane == 0 ? R.inst.count[kk] : 0;
-                    const float qk = lane == 0 ? R.inst.Q[kk] : 0.0f;
-                    const int ok = lane == 0 ? R.inst.n_obs[kk] : 0;
-                    if (warp_cosine_gate(fp, gf, R.inst, mm, kk, &border) && lane == 0) {
-                        const int e = dsm_add(r_ne, 1);
+                __syncthreads();
+                const int nlive = A.nlive;
+                if (nlive > 0) {
+                    const GateFeatures gf = gate_features(fp, sc, st.view.frame(slot), inst);
+                    int rescored = 0;
+                    for (int q = wid; q < nlive; q += NT >> 5) {
+                        const int m = A.live[q].x & 511, h = A.live[q].x >> 9, k = A.live[q].y;
+                        // the instance's values the union needs, read beside the gate
+                        const long long ck = lane == 0 ? inst.count[k] : 0;
+                        const float qk = lane == 0 ? inst.Q[k] : 0.0f;
+                        const int ok = lane == 0 ? inst.n_obs[k] : 0;
+                        if (!warp_cosine_gate(fp, gf, inst, m, k, &rescored) || lane != 0) continue;
+                        const int e = atomicAdd(&A.ne, 1);
                         if (e < ASSOC_EDGES) {
-                            dsm_st32(r_em + 4u * e, mm);
-                            dsm_st32(r_ek + 4u * e, kk);
-                            dsm_st64(r_ec + 8u * e, (unsigned long long)ck);
-                            dsm_st32(r_eq + 4u * e, __float_as_int(qk));
-                            dsm_st32(r_eo + 4u * e, ok);
-                        }  // more edges than the shared list holds: the global path below
+                            A.em[e] = m;
+                            A.eh[e] = h;
+                        }
+                        claim_root(A, h, k, ck, qk, ok);
+                    }
+                    if (lane == 0 && rescored) atomicAdd(&A.border, rescored);
+                    __syncthreads();
+                }
+                global_pairs = A.ne > ASSOC_EDGES || A.nloc > ASSOC_ROOTS;  // uniform
+            }
+            // the next frame's items and segment values, on their way while
+            // this one is united
+            prefetch(j + 1);
+            if (!global_pairs) {
+                // (3) components: a segment joins every root it has an edge
+                //     with; a set's root is its smallest instance id
+                const int ne = A.ne, nloc = A.nloc;
+                for (int e = tid; e < ne; e += NT)
+                    if (atomicMin(&A.anchor[A.em[e]], A.rval[A.eh[e]]) != INT_MAX) A.multi = 1;
+                __syncthreads();
+                if (A.multi) {  // some segment has several edges: every edge hooks its root onto the segment's anchor
+                    for (int e = tid; e < ne; e += NT) {
+                        int x = A.rval[A.eh[e]], y = A.anchor[A.em[e]];
+                        while (true) {
+                            x = uf_find(A.uf, x);
+                            y = uf_find(A.uf, y);
+                            if (x == y) break;
+                            const int lo = A.gid[x] < A.gid[y] ? x : y, hi = lo == x ? y : x;
+                            if (atomicCAS(&A.uf[hi], hi, lo) == hi) break;
+                        }
+                    }
+                    __syncthreads();
+                    int root = -1;
+                    if (tid < nloc) root = uf_find(A.uf, tid);
+                    __syncthreads();
+                    if (tid < nloc) A.uf[tid] = root;
+                    __syncthreads();
+                }
+                // fusion candidates: the members of a component by id, then its
+                // segments by mask; the first with the highest Q wins.  New
+                // instances: live segments without an edge, in mask order.
+                int comp = -1;  // the segment's component
+                if (tid < MAX_MASKS) {
+                    if (tid < M && A.anchor[tid] != INT_MAX) comp = A.uf[A.anchor[tid]];
+                    const unsigned w = __ballot_sync(0xffffffffu, tid < M && nv > 0 && comp < 0);
+                    if (lane == 0) A.want[wid] = w;
+                    if (comp >= 0) {
+                        atomicMax(&A.best[comp], cand_key(sq, 0x80000000u | (unsigned)tid));
+                        atomicAdd(&A.obs[comp], 1);
+                    }
+                } else {
+                    const int x = tid - MAX_MASKS;
+                    if (x < nloc && A.uf[x] != x) {
+                        atomicMax(&A.best[A.uf[x]], A.best[x]);  // (only roots' entries change)
+                        atomicAdd(&A.obs[A.uf[x]], A.oloc[x]);
                     }
                 }
-                if (lane == 0 && border) atomicAdd(&sc.ctr->borderline, border);
-                // the leader reads its segments' values for the union while
-                // the cluster arrives (nothing in the cluster writes them)
-                cluster_arrive();
-                if (leader) {
-                    if (tid < fp.M) {
-                        up.nv = sc.nvox[tid];
-                        up.q = sc.S[5 * tid + 4];
-                        up.nnew = sc.newcnt[tid];
-                    }
-                    up.next = *(volatile const int*)R.next_id;
+                __syncthreads();
+                int first = 0, total = 0;
+#pragma unroll
+                for (int w = 0; w < MAX_MASKS / 32; w++) {
+                    const int c = __popc(A.want[w]);
+                    if (w < wid) first += c;
+                    total += c;
                 }
-                cluster_wait();
-                // (3) union, new ids, merges, fusion winners: the leader, in
-                //     its shared memory unless a shared capacity is exceeded
-                if (leader) {
-                    bool done = s_ne <= ASSOC_EDGES;
-                    if (done && !block_read(&sc.ctr->err)) {
-                        done = union_frame(fp, sc, R.ss, R.inst, R.next_id, ureg, 2 * APH, ASSOC_ROOTS, ASSOC_EDGES,
-                                           true, np, s_ne, true, [&](int i) { return (unsigned)(pk[pl[i]] & 0xffffffffu); },
-                                           &up);
+                const int base = A.next;
+                if (base + total > inst.cap) {  // uniform
+                    if (tid == 0) set_err(sc.ctr, DISC_ERR_CAPACITY);
+                    __syncthreads();
+                } else {
+                    united = true;
+                    if (tid < MAX_MASKS) {
+                        if (tid < M) {
+                            int rep = comp >= 0 ? A.gid[comp] : -1;
+                            if ((A.want[wid] >> lane) & 1u) {
+                                first += __popc(A.want[wid] & ((1u << lane) - 1));
+                                rep = base + first;
+                                inst.parent[rep] = rep;
+                                inst.count[rep] = nnew;
+                                inst.Q[rep] = sq;
+                                inst.n_obs[rep] = 1;
+                                R.ss.copy_dst[first] = rep;
+                                R.ss.copy_src[first] = -(tid + 1);
+                            } else if (rep >= 0 && nnew) {
+                                atomicAdd((unsigned long long*)&inst.count[rep], (unsigned long long)nnew);
+                            }
+                            sc.segrep[tid] = rep;
+                        }
+                    } else if (tid - MAX_MASKS < nloc) {
+                        const int x = tid - MAX_MASKS, r = A.uf[x], k = A.gid[x];
+                        if (r != x) {  // merged into its representative
+                            inst.parent[k] = A.gid[r];
+                            atomicAdd((unsigned long long*)&inst.count[A.gid[r]], (unsigned long long)A.cloc[x]);
+                            inst.count[k] = 0;
+                            atomicAdd(&A.merges, 1);
+                        } else {
+                            const unsigned order = ~(unsigned)A.best[x];
+                            inst.n_obs[k] = A.obs[x];
+                            if (order != (unsigned)k) {  // another member's or a segment's embedding
+                                const int c = total + atomicAdd(&A.ncopy, 1);
+                                R.ss.copy_dst[c] = k;
+                                R.ss.copy_src[c] = (order & 0x80000000u) ? -(int)(order & 0x7fffffffu) - 1 : (int)order;
+                                inst.Q[k] = key2f((unsigned)(A.best[x] >> 32));
+                                const unsigned bit = chg_bit(k);
+                                atomicOr(&A.chg[bit >> 5], 1u << (bit & 31));
+                            }
+                        }
                     }
-                    if (!done && tid == 0) {  // steps (1)-(3) again on global memory
-                        sc.ctr->n_pairs = 0;
-                        sc.ctr->n_scored = 0;
-                        sc.ctr->borderline = 0;
+                    __syncthreads();
+                    if (tid == 0) {
+                        FrameCounters* ctr = sc.ctr;
+                        ctr->n_pairs = np;
+                        ctr->n_scored = A.nsc;
+                        if (A.border) atomicAdd(&ctr->borderline, A.border);
+                        ctr->active_instances = A.nroots;
+                        ctr->new_instances = total;
+                        ctr->merges = A.merges;
+                        ctr->next_id = base + total;
+                        ctr->n_copies = total + A.ncopy;
+                        *R.next_id = base + total;
+                        A.next = base + total;
+                        if (A.merges) A.merged_any = 1;
+                        A.err = 0;
+                        A.ncopies = total + A.ncopy;
                     }
-                    global_pairs = !done;  // uniform in the leader
                 }
             }
-            if (leader && global_pairs) {
-                // more pairs, edges or edge roots than the leader's shared
-                // memory holds: the leader alone, with the map's global pair
-                // hash and union region
+            if (global_pairs) {
+                // more pairs, edges or edge roots than the shared memory holds:
+                // with the map's global pair hash and union region
                 __syncthreads();
-                for (int i = tid; i < npre; i += NT) {
+                for (int i = tid; i < mt.y; i += NT) {
                     const unsigned long long key = sc.ikey[i];
-                    const unsigned x = (unsigned)key;
-                    const int lab = ((key >> 32) & 1ull)
-                                        ? bs.frame(st.slot_of[g * st.J + (int)(x >> 9)]).segrep[(x & 511u) - 1]
-                                        : (int)x;
+                    const int lab = label_of(key);
                     if (lab >= 0)
-                        add_pair(sc, R.ss, ((key >> 33) << 32) | (unsigned)find_root(R.inst.parent, lab), sc.icnt[i]);
+                        add_pair(sc, R.ss, ((key >> 33) << 32) | (unsigned)find_root(inst.parent, lab),
+                                 sc.icnt[i] & ITEM_COUNT);
                 }
                 if (!block_read(&sc.ctr->err))
-                    phase_score(fp, sc, st.view.frame(slot), R.ss, R.inst, tid >> 5, NT >> 5);
-                if (!block_read(&sc.ctr->err)) phase_union(fp, sc, R.ss, R.inst, R.next_id, R.ss.ureg);
+                    phase_score(fp, sc, st.view.frame(slot), R.ss, inst, wid, NT >> 5);
+                if (!block_read(&sc.ctr->err)) phase_union(fp, sc, R.ss, inst, R.next_id, R.ss.ureg);
                 // empty the global pair hash
                 __syncthreads();
-                const int np = *(volatile int32_t*)&sc.ctr->n_pairs;
-                for (int i = tid; i < np; i += NT) {
+                const int ng = *(volatile int32_t*)&sc.ctr->n_pairs;
+                for (int i = tid; i < ng; i += NT) {
                     const int t = R.ss.olist[i];
                     R.ss.okeys[t] = EMPTY_KEY;
                     R.ss.ocnt[t] = 0;
                 }
             }
         }
-        // the leader closes the frame: its status and copy count for step (4)
-        // and the next frame, its pair hash emptied for the next frame
-        if (leader) {
-            __syncthreads();
-            const int err = up.ok ? 0 : *(volatile int32_t*)&sc.ctr->err;
-            const int nc = up.ok ? up.ncopy : err ? 0 : *(volatile int32_t*)R.ss.copy_n;
-            for (int i = tid; i < APH; i += NT) {
-                pk[i] = EMPTY_KEY;
-                pc[i] = 0;
-            }
-            if (tid == 0) {
-                s_err[par] = err;
-                s_nc[par] = nc;
-                s_np = s_ovf = s_ne = s_nsc = 0;
-            }
+        // the frame closes: its status and copy count for step (4) and the next
+        // frame, the shared state emptied
+        __syncthreads();
+        if (!united && tid == 0) {
+            const int err = *(volatile int32_t*)&sc.ctr->err;
+            A.err = err;
+            A.ncopies = err ? 0 : *(volatile int32_t*)R.ss.copy_n;
+            A.next = *(volatile const int*)R.next_id;
+            if (!err && *(volatile int32_t*)&sc.ctr->merges > 0) A.merged_any = 1;
+            if (!blocked) A.all_changed = 1;  // the global path keeps no record of changed embeddings
         }
-        cluster_sync();
-        // (4) the winners' embeddings (every warp of the cluster) and the
-        //     new voxels' counts (the leader)
-        if (!dsm_ld32(r_err + 4u * par)) {
+        for (int i = tid; i < ARH / 4; i += NT) {
+            ((uint4*)A.rkey)[i] = make_uint4(UH_EMPTY, UH_EMPTY, UH_EMPTY, UH_EMPTY);
+            ((int4*)A.rval)[i] = make_int4(RV_FREE, RV_FREE, RV_FREE, RV_FREE);
+        }
+        if (tid < MAX_MASKS) A.anchor[tid] = INT_MAX;
+        if (tid == 0)
+            A.ne = A.nlive = A.nloc = A.nroots = A.np = A.nsc = A.border = A.ovf = A.multi = A.ncopy = A.merges = 0;
+        if (global_pairs)  // pairs may be left where the walk never came
+            for (int i = tid; i < APH; i += NT) {
+                A.pk[i] = EMPTY_KEY;
+                A.pc[i] = A.pd[i] = 0;
+            }
+        if (blocked) prefetch(j + 1);
+        __syncthreads();
+        // (4) the winners' embeddings; on the global path also the new voxels
+        //     into the counts
+        if (!A.err) {
             const int D = fp.D;
-            const int nc = dsm_ld32(r_nc + 4u * par);
-            // from the cluster's last warp down: the first warps take the
-            // next frame's items, so the two run side by side
-            for (int c = CW - 1 - cw; c < nc; c += CW) {
+            const int nc = A.ncopies;
+            // from the last warp down: the first warps take the next frame's
+            // items, so the two run side by side
+            for (int c = (NT >> 5) - 1 - wid; c < nc; c += NT >> 5) {
                 const int src = R.ss.copy_src[c], dst = R.ss.copy_dst[c];
-                const Instances& inst = R.inst;
                 const float* from = src >= 0 ? inst.E + (size_t)src * D : sc.Ecan + (size_t)(-src - 1) * D;
                 if (inst.A) {
                     const Scratch va = st.view.frame(slot);
@@ -1748,22 +1878,18 @@ __global__ void __launch_bounds__(ASSOC_THREADS, 1) k_associate(const FrameParam
                     if (inst.E8) e4m3_copy_row(from, D, inst.E8 + (size_t)dst * D, inst.Er + dst);
                 }
             }
-            if (leader) {
-                for (int m = tid; m < fp.M && !up.ok; m += NT) {
+            if (!united && !blocked)
+                for (int m = tid; m < M; m += NT) {
                     const int n = sc.newcnt[m], rep = sc.segrep[m];
-                    if (n && rep >= 0) atomicAdd((unsigned long long*)&R.inst.count[rep], (unsigned long long)n);
+                    if (n && rep >= 0) atomicAdd((unsigned long long*)&inst.count[rep], (unsigned long long)n);
                 }
-                if (tid == 0 && (up.ok ? up.merges : sc.ctr->merges) > 0) s_merged = 1;
-            }
         }
-        if (leader && tid == 0) {
+        if (tid == 0 && !united) {
             *R.ss.edge_n = 0;
             *R.ss.copy_n = 0;
         }
     }
-    // no CTA leaves while another may still reach its shared memory
-    cluster_sync();
-    if (leader && tid == 0) st.merged[g] = s_merged;
+    if (tid == 0) st.merged[g] = A.merged_any;
 }
 
 // After the batch's frames: every voxel of the absent-voxel hash whose first
@@ -1895,8 +2021,8 @@ int launch_serial_step(const FrameParams* fps, const BatchScratch& bs, const Ser
     }
 }
 
-int launch_lookup(const FrameParams* fps, const BatchScratch& bs, const MapRefs* refs, const AbsentHash& ah, int S,
-                  int probe_width, cudaStream_t st)
+int launch_lookup(const FrameParams* fps, const BatchScratch& bs, const BatchScratch& view, const MapRefs* refs,
+                  const AbsentHash& ah, int S, int probe_width, cudaStream_t st)
 {
     const dim3 grid(152, S);
     switch (probe_width) {
@@ -1906,71 +2032,20 @@ int launch_lookup(const FrameParams* fps, const BatchScratch& bs, const MapRefs*
         default: k_lookup1<<<grid, LK_THREADS, 0, st>>>(fps, bs, refs, ah); break;
     }
     k_absent<<<dim3(38, S), 256, 0, st>>>(fps, bs, ah);
-    k_items<<<dim3(16, S), 256, 0, st>>>(bs);
-    return 3;
-}
-
-// CTAs per map: a cluster of up to 8 when the maps leave SMs free (152 SMs,
-// one CTA each); checked once against what the device can co-schedule.
-static int g_assoc_max_cluster = -1;  // set once by set_serial_kernel_attrs
-
-static void probe_assoc_cluster()
-{
-    if (g_assoc_max_cluster < 0) {
-        int& max_c = g_assoc_max_cluster;
-        max_c = 1;
-        for (int c = ASSOC_CLUSTER_MAX; c > 1; c >>= 1) {
-            cudaLaunchConfig_t cfg = {};
-            cudaLaunchAttribute at[1];
-            at[0].id = cudaLaunchAttributeClusterDimension;
-            at[0].val.clusterDim.x = c;
-            at[0].val.clusterDim.y = 1;
-            at[0].val.clusterDim.z = 1;
-            cfg.gridDim = dim3(c);
-            cfg.blockDim = dim3(ASSOC_THREADS);
-            cfg.dynamicSmemBytes = ASSOC_SMEM;
-            cfg.attrs = at;
-            cfg.numAttrs = 1;
-            int n = 0;
-            if (cudaOccupancyMaxActiveClusters(&n, k_associate, &cfg) == cudaSuccess && n > 0) {
-                max_c = c;
-                break;
-            }
-            cudaGetLastError();
-        }
-    }
-}
-
-static int assoc_cluster(int G, int want)
-{
-    int c = 1;
-    if (want > 0) {
-        while (c * 2 <= want && c * 2 <= g_assoc_max_cluster) c *= 2;
-        return c;
-    }
-    while (c * 2 <= g_assoc_max_cluster && (c * 2) * G <= 152) c *= 2;
-    return c;
+    k_items<<<dim3(16, S), 256, 0, st>>>(fps, bs, refs);
+    k_gates<<<dim3(32, S), 256, 0, st>>>(fps, bs, view, refs);
+    return 4;
 }
 
 size_t union_region_bytes_full() { return UNION_SMEM; }
 
-int launch_associate(const FrameParams* fps, const BatchScratch& bs, const SerialStep& st, int G, int cluster,
-                     cudaStream_t s)
+int launch_associate(const FrameParams* fps, const BatchScratch& bs, const SerialStep& st, int G, cudaStream_t s)
 {
-    const int c = assoc_cluster(G, cluster);
-    cudaLaunchConfig_t cfg = {};
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = c;
-    at[0].val.clusterDim.y = 1;
-    at[0].val.clusterDim.z = 1;
-    cfg.gridDim = dim3(G * c);
-    cfg.blockDim = dim3(ASSOC_THREADS);
-    cfg.dynamicSmemBytes = ASSOC_SMEM;
-    cfg.stream = s;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    cudaLaunchKernelEx(&cfg, k_associate, fps, bs, st);
+    // A CTA of few maps keeps its SM to itself (a row of dependent steps that
+    // shares its issue slots with stateless blocks runs 1.4 times as long):
+    // it asks for all of the SM's shared memory.
+    const size_t smem = G <= 4 ? ASSOC_SMEM_ALONE : ASSOC_SMEM;
+    k_associate<<<G, ASSOC_THREADS, smem, s>>>(fps, bs, st);
     return 1;
 }
 
@@ -1984,8 +2059,7 @@ cudaError_t set_serial_kernel_attrs()
 {
     cudaError_t e = cudaFuncSetAttribute(k_union, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)UNION_SMEM);
     if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_associate, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ASSOC_SMEM);
-    if (e == cudaSuccess) probe_assoc_cluster();
+        e = cudaFuncSetAttribute(k_associate, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ASSOC_SMEM_ALONE);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k_overlap, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)OV_SMEM);
     return e;
 }
