@@ -891,6 +891,8 @@ disc_status ensure_instance_room(disc_map* m, int64_t incoming, cudaStream_t st)
     return DISC_OK;
 }
 
+constexpr size_t kKeepQueryBytes = 64 << 20;  // query scratch a map keeps between calls
+
 // device scratch of at least `bytes` for query calls (no allocation once it
 // is large enough: a freed buffer would synchronise the device each call)
 unsigned char* query_scratch(disc_map* m, size_t bytes)
@@ -2581,12 +2583,10 @@ disc_status disc_map_counts(disc_map* m, int64_t* nv, int32_t* nid)
     return DISC_OK;
 }
 
-disc_status disc_map_export_voxels(disc_map* m, uint64_t* keys, int32_t* ids, int64_t cap)
+// The map's voxels on the host, sorted there: maps whose voxels lie too far
+// apart for a bitmap over their box.
+static disc_status export_voxels_host(disc_map* m, uint64_t* keys, int32_t* ids, int64_t cap)
 {
-    if (!m || (cap > 0 && (!keys || !ids))) return DISC_ERR_INVALID_ARG;
-    CK(cudaSetDevice(m->cfg.device));
-    wait_pending(m);
-    CK(cudaStreamSynchronize(m->stream));
     const uint64_t tc = m->vt.mask + 1;
     std::vector<unsigned long long> k(tc);
     std::vector<int32_t> l(tc);
@@ -2605,6 +2605,78 @@ disc_status disc_map_export_voxels(disc_map* m, uint64_t* keys, int32_t* ids, in
         ids[i] = v[i].second;
     }
     return DISC_OK;
+}
+
+disc_status disc_map_export_voxels(disc_map* m, uint64_t* keys, int32_t* ids, int64_t cap)
+{
+    if (!m || (cap > 0 && (!keys || !ids))) return DISC_ERR_INVALID_ARG;
+    CK(cudaSetDevice(m->cfg.device));
+    wait_pending(m);
+    CK(cudaStreamSynchronize(m->stream));
+    const uint64_t n = read_used(m, m->stream);
+    if ((int64_t)n > cap) return DISC_ERR_INVALID_ARG;
+    if (n == 0) return DISC_OK;
+    // The bitmap over the voxels' box pays up to 512 MB, and while it has no
+    // more than 4096 bits per voxel (its passes then move no more than a few
+    // times what the table holds).
+    constexpr uint64_t kMaxBits = 1ull << 32;
+    if (n >= (1ull << 31) || m->vt.mask >= (1ull << 32)) return export_voxels_host(m, keys, ids, cap);
+    cudaStream_t st = m->stream;
+    ExportScratch es{};
+    const size_t b_head = 256, b_list = align256(sizeof(unsigned) * n);
+    const size_t b_keys = align256(sizeof(unsigned long long) * n), b_ids = align256(sizeof(int32_t) * n);
+    unsigned char* base = query_scratch(m, b_head + b_list);
+    if (!base) return export_voxels_host(m, keys, ids, cap);
+    es.head = (int*)base;
+    es.list = (unsigned*)(base + b_head);
+    es.list_cap = (int)n;
+    int head[7] = {0, INT_MAX, INT_MAX, INT_MAX, INT_MIN, INT_MIN, INT_MIN};
+    CK(cudaMemcpyAsync(es.head, head, sizeof(head), cudaMemcpyHostToDevice, st));
+    launch_export_list(m->vt, es, st);
+    CK(cudaMemcpyAsync(head, es.head, sizeof(head), cudaMemcpyDeviceToHost, st));
+    const int nid = read_next_id(m, st);  // waits for both
+    if (head[0] != (int)n) return export_voxels_host(m, keys, ids, cap);
+    uint64_t ext[3];
+    for (int a = 0; a < 3; a++) ext[a] = (uint64_t)((int64_t)head[4 + a] - head[1 + a] + 1);
+    // (three extents of at most 2^18: no overflow)
+    const uint64_t volume = ext[0] * ext[1] * ext[2];
+    if (volume > kMaxBits || volume > std::max<uint64_t>(1ull << 26, 4096 * n))
+        return export_voxels_host(m, keys, ids, cap);
+    es.n = (int)n;
+    for (int a = 0; a < 3; a++) es.lo[a] = head[1 + a];
+    es.ny = ext[1];
+    es.nz = ext[2];
+    es.groups = (long long)((volume + 1023) / 1024);
+    const long long spans = (es.groups + EXPORT_SPAN - 1) / EXPORT_SPAN;
+    const size_t b_bits = align256(128 * (size_t)es.groups), b_before = align256(sizeof(int) * (size_t)es.groups);
+    const size_t b_spans = align256(sizeof(int) * (size_t)spans);
+    const size_t all = b_head + b_list + b_keys + b_ids + b_bits + b_before + b_spans;
+    if (all > m->qcap) {  // a larger buffer: the list is made again in it
+        base = query_scratch(m, all);
+        if (!base) return export_voxels_host(m, keys, ids, cap);
+        es.head = (int*)base;
+        es.list = (unsigned*)(base + b_head);
+        CK(cudaMemsetAsync(es.head, 0, sizeof(int), st));
+        launch_export_list(m->vt, es, st);
+    }
+    unsigned char* p = base + b_head + b_list;
+    es.keys = (unsigned long long*)p;
+    es.ids = (int32_t*)(p + b_keys);
+    es.bits = (unsigned*)(p + b_keys + b_ids);
+    es.before = (int*)(p + b_keys + b_ids + b_bits);
+    es.spans = (int*)(p + b_keys + b_ids + b_bits + b_before);
+    CK(cudaMemsetAsync(es.bits, 0, b_bits, st));
+    launch_export_place(m->vt, m->inst.parent, nid, es, st);
+    CK(cudaMemcpyAsync(keys, es.keys, sizeof(uint64_t) * n, cudaMemcpyDeviceToHost, st));
+    CK(cudaMemcpyAsync(ids, es.ids, sizeof(int32_t) * n, cudaMemcpyDeviceToHost, st));
+    CK(cudaGetLastError());
+    const disc_status s = cuda_status(cudaStreamSynchronize(st));
+    if (m->qcap > kKeepQueryBytes) {  // a large map's scratch goes back
+        m->mem.release(m->qscratch, m->qcap);
+        m->qscratch = nullptr;
+        m->qcap = 0;
+    }
+    return s;
 }
 
 disc_status disc_map_export_assoc(disc_map* m, float* A, int32_t cap)

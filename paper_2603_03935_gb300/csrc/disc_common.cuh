@@ -411,6 +411,23 @@ struct FinalizeScratch {
     unsigned long long* removed_voxels;
 };
 
+// Sorted export of a map's voxels (k_export.cu)
+constexpr int EXPORT_SPAN = 8192;  // counts that one block scans
+struct ExportScratch {
+    int* head;                  // [7] voxels listed; least and largest x, y, z
+    unsigned* list;             // [list_cap] occupied table slots
+    int list_cap;
+    int n;                      // voxels
+    int lo[3];                  // the box's least corner
+    unsigned long long ny, nz;  // its extents in y and z
+    unsigned* bits;             // [groups * 32] one bit per voxel of the box, x major, z minor
+    long long groups;           // 1024-bit groups of them
+    int* before;                // [groups] set bits of the span before the group
+    int* spans;                 // [groups / EXPORT_SPAN, rounded up] set bits before the span
+    unsigned long long* keys;   // [n] the export
+    int32_t* ids;               // [n]
+};
+
 // One step of the serial part over the maps of a batch: block row g runs the
 // j-th frame of map g.
 struct SerialStep {

@@ -97,6 +97,12 @@ cudaError_t set_serial_kernel_attrs();
 int launch_finalize(int phase, const VoxelTable& vt, const Instances& inst, int nid, int D, const FinalizeScratch& fs,
                     int min_voxels, int num, int den, float tau, cudaStream_t st);
 
+// voxels sorted by key (k_export.cu): the occupied slots and their box, then
+// (with the box's extents and a zeroed bitmap) the export in place
+void launch_export_list(const VoxelTable& vt, const ExportScratch& es, cudaStream_t st);
+void launch_export_place(const VoxelTable& vt, const int32_t* parent, int nid, const ExportScratch& es,
+                         cudaStream_t st);
+
 // maintenance and queries
 void launch_rehash(const VoxelTable& from, const VoxelTable& to, int* err, cudaStream_t st);
 void launch_query_topk(const float* q, int nq, int D, const Instances& inst, int nid, float* scores, int k,
