@@ -126,7 +126,9 @@ __device__ __forceinline__ void unpack_key(unsigned long long key, int k[3])
 // voxels of a block have eight consecutive home slots (64 bytes of keys, 32 of
 // labels), so a surface's lookups read a fraction of the sectors that slots
 // hashed voxel by voxel do, and a voxel's neighbours lie in at most eight
-// places.  The probe sequence keeps the place within the eight and moves on
+// places.  A block's hash also permutes its eight, so that maps of voxels of
+// one parity (a floor one voxel thick) fill every place alike.  The probe
+// sequence keeps the place within the eight and moves on
 // by whole groups: two blocks hashed to one group (half full, as surfaces
 // are) collide only where both hold a voxel, and the sequence's length is that
 // of plain hashing at the same load.  (Moving on slot by slot chained the
@@ -137,7 +139,8 @@ __device__ __forceinline__ unsigned long long vt_home(unsigned long long key, un
 {
     const unsigned long long low = (1ull << (2 * KEY_BITS)) | (1ull << KEY_BITS) | 1ull;
     const unsigned long long local = ((key >> (2 * KEY_BITS - 2)) & 4) | ((key >> (KEY_BITS - 1)) & 2) | (key & 1);
-    return ((mix64(key & ~low) << 3) | local) & mask;
+    const unsigned long long h = mix64(key & ~low);
+    return ((h << 3) | (local ^ (h >> 61))) & mask;
 }
 // the slot after h, the n-th of the sequence (n = 1 for the home slot)
 __device__ __forceinline__ unsigned long long vt_next(unsigned long long h, unsigned long long n,
