@@ -27,60 +27,130 @@ __global__ void k_rehash(VoxelTable from, VoxelTable to, int* err)
 }
 
 // ---- queries -----------------------------------------------------------------------
-// cosine of each query against every live instance; scores [nq][nid]
-__global__ void k_query_scores(const float* q, int nq, int D, Instances inst, int nid, float* scores)
+// cosine of each query against every live instance; scores [nq][nid].  A block
+// holds QUERY_TILE queries in shared memory (in chunks of the dimension) and
+// each of its warps four instances, whose rows it reads once for all of them;
+// the norms are taken beside.  Every sum keeps its order (a lane its dimensions
+// in turn, then the lanes by halves), so scores do not depend on the tiling.
+// Bound by the shared-memory reads of the queries.  4000 instances x 64
+// queries of 768: 122 us with a warp per (query, instance), which read both
+// rows and took both norms each time; 45 us so.
+constexpr int QUERY_TILE = 8, QUERY_DIM = 1024, QUERY_INST = 4, QUERY_WARPS = 8;
+static_assert(QUERY_TILE * QUERY_INST == 32 && QUERY_WARPS == QUERY_TILE, "a lane per product, a warp per query's norm");
+
+__global__ void __launch_bounds__(32 * QUERY_WARPS) k_query_scores(const float* q, int nq, int D, Instances inst,
+                                                                   int nid, float* scores)
 {
-    const int lane = threadIdx.x & 31;
-    const int qi = blockIdx.y;
-    const int i = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    if (i >= nid || qi >= nq) return;
-    float s = -INFINITY;
-    if (inst.parent[i] == i && inst.n_obs[i] > 0) {  // live (a dropped instance has no observations)
-        const float* a = q + (size_t)qi * D;
-        const float* b = inst.E + (size_t)i * D;
-        float dt = 0.0f, na = 0.0f, nb = 0.0f;
-        for (int d = lane; d < D; d += 32) {
-            dt += a[d] * b[d];
-            na += a[d] * a[d];
-            nb += b[d] * b[d];
-        }
-        dt = warp_sum(dt);
-        na = warp_sum(na);
-        nb = warp_sum(nb);
-        s = (na > 0.0f && nb > 0.0f) ? dt / (sqrtf(na) * sqrtf(nb)) : 0.0f;
+    __shared__ float qs[QUERY_TILE][QUERY_DIM];
+    __shared__ float s_na[QUERY_TILE];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int q0 = blockIdx.y * QUERY_TILE;
+    const int i0 = (blockIdx.x * QUERY_WARPS + warp) * QUERY_INST;
+    const float* row[QUERY_INST];
+    unsigned live = 0;  // (a dropped instance has no observations)
+#pragma unroll
+    for (int u = 0; u < QUERY_INST; u++) {
+        const int i = i0 + u;
+        if (i < nid && inst.parent[i] == i && inst.n_obs[i] > 0) live |= 1u << u;
+        row[u] = inst.E + (size_t)((live >> u) & 1u ? i : 0) * D;
     }
-    if (lane == 0) scores[(size_t)qi * nid + i] = s;
+    float dt[32] = {}, nb[QUERY_INST] = {}, na = 0.0f;  // product (u, t) in dt[u * QUERY_TILE + t]
+    for (int c0 = 0; c0 < D; c0 += QUERY_DIM) {
+        const int cn = min(QUERY_DIM, D - c0);
+        __syncthreads();
+        for (int t = 0; t < QUERY_TILE; t++)
+            for (int d = threadIdx.x; d < cn; d += 32 * QUERY_WARPS)
+                qs[t][d] = q0 + t < nq ? q[(size_t)(q0 + t) * D + c0 + d] : 0.0f;
+        __syncthreads();
+        for (int d = lane; d < cn; d += 32) na += qs[warp][d] * qs[warp][d];
+#pragma unroll 2
+        for (int d = lane; d < cn; d += 32) {
+            float b[QUERY_INST];
+#pragma unroll
+            for (int u = 0; u < QUERY_INST; u++) b[u] = row[u][c0 + d];
+#pragma unroll
+            for (int u = 0; u < QUERY_INST; u++) nb[u] += b[u] * b[u];
+#pragma unroll
+            for (int t = 0; t < QUERY_TILE; t++) {
+                const float a = qs[t][d];
+#pragma unroll
+                for (int u = 0; u < QUERY_INST; u++) dt[u * QUERY_TILE + t] += a * b[u];
+            }
+        }
+    }
+    na = warp_sum(na);
+    if (lane == 0) s_na[warp] = na;
+    float nbl = 0.0f;  // of the lane's instance
+#pragma unroll
+    for (int u = 0; u < QUERY_INST; u++) {
+        const float n = warp_sum(nb[u]);
+        if (lane / QUERY_TILE == u) nbl = n;
+    }
+    // the 32 sums, one to a lane: as the lanes halve, so do the sums each holds
+    // (the additions of every sum are those of a butterfly of its own)
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const bool upper = lane & o;
+#pragma unroll
+        for (int i = 0; i < o; i++) {
+            const float keep = upper ? dt[i + o] : dt[i], give = upper ? dt[i] : dt[i + o];
+            dt[i] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+        }
+    }
+    __syncthreads();
+    const int u = lane / QUERY_TILE, t = lane % QUERY_TILE;
+    const float n = s_na[t];
+    const float s = (n > 0.0f && nbl > 0.0f) ? dt[0] / (sqrtf(n) * sqrtf(nbl)) : 0.0f;
+    if (q0 + t < nq && i0 + u < nid) scores[(size_t)(q0 + t) * nid + i0 + u] = (live >> u) & 1u ? s : -INFINITY;
 }
 
-// k best per query: repeated block arg-max (score descending, id ascending)
-__global__ void k_query_topk(float* scores, int nid, int k, int* ids, float* out)
+// k best per query (score descending, id ascending).  A thread keeps the best
+// of its share of the scores; each round the block takes the best of those,
+// and only its owner looks its share over again.  (A pass of the block over
+// all scores per round took 22 us for 10 of 4000, 11 us so.)
+constexpr int TOPK_THREADS = 512;
+
+__global__ void __launch_bounds__(TOPK_THREADS) k_query_topk(float* scores, int nid, int k, int* ids, float* out)
 {
-    __shared__ float bs[32];
-    __shared__ int bi[32];
-    const int qi = blockIdx.x;
+    __shared__ unsigned long long best[TOPK_THREADS / 32];
+    const int qi = blockIdx.x, tid = threadIdx.x, lane = tid & 31;
     float* sc = scores + (size_t)qi * nid;
+    // score and id as one number (0: no score above -inf, NaN among them):
+    // the higher score first (-0 as 0), then the smaller id
+    auto mine = [&]() -> unsigned long long {
+        unsigned long long m = 0ull;
+        for (int i = tid; i < nid; i += TOPK_THREADS) {
+            const float s = sc[i];
+            if (!(s > -INFINITY)) continue;
+            const unsigned b = __float_as_uint(s + 0.0f);
+            const unsigned key = (b & 0x80000000u) ? ~b : (b | 0x80000000u);
+            m = max(m, ((unsigned long long)key << 32) | (unsigned)~i);
+        }
+        return m;
+    };
+    unsigned long long own = mine();
     for (int j = 0; j < k; j++) {
-        float best = -INFINITY;
-        int bid = INT_MAX;
-        for (int i = threadIdx.x; i < nid; i += blockDim.x) {
-            float s = sc[i];
-            if (s > best || (s == best && i < bid)) { best = s; bid = i; }
-        }
-        for (int o = 16; o > 0; o >>= 1) {
-            float s2 = __shfl_xor_sync(0xffffffffu, best, o);
-            int i2 = __shfl_xor_sync(0xffffffffu, bid, o);
-            if (s2 > best || (s2 == best && i2 < bid)) { best = s2; bid = i2; }
-        }
-        if ((threadIdx.x & 31) == 0) { bs[threadIdx.x >> 5] = best; bi[threadIdx.x >> 5] = bid; }
+        unsigned long long m = own;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+        if (lane == 0) best[tid >> 5] = m;
         __syncthreads();
-        if (threadIdx.x == 0) {
-            for (int w = 1; w < (int)(blockDim.x >> 5); w++)
-                if (bs[w] > bs[0] || (bs[w] == bs[0] && bi[w] < bi[0])) { bs[0] = bs[w]; bi[0] = bi[w]; }
-            const bool found = bi[0] != INT_MAX && bs[0] > -INFINITY;
-            ids[(size_t)qi * k + j] = found ? bi[0] : -1;
-            out[(size_t)qi * k + j] = found ? bs[0] : -INFINITY;
-            if (found) sc[bi[0]] = -INFINITY;
-            else bi[0] = INT_MAX;
+        m = best[0];
+#pragma unroll
+        for (int w = 1; w < TOPK_THREADS / 32; w++) m = max(m, best[w]);
+        if (m == 0ull) {  // none left (uniform)
+            for (int r = j + tid; r < k; r += TOPK_THREADS) {
+                ids[(size_t)qi * k + r] = -1;
+                out[(size_t)qi * k + r] = -INFINITY;
+            }
+            return;
+        }
+        if (own == m) {
+            const int i = (int)~(unsigned)m;
+            ids[(size_t)qi * k + j] = i;
+            out[(size_t)qi * k + j] = sc[i];
+            sc[i] = -INFINITY;
+            own = mine();
         }
         __syncthreads();
     }
@@ -133,9 +203,10 @@ void launch_rehash(const VoxelTable& from, const VoxelTable& to, int* err, cudaS
 void launch_query_topk(const float* q, int nq, int D, const Instances& inst, int nid, float* scores, int k,
                        int* ids, float* out, cudaStream_t st)
 {
-    dim3 g((nid + 7) / 8, nq);
-    k_query_scores<<<g, 256, 0, st>>>(q, nq, D, inst, nid, scores);
-    k_query_topk<<<nq, 256, 0, st>>>(scores, nid, k, ids, out);
+    const int per = QUERY_WARPS * QUERY_INST;
+    const dim3 g((nid + per - 1) / per, (nq + QUERY_TILE - 1) / QUERY_TILE);
+    k_query_scores<<<g, 32 * QUERY_WARPS, 0, st>>>(q, nq, D, inst, nid, scores);
+    k_query_topk<<<nq, TOPK_THREADS, 0, st>>>(scores, nid, k, ids, out);
 }
 
 void launch_query_points(const float* xyz, long long n, float voxel, const VoxelTable& vt, const Instances& inst,

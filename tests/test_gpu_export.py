@@ -39,3 +39,45 @@ def test_export_is_sorted_and_complete(offsets, width, height):
     assert lib.disc_map_export_voxels(gmap._h, keys.ctypes.data, ids.ctypes.data, n + 5) == 0
     assert (np.diff(keys.astype(np.int64)) > 0).all()
     gmap.close()
+
+
+@pytest.mark.parametrize("nid,nq,k,dim", [(3, 1, 5, 7), (96, 9, 20, 64), (97, 8, 1, 1030), (700, 17, 96, 60)])
+def test_topk_at_tile_edges(nid, nq, k, dim):
+    """Scores within fp32 rounding of float64, ids ordered by (score, id); dead instances and padding at the end."""
+    import torch
+    from paper_2603_03935_gb300 import DiscMap, device_frame
+    dev = torch.device("cuda:0")
+    gen = torch.Generator(device=dev).manual_seed(nid + dim)
+    per = min(nid, 96)
+    frames, made = [], 0
+    gmap = DiscMap(voxel_size=0.025, embed_dim=dim, patch_h=8, patch_w=12, max_width=96, max_height=64, max_masks=96,
+                   min_mask_pixels=1, voxel_capacity=1 << 16, max_load=0.5, instance_capacity=128)
+    v, u = torch.arange(64, device=dev)[:, None] // 8, torch.arange(96, device=dev)[None, :] // 8
+    while made < nid:
+        n = min(per, nid - made)
+        labels = (v * 12 + u + 1).clamp(max=97)
+        labels = torch.where(labels <= n, labels, torch.zeros_like(labels)).to(torch.int16).contiguous()
+        pose = np.eye(4)
+        pose[0, 3] = 40.0 * len(frames)
+        tokens = torch.randn(96, dim, device=dev, generator=gen)
+        frames.append(device_frame(torch.full((64, 96), 2.0, device=dev), labels, tokens, pose, (80.0, 80.0, 48.0, 32.0), n))
+        made += n
+    gmap.integrate_frames(frames)
+    E = gmap.instances()["E"]
+    assert len(E) == nid
+    if dim % 2 == 0:
+        q = E[:nq] + 0.1 * np.random.default_rng(1).normal(size=(nq, dim)).astype(np.float32)
+    else:
+        q = np.repeat(E[:1], nq, 0)  # equal queries: equal answers
+    ids, sc = gmap.query_topk(q, k)
+    e64, q64 = E.astype(np.float64), q.astype(np.float64)
+    want = q64 @ e64.T / (np.linalg.norm(q64, axis=1)[:, None] * np.linalg.norm(e64, axis=1))
+    m = min(k, nid)
+    assert (ids[:, m:] == -1).all() and np.isneginf(sc[:, m:]).all()
+    assert np.abs(np.take_along_axis(want, ids[:, :m], 1) - sc[:, :m]).max() <= 3 * dim * 2.0 ** -24 + 2.0 ** -22
+    assert all(len(set(r)) == m for r in ids[:, :m].tolist())
+    for r, s in zip(ids[:, :m], sc[:, :m]):
+        assert all(s[i] > s[i + 1] or (s[i] == s[i + 1] and r[i] < r[i + 1]) for i in range(m - 1))
+    best = -np.sort(-want, axis=1)[:, :m]
+    assert np.abs(best - sc[:, :m]).max() <= 3 * dim * 2.0 ** -24 + 2.0 ** -22
+    gmap.close()
