@@ -135,12 +135,16 @@ __device__ __forceinline__ void unpack_key(unsigned long long key, int k[3])
 // groups: a commit of 1,700 voxels at load 0.25 took 29 us in the place of
 // 15.)  After a whole round at one place it moves to the next, so every slot
 // is reached.
+__device__ __forceinline__ unsigned long long vt_place(unsigned long long h, unsigned long long key,
+                                                       unsigned long long mask)  // h: mix64 of the block's least key
+{
+    const unsigned long long local = ((key >> (2 * KEY_BITS - 2)) & 4) | ((key >> (KEY_BITS - 1)) & 2) | (key & 1);
+    return ((h << 3) | (local ^ (h >> 61))) & mask;
+}
 __device__ __forceinline__ unsigned long long vt_home(unsigned long long key, unsigned long long mask)
 {
     const unsigned long long low = (1ull << (2 * KEY_BITS)) | (1ull << KEY_BITS) | 1ull;
-    const unsigned long long local = ((key >> (2 * KEY_BITS - 2)) & 4) | ((key >> (KEY_BITS - 1)) & 2) | (key & 1);
-    const unsigned long long h = mix64(key & ~low);
-    return ((h << 3) | (local ^ (h >> 61))) & mask;
+    return vt_place(mix64(key & ~low), key, mask);
 }
 // the slot after h, the n-th of the sequence (n = 1 for the home slot)
 __device__ __forceinline__ unsigned long long vt_next(unsigned long long h, unsigned long long n,

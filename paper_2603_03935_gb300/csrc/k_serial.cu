@@ -30,6 +30,7 @@ __device__ __forceinline__ void set_err(FrameCounters* c, int code) { atomicCAS(
 // to the new-voxel hash with the lowest segment that contains them.
 constexpr int SER_THREADS = 1024;
 constexpr int OV_SLOTS = 2 * SER_THREADS;
+constexpr int OV_PROBES = 64;  // longest probe of the shared pair hash
 
 // label of a key in the voxel table, -1 if absent
 __device__ __forceinline__ int vt_label(const VoxelTable& vt, unsigned long long key)
@@ -70,44 +71,60 @@ __device__ void add_pair(const Scratch& sc, const SerialScratch& ss, unsigned lo
 
 // Neighbourhood overlap (overlap_dilation): segment voxel `key` (label lab,
 // -1 if absent) overlaps each distinct instance labelling it or one of its 26
-// neighbours, once.  One entry may add up to 27 pairs, so they go straight to
-// the frame's pair hash.
-__device__ void dilated_pairs(const Scratch& sc, const SerialScratch& ss, const VoxelTable& vt, const Instances& inst,
-                              int m, unsigned long long key, int lab)
+// neighbours, once: their roots into roots[27], returns how many.  Nine
+// neighbours at a time (one x offset), whose table slots, labels and parents
+// are each loaded together; they lie in four blocks of the table, hashed once
+// each.  Only a collision walks on.
+__device__ __forceinline__ int dilated_roots(const VoxelTable& vt, const Instances& inst, unsigned long long key,
+                                             int lab, int roots[27])
 {
-    int roots[27];
     int nr = 0;
     if (lab >= 0) roots[nr++] = inst.parent[lab];
     int k[3];
     unpack_key(key, k);
-    // nine neighbours at a time (one x offset): every first probe slot loaded
-    // at once; only a collision walks on
+#pragma unroll 1
     for (int dx = -1; dx <= 1; dx++) {
-        unsigned long long nk[9], cur[9];
-        unsigned long long h[9];
-        bool in[9];
+        const int x = k[0] + dx;
+        if (x < -KEY_BIAS || x > KEY_BIAS - 1) continue;
+        unsigned long long nk[9], h[9], cur[9], block[4];
+        int nl[9];
+        // blocks of the lower and upper y and z neighbours
+        const unsigned long long bx = (unsigned long long)((x + KEY_BIAS) & ~1) << (2 * KEY_BITS);
+        const int y0 = (k[1] - 1 + KEY_BIAS) >> 1, z0 = (k[2] - 1 + KEY_BIAS) >> 1;
+#pragma unroll
+        for (int q = 0; q < 4; q++)
+            block[q] = mix64(bx | ((unsigned long long)(unsigned)(2 * (y0 + (q >> 1))) << KEY_BITS) |
+                             (unsigned long long)(unsigned)(2 * (z0 + (q & 1))));
 #pragma unroll
         for (int j = 0; j < 9; j++) {
-            const int q[3] = {k[0] + dx, k[1] + j / 3 - 1, k[2] + j % 3 - 1};
-            in[j] = !(dx == 0 && j == 4) && q[0] >= -KEY_BIAS && q[0] <= KEY_BIAS - 1 && q[1] >= -KEY_BIAS &&
-                    q[1] <= KEY_BIAS - 1 && q[2] >= -KEY_BIAS && q[2] <= KEY_BIAS - 1;
-            nk[j] = ((unsigned long long)(q[0] + KEY_BIAS) << (2 * KEY_BITS)) |
-                    ((unsigned long long)(q[1] + KEY_BIAS) << KEY_BITS) | (unsigned long long)(q[2] + KEY_BIAS);
-            h[j] = vt_home(nk[j], vt.mask);
-            cur[j] = in[j] ? vt.keys[h[j]] : EMPTY_KEY;
+            const int y = k[1] + j / 3 - 1, z = k[2] + j % 3 - 1;
+            const bool in = !(dx == 0 && j == 4) && y >= -KEY_BIAS && y <= KEY_BIAS - 1 && z >= -KEY_BIAS &&
+                            z <= KEY_BIAS - 1;
+            nk[j] = ((unsigned long long)(x + KEY_BIAS) << (2 * KEY_BITS)) |
+                    ((unsigned long long)(y + KEY_BIAS) << KEY_BITS) | (unsigned long long)(z + KEY_BIAS);
+            const bool uy = ((y + KEY_BIAS) >> 1) != y0, uz = ((z + KEY_BIAS) >> 1) != z0;
+            const unsigned long long b = uy ? (uz ? block[3] : block[2]) : (uz ? block[1] : block[0]);
+            h[j] = vt_place(b, nk[j], vt.mask);
+            cur[j] = in ? vt.keys[h[j]] : EMPTY_KEY;
         }
 #pragma unroll
         for (int j = 0; j < 9; j++) {
-            if (!in[j] || cur[j] == EMPTY_KEY) continue;
-            const int nl = cur[j] == nk[j] ? vt.labels[h[j]] : vt_label(vt, nk[j]);
-            if (nl < 0) continue;
-            const int r = inst.parent[nl];
+            nl[j] = -1;
+            if (cur[j] == EMPTY_KEY) continue;
+            nl[j] = cur[j] == nk[j] ? vt.labels[h[j]] : vt_label(vt, nk[j]);
+        }
+#pragma unroll
+        for (int j = 0; j < 9; j++)
+            if (nl[j] >= 0) nl[j] = inst.parent[nl[j]];
+#pragma unroll
+        for (int j = 0; j < 9; j++) {
+            if (nl[j] < 0 || (j > 0 && nl[j] == nl[j - 1])) continue;  // (neighbours mostly share their root)
             bool seen = false;
-            for (int t = 0; t < nr; t++) seen |= roots[t] == r;
-            if (!seen) roots[nr++] = r;
+            for (int t = 0; t < nr; t++) seen |= roots[t] == nl[j];
+            if (!seen) roots[nr++] = nl[j];
         }
     }
-    for (int j = 0; j < nr; j++) add_pair(sc, ss, ((unsigned long long)m << 32) | (unsigned)roots[j]);
+    return nr;
 }
 
 __device__ void phase_overlap(const Scratch& sc, const SerialScratch& ss, const VoxelTable& vt, const Instances& inst,
@@ -142,17 +159,24 @@ __device__ void phase_overlap(const Scratch& sc, const SerialScratch& ss, const 
                     h = vt_next(h, pr + 1, vt.mask);
                 }
             }
-            if (dilate) dilated_pairs(sc, ss, vt, inst, m, key, lab);
-            if (lab >= 0 && !dilate) {
-                const unsigned long long okey = ((unsigned long long)m << 32) | (unsigned)inst.parent[lab];
+            // an entry adds one pair, or up to 27 (then a pair that finds no
+            // place in the shared hash goes straight to the frame's)
+            int roots[27];
+            const int nr = dilate ? dilated_roots(vt, inst, key, lab, roots)
+                                  : lab >= 0 ? (roots[0] = inst.parent[lab], 1) : 0;
+            for (int r = 0; r < nr; r++) {
+                const unsigned long long okey = ((unsigned long long)m << 32) | (unsigned)roots[r];
                 unsigned t = (unsigned)(mix64(okey) & (OV_SLOTS - 1));
-                while (true) {
+                int pr = 0;
+                for (; pr < OV_PROBES; pr++) {
                     const unsigned long long prev = atomicCAS(&pkey[t], EMPTY_KEY, okey);
                     if (prev == EMPTY_KEY || prev == okey) break;
                     t = (t + 1) & (OV_SLOTS - 1);
                 }
-                atomicAdd(&pcnt[t], 1);
-            } else if (lab < 0) {
+                if (pr < OV_PROBES) atomicAdd(&pcnt[t], 1);
+                else add_pair(sc, ss, okey);
+            }
+            if (lab < 0) {
                 unsigned long long t = mix64(key) & ss.nmask;
                 for (int pr = 0;; pr++) {
                     const unsigned long long cur = ss.nkeys[t];
