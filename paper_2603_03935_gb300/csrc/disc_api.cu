@@ -1320,18 +1320,16 @@ disc_status frame_params(Runner& r, const disc_map* m, const disc_frame* f, int 
     fp.Pw = r.Pw;
     fp.Kpad = r.Kpad;
     fp.Npad = std::max(16, (fp.M + 15) / 16 * 16);
-    fp.fx = f->fx;
-    fp.fy = f->fy;
-    fp.cx = f->cx;
-    fp.cy = f->cy;
+    fp.cam.cx = f->cx;
+    fp.cam.cy = f->cy;
     for (int i = 0; i < 3; i++) {
-        for (int c = 0; c < 3; c++) fp.R[3 * i + c] = (float)f->T_world_cam[4 * i + c];
-        fp.t[i] = (float)f->T_world_cam[4 * i + 3];
+        for (int c = 0; c < 3; c++) fp.cam.R[3 * i + c] = (float)f->T_world_cam[4 * i + c];
+        fp.cam.t[i] = (float)f->T_world_cam[4 * i + 3];
     }
     fp.voxel = m->cfg.voxel_size;
     // reciprocals rounded once to fp32 (host fp32 division is IEEE)
-    fp.inv_fx = 1.0f / f->fx;
-    fp.inv_fy = 1.0f / f->fy;
+    fp.cam.inv_fx = 1.0f / f->fx;
+    fp.cam.inv_fy = 1.0f / f->fy;
     fp.inv_voxel = 1.0f / m->cfg.voxel_size;
     fp.z_min = m->cfg.z_min;
     fp.z_max = m->cfg.z_max;

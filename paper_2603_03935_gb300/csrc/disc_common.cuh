@@ -73,16 +73,20 @@ __device__ __forceinline__ double unfix(long long n, int S)
 }
 
 // fp32 of n * 2^-S, rounded as double first and then as float.  Below 2^53
-// in magnitude the double is exact, so the value rounds once: its 32 leading
-// bits, the dropped ones gathered in the last of them, convert to fp32 (8
-// bits below the significand, so the gathered one decides ties only), then
-// an exact power of two.  Conversions from 64-bit integers run on the fp64
-// pipe, which this keeps idle.
+// in magnitude the double is exact, so the value rounds once.  Below 2^40 a
+// fused multiply-add of n's two parts, each exact in fp32, rounds it; from
+// there its 32 leading bits, the dropped ones gathered in the last of them,
+// convert to fp32 (8 bits below the significand, so the gathered one decides
+// ties only).  Conversions from 64-bit integers run on the fp64 pipe, which
+// this keeps idle.
 __device__ __forceinline__ float unfix32f(long long n, int S)
 {
+    if ((unsigned long long)(n + (1ll << 40)) < (1ull << 41)) {
+        const float hi = (float)(int)(n >> 16), lo = (float)(int)(n & 0xffff);
+        return __fmaf_rn(hi, __int_as_float((127 + 16 - S) << 23), __fmul_rn(lo, __int_as_float((127 - S) << 23)));
+    }
     const unsigned long long u = n < 0 ? 0ull - (unsigned long long)n : (unsigned long long)n;
     if (u >> 53) return __double2float_rn(unfix(n, S));
-    if (u == 0) return 0.0f;
     const int lz = __clzll((long long)u);
     const unsigned long long m = u << lz;
     const unsigned top = (unsigned)(m >> 32) | ((unsigned)m != 0u ? 1u : 0u);
@@ -462,14 +466,20 @@ struct AbsentHash {
     unsigned long long mask;    // cap - 1
 };
 
-// frame parameters passed by value
-struct FrameParams {
-    int32_t H, W, M, P, D, Ph, Pw, Kpad, Npad;
-    float fx, fy, cx, cy;
+// The camera of a frame, first in its parameters: four 16-byte loads.
+struct __align__(16) Camera {
     float R[9];
     float t[3];
+    float cx, cy;
+    float inv_fx, inv_fy;  // 1/fx, 1/fy rounded once to fp32
+};
+
+// frame parameters passed by value
+struct __align__(16) FrameParams {
+    Camera cam;
+    int32_t H, W, M, P, D, Ph, Pw, Kpad, Npad;
     float voxel, z_min, z_max, eps, tau, lambda_size;
-    float inv_fx, inv_fy, inv_voxel;   // 1/fx, 1/fy, 1/voxel rounded once to fp32
+    float inv_voxel;       // 1/voxel rounded once to fp32
     int32_t ov_num, ov_den, min_px;
     int32_t token_bf16;
     int32_t map;           // position of the frame's map in the batch (MapRefs index)
@@ -490,15 +500,15 @@ struct FrameParams {
 };
 
 // ---- Sec. III-A: world point of pixel (u, v) at depth z -------------------------
-__device__ __forceinline__ void world_point(const FrameParams& fp, int u, int v, float z, float p[3])
+__device__ __forceinline__ void world_point(const Camera& c, int u, int v, float z, float p[3])
 {
-    float xc = __fmul_rn(__fmul_rn(__fsub_rn(__fadd_rn((float)u, 0.5f), fp.cx), z), fp.inv_fx);
-    float yc = __fmul_rn(__fmul_rn(__fsub_rn(__fadd_rn((float)v, 0.5f), fp.cy), z), fp.inv_fy);
+    float xc = __fmul_rn(__fmul_rn(__fsub_rn(__fadd_rn((float)u, 0.5f), c.cx), z), c.inv_fx);
+    float yc = __fmul_rn(__fmul_rn(__fsub_rn(__fadd_rn((float)v, 0.5f), c.cy), z), c.inv_fy);
 #pragma unroll
     for (int r = 0; r < 3; r++)
-        p[r] = __fadd_rn(__fadd_rn(__fadd_rn(__fmul_rn(fp.R[3 * r], xc), __fmul_rn(fp.R[3 * r + 1], yc)),
-                                   __fmul_rn(fp.R[3 * r + 2], z)),
-                         fp.t[r]);
+        p[r] = __fadd_rn(__fadd_rn(__fadd_rn(__fmul_rn(c.R[3 * r], xc), __fmul_rn(c.R[3 * r + 1], yc)),
+                                   __fmul_rn(c.R[3 * r + 2], z)),
+                         c.t[r]);
 }
 
 // ---- E4M3 (OCP FP8: 4 exponent bits, 3 mantissa bits, largest finite 448) ----

@@ -167,7 +167,7 @@ __global__ void k_db_points(const FrameParams* fps, BatchScratch bs, int f0)
         lab = fp.labels[idx];
         const float z = fp.depth[idx];
         if (lab >= 1 && lab <= fp.M && sc.npix[lab - 1] >= fp.min_px && z >= fp.z_min && z <= fp.z_max) {
-            world_point(fp, u, v, z, p);
+            world_point(fp.cam, u, v, z, p);
             unsigned long long vk;
             pt = voxel_key(p[0], p[1], p[2], fp.inv_voxel, &vk);
         }

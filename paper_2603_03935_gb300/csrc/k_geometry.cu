@@ -91,13 +91,14 @@ __global__ void k_slot_reset(BatchScratch bs, int B)
 // the pixels first meet in a shared hash that sums their normals, and only
 // the tile's distinct keys become records, so many pixels of one voxel do not
 // pile up in one partition.
-// Bound by instruction issue and by the latency of the loads and counters
-// (42 % issue active).  Measured on Room frames (640x480, 2.5 cm voxels, 8
-// frames per launch) in place of one global (segment, voxel) hash per frame
-// with 32-byte slots, whose probes and three 64-bit atomics per key missed
-// L2: 18.1 -> 7.2 us per frame, and 2.6 -> 0.3 us for clearing the slot; with
-// k_entries (4.5 -> 7.9 us) 25.2 -> 15.4 us.  The partition counters lie a
-// cache line apart: side by side (8 to a sector) the same kernel took 28.8 us.
+// Bound by instruction issue (58 % active) and by the scattered record stores
+// and counter increments, one line per lane (L1 70 % busy).  Measured on Room
+// frames (640x480, 2.5 cm voxels, 8 frames per launch) in place of one global
+// (segment, voxel) hash per frame with 32-byte slots, whose probes and three
+// 64-bit atomics per key missed L2: 18.1 -> 6.9 us per frame, and 2.6 -> 0.3 us
+// for clearing the slot; with k_entries (4.5 -> 7.3 us, they now also sum the
+// pixels) 25.2 -> 14.5 us.  The partition counters lie a cache line apart: side
+// by side (8 to a sector) the kernel took 28.8 us.
 constexpr int BP_TX = 32, BP_TY = 16, BP_PER = 2;      // tile; pixels per thread (rows 2 ty and 2 ty + 1)
 constexpr int BP_ROWS = BP_TY / BP_PER, BP_THREADS = BP_TX * BP_ROWS;
 constexpr int BP_HX = BP_TX + 2, BP_HY = BP_TY + 2, BP_HALO = BP_HX * BP_HY;
@@ -108,24 +109,21 @@ struct __align__(16) TilePoint {
     int lab;   // mask label if the pixel has valid depth (and is inside the image), else 0
 };
 
-// Normal of the pixel at halo position (hx, hy) as three fixed-point
-// components; zero when it has none.
-__device__ __forceinline__ void pixel_normal(const FrameParams& fp, const TilePoint* tp, int at, const TilePoint& me,
+// Normal of a pixel from its neighbours to the right, left, below and above,
+// as three fixed-point components; zero when it has none.
+__device__ __forceinline__ void pixel_normal(const float t[3], const TilePoint& me, const TilePoint& right,
+                                             const TilePoint& left, const TilePoint& below, const TilePoint& above,
                                              long long nfix[3])
 {
-    nfix[0] = nfix[1] = nfix[2] = 0;
     // image-space tangents: forward differences, backward at the mask's
     // edge; a neighbour counts if it has valid depth and the same label
-    TilePoint a = tp[at + 1], c = tp[at + BP_HX];
-    const bool fa = a.lab == me.lab, fc = c.lab == me.lab;
-    if (!fa) a = tp[at - 1];
-    if (!fc) c = tp[at - BP_HX];
-    if (a.lab != me.lab || c.lab != me.lab) return;
+    const bool fa = right.lab == me.lab, fc = below.lab == me.lab;
+    if ((!fa && left.lab != me.lab) || (!fc && above.lab != me.lab)) return;
     float e1[3], e2[3], n[3];
 #pragma unroll
     for (int r = 0; r < 3; r++) {
-        e1[r] = fa ? __fsub_rn(a.p[r], me.p[r]) : __fsub_rn(me.p[r], a.p[r]);
-        e2[r] = fc ? __fsub_rn(c.p[r], me.p[r]) : __fsub_rn(me.p[r], c.p[r]);
+        e1[r] = fa ? __fsub_rn(right.p[r], me.p[r]) : __fsub_rn(me.p[r], left.p[r]);
+        e2[r] = fc ? __fsub_rn(below.p[r], me.p[r]) : __fsub_rn(me.p[r], above.p[r]);
     }
     n[0] = __fsub_rn(__fmul_rn(e2[1], e1[2]), __fmul_rn(e2[2], e1[1]));
     n[1] = __fsub_rn(__fmul_rn(e2[2], e1[0]), __fmul_rn(e2[0], e1[2]));
@@ -136,9 +134,9 @@ __device__ __forceinline__ void pixel_normal(const FrameParams& fp, const TilePo
 #pragma unroll
     for (int r = 0; r < 3; r++) n[r] = __fmul_rn(n[r], il);
     // orient toward the camera
-    const float vd = __fadd_rn(__fadd_rn(__fmul_rn(__fsub_rn(me.p[0], fp.t[0]), n[0]),
-                                         __fmul_rn(__fsub_rn(me.p[1], fp.t[1]), n[1])),
-                               __fmul_rn(__fsub_rn(me.p[2], fp.t[2]), n[2]));
+    const float vd = __fadd_rn(__fadd_rn(__fmul_rn(__fsub_rn(me.p[0], t[0]), n[0]),
+                                         __fmul_rn(__fsub_rn(me.p[1], t[1]), n[1])),
+                               __fmul_rn(__fsub_rn(me.p[2], t[2]), n[2]));
 #pragma unroll
     for (int r = 0; r < 3; r++) nfix[r] = fix_split<S_VEC>(vd > 0.0f ? -n[r] : n[r]);
 }
@@ -167,36 +165,52 @@ __global__ void __launch_bounds__(BP_THREADS) k_backproject(const FrameParams* f
         const unsigned act = __ballot_sync(0xffffffffu, tid < M && sc.npix[tid] >= fp.min_px);
         if (lane == 0) s_act[threadIdx.y] = act;
     }
-    // tile + halo: label (0 unless the depth is valid) and world point; all of
-    // a thread's pixels are loaded before the first is used
-    constexpr int PER = (BP_HALO + BP_THREADS - 1) / BP_THREADS;
-    int plab[PER];
-    float pz[PER];
+    // The thread's two pixels and, in the first threads, one of the halo: label
+    // (0 unless the depth is valid) and world point, into the tile; all loaded
+    // before the first is used.
+    static_assert(BP_PER == 2 && BP_HALO - BP_TX * BP_TY <= BP_THREADS, "two pixels and at most one of the halo");
+    const Camera cam = fp.cam;
+    const int at0 = (2 * threadIdx.y + 1) * BP_HX + threadIdx.x + 1;
+    int hx = 0, hy = 0;  // the halo pixel: top and bottom rows, then left and right columns
+    const bool halo = tid < BP_HALO - BP_TX * BP_TY;
+    if (tid < 2 * BP_HX) {
+        hx = tid < BP_HX ? tid : tid - BP_HX;
+        hy = tid < BP_HX ? 0 : BP_HY - 1;
+    } else {
+        const int k = tid - 2 * BP_HX;
+        hx = k < BP_TY ? 0 : BP_HX - 1;
+        hy = 1 + (k < BP_TY ? k : k - BP_TY);
+    }
+    int plab[3];
+    float pz[3];
 #pragma unroll
-    for (int j = 0; j < PER; j++) {
-        const int i = tid + j * BP_THREADS;
-        const int hu = u0 + i % BP_HX, hv = v0 + i / BP_HX;
+    for (int j = 0; j < 3; j++) {
+        const int u = u0 + (j < 2 ? (int)threadIdx.x + 1 : hx), v = v0 + (j < 2 ? 2 * (int)threadIdx.y + 1 + j : hy);
         plab[j] = 0;
         pz[j] = 0.0f;
-        if (i < BP_HALO && hu >= 0 && hv >= 0 && hu < W && hv < H) {
-            const int idx = hv * W + hu;
+        if ((j < 2 || halo) && (unsigned)u < (unsigned)W && (unsigned)v < (unsigned)H) {
+            const int idx = v * W + u;
             plab[j] = fp.labels[idx];
             pz[j] = fp.depth[idx];
             // a DBSCAN noise pixel counts as invalid depth
             if (fp.db_min_pts > 0 && (sc.dflag[idx] & 2)) plab[j] = 0;
         }
     }
+    const float z_min = fp.z_min, z_max = fp.z_max, inv_voxel = fp.inv_voxel;
+    TilePoint me[BP_PER];
 #pragma unroll
-    for (int j = 0; j < PER; j++) {
-        const int i = tid + j * BP_THREADS;
+    for (int j = 0; j < 3; j++) {
+        if (j == 2 && !halo) break;
         TilePoint t;
         t.lab = 0;
         t.p[0] = t.p[1] = t.p[2] = 0.0f;
-        if (plab[j] >= 1 && plab[j] <= M && pz[j] >= fp.z_min && pz[j] <= fp.z_max) {
+        if (plab[j] >= 1 && plab[j] <= M && pz[j] >= z_min && pz[j] <= z_max) {
             t.lab = plab[j];
-            world_point(fp, u0 + i % BP_HX, v0 + i / BP_HX, pz[j], t.p);
+            world_point(cam, u0 + (j < 2 ? (int)threadIdx.x + 1 : hx), v0 + (j < 2 ? 2 * (int)threadIdx.y + 1 + j : hy),
+                        pz[j], t.p);
         }
-        if (i < BP_HALO) tp[i] = t;
+        if (j < 2) me[j < 2 ? j : 0] = t;
+        tp[j < 2 ? at0 + j * BP_HX : hy * BP_HX + hx] = t;
     }
     __syncthreads();
     if (s_err) return;
@@ -205,17 +219,17 @@ __global__ void __launch_bounds__(BP_THREADS) k_backproject(const FrameParams* f
     int nvalid = 0, ndrop = 0, nrun = 0;
 #pragma unroll
     for (int j = 0; j < BP_PER; j++) {
-        const int at = (threadIdx.y * BP_PER + j + 1) * BP_HX + threadIdx.x + 1;
-        const TilePoint me = tp[at];
+        const int at = at0 + j * BP_HX;
         hk[j] = 0ull;
         nfix[j][0] = nfix[j][1] = nfix[j][2] = 0;
-        const int lab = me.lab;
+        const int lab = me[j].lab;
         const bool active = lab > 0 && ((s_act[(lab - 1) >> 5] >> ((lab - 1) & 31)) & 1u);
         unsigned long long key = 0;
-        const bool keyed = active && voxel_key(me.p[0], me.p[1], me.p[2], fp.inv_voxel, &key);
+        const bool keyed = active && voxel_key(me[j].p[0], me[j].p[1], me[j].p[2], inv_voxel, &key);
         if (keyed) {
             hk[j] = ((unsigned long long)lab << 54) | key;
-            pixel_normal(fp, tp, at, me, nfix[j]);
+            pixel_normal(cam.t, me[j], tp[at + 1], tp[at - 1], j == 0 ? me[1] : tp[at + BP_HX],
+                         j == 0 ? tp[at - BP_HX] : me[0], nfix[j]);
         }
         nvalid += __popc(__ballot_sync(0xffffffffu, keyed));
         ndrop += __popc(__ballot_sync(0xffffffffu, active && !keyed));
@@ -236,7 +250,6 @@ __global__ void __launch_bounds__(BP_THREADS) k_backproject(const FrameParams* f
     }
     // the thread's two pixels, then the pixels of two neighbouring threads,
     // add up where they share a voxel
-    static_assert(BP_PER == 2, "a pair");
     if (hk[0] == hk[1]) {
         hk[1] = 0ull;
 #pragma unroll
@@ -437,7 +450,7 @@ __global__ void __launch_bounds__(SEG_THREADS) k_entries(const FrameParams* fps,
                 float r[3];
 #pragma unroll
                 for (int a = 0; a < 3; a++)
-                    r[a] = __fsub_rn(__fmul_rn(__fadd_rn((float)k[a], 0.5f), fp.voxel), fp.t[a]);
+                    r[a] = __fsub_rn(__fmul_rn(__fadd_rn((float)k[a], 0.5f), fp.voxel), fp.cam.t[a]);
                 float rl2 = __fadd_rn(__fadd_rn(__fmul_rn(r[0], r[0]), __fmul_rn(r[1], r[1])), __fmul_rn(r[2], r[2]));
                 if (rl2 > 0.0f) {
                     float rl = __fsqrt_rn(rl2);
