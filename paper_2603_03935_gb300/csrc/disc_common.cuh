@@ -422,6 +422,17 @@ struct FinalizeScratch {
     unsigned long long* removed_voxels;
 };
 
+// The instance table on its way to the host (k_export.cu): pinned memory
+struct TableStage {
+    int* n;                     // [1] ids handed out
+    int rows;                   // rows the arrays hold
+    long long* count;
+    int* parent;
+    float* Q;
+    int* n_obs;
+    float* E;                   // [rows][D], or NULL
+};
+
 // Sorted export of a map's voxels (k_export.cu)
 constexpr int EXPORT_SPAN = 8192;  // counts that one block scans
 struct ExportScratch {

@@ -137,10 +137,36 @@ __global__ void k_export_place(VoxelTable vt, const int32_t* parent, int nid, Ex
     }
 }
 
+// Instance table into pinned host memory, the rows handed out so far (none
+// when they are more than fit)
+__global__ void k_stage_table(Instances inst, const int* next_id, int D, TableStage ts)
+{
+    const int n = *next_id;
+    const long long at = (long long)blockIdx.x * blockDim.x + threadIdx.x, step = (long long)gridDim.x * blockDim.x;
+    if (at == 0) *ts.n = n;
+    if (n > ts.rows) return;
+    for (long long i = at; i < n; i += step) {
+        ts.count[i] = inst.count[i];
+        ts.parent[i] = inst.parent[i];
+        ts.Q[i] = inst.Q[i];
+        ts.n_obs[i] = inst.n_obs[i];
+    }
+    if (!ts.E) return;
+    const long long words = (long long)n * D, quads = words >> 2;
+    for (long long i = at; i < quads; i += step) ((float4*)ts.E)[i] = ((const float4*)inst.E)[i];
+    for (long long i = 4 * quads + at; i < words; i += step) ts.E[i] = inst.E[i];
+}
+
 // ---- host launchers ------------------------------------------------------------------
 void launch_export_list(const VoxelTable& vt, const ExportScratch& es, cudaStream_t st)
 {
     k_export_list<<<152 * 8, 256, 0, st>>>(vt, es);
+}
+
+void launch_stage_table(const Instances& inst, const int* next_id, int D, const TableStage& ts, cudaStream_t st)
+{
+    const long long quads = (long long)ts.rows * (ts.E ? D / 4 + 1 : 1);
+    k_stage_table<<<(int)(quads / 256 + 1 < 152 ? quads / 256 + 1 : 152), 256, 0, st>>>(inst, next_id, D, ts);
 }
 
 // es.bits zero; at most EXPORT_SPAN spans

@@ -103,6 +103,9 @@ void launch_export_list(const VoxelTable& vt, const ExportScratch& es, cudaStrea
 void launch_export_place(const VoxelTable& vt, const int32_t* parent, int nid, const ExportScratch& es,
                          cudaStream_t st);
 
+// the instance table into pinned memory (k_export.cu)
+void launch_stage_table(const Instances& inst, const int* next_id, int D, const TableStage& ts, cudaStream_t st);
+
 // maintenance and queries
 void launch_rehash(const VoxelTable& from, const VoxelTable& to, int* err, cudaStream_t st);
 void launch_query_topk(const float* q, int nq, int D, const Instances& inst, int nid, float* scores, int k,

@@ -81,3 +81,49 @@ def test_topk_at_tile_edges(nid, nq, k, dim):
     best = -np.sort(-want, axis=1)[:, :m]
     assert np.abs(best - sc[:, :m]).max() <= 3 * dim * 2.0 ** -24 + 2.0 ** -22
     gmap.close()
+
+
+@pytest.mark.parametrize("dim,per", [(7, 3), (64, 96), (4096, 90)])
+def test_instance_table_read_again_and_again(dim, per):
+    """The first read of a map's table, later ones through pinned memory and tables too large for it are the same
+    bytes; short buffers are refused and NULL arrays left out by all of them."""
+    import torch
+    from paper_2603_03935_gb300 import DiscMap, binding, device_frame
+    dev = torch.device("cuda:0")
+    lib = binding.lib()
+    gen = torch.Generator(device=dev).manual_seed(dim)
+    cfg = dict(voxel_size=0.025, embed_dim=dim, patch_h=8, patch_w=12, max_width=96, max_height=64, max_masks=96,
+               min_mask_pixels=1, voxel_capacity=1 << 16, max_load=0.5, instance_capacity=64)
+    again, empty = DiscMap(**cfg), DiscMap(**cfg)
+    for _ in range(3):
+        assert lib.disc_map_export_instances(empty._h, None, None, None, None, None, 0) == 0
+    v, u = torch.arange(64, device=dev)[:, None] // 8, torch.arange(96, device=dev)[None, :] // 8
+    labels = (v * 12 + u + 1).clamp(max=97)
+    labels = torch.where(labels <= per, labels, torch.zeros_like(labels)).to(torch.int16).contiguous()
+    frames = []
+    for t in range(4):  # 4 x 90 rows of 4096 floats: 5.9 MB, above the pinned buffer's bound
+        pose = np.eye(4)
+        pose[0, 3] = 40.0 * t
+        tokens = torch.randn(96, dim, device=dev, generator=gen)
+        frames.append(device_frame(torch.full((64, 96), 2.0, device=dev), labels, tokens, pose,
+                                   (80.0, 80.0, 48.0, 32.0), per))
+        again.integrate(frames[-1])
+        once = DiscMap(**cfg)
+        for f in frames:
+            once.integrate(f)
+        want = once.instances()
+        n = len(want["parent"])
+        assert n == per * (t + 1)
+        for _ in range(2):
+            got = again.instances()
+            assert sorted(got) == sorted(want)
+            for k in want:
+                assert np.array_equal(np.asarray(got[k]).view(np.uint8), np.asarray(want[k]).view(np.uint8)), (k, t)
+        count = np.full(n, -1, np.int64)
+        assert lib.disc_map_export_instances(again._h, None, count.ctypes.data, None, None, None, n - 1) == -1
+        assert (count == -1).all()
+        assert lib.disc_map_export_instances(again._h, None, count.ctypes.data, None, None, None, n + 7) == 0
+        assert np.array_equal(count, want["count"])
+        once.close()
+    again.close()
+    empty.close()
