@@ -2696,12 +2696,14 @@ disc_status disc_map_export_assoc(disc_map* m, float* A, int32_t cap)
 
 // The instance table through pinned memory that a kernel fills over the link,
 // with one launch and one wait: the read of the row count and five copies into
-// pageable memory waited six times, a third of a small frame's integration and
-// read-back (168 us, now 135; a 640x480 frame with 40 masks 226, now 221).
-// The pinned buffer is made at a map's second read: a map that is read once
-// would pay more for it than it saves.  Tables above kStageBytes, where the
-// copies themselves take the time, keep them.  *done: the call is answered.
-constexpr size_t kStageBytes = 4 << 20;
+// pageable memory waited six times (60 us for 8 rows, now 13).  Embeddings of
+// up to kStageE bytes come the same way; larger ones take one copy straight
+// into the caller's memory, which the device writes at 200 GB/s where the
+// host's copy out of the pinned buffer runs at 13 (2 MB: 152 us staged, 72 by
+// the six copies, 37 so; at 256 KB both ways take 27).  The pinned buffer, of
+// at most kStageBytes, is made at a map's second read: a map that is read once
+// would pay more for it than it saves.  *done: the call is answered.
+constexpr size_t kStageBytes = 2 << 20, kStageE = 256 << 10;
 
 static disc_status export_staged(disc_map* m, int32_t* parent, int64_t* count, float* Q, float* E, int32_t* n_obs,
                                  int32_t cap, bool* done)
@@ -2712,7 +2714,9 @@ static disc_status export_staged(disc_map* m, int32_t* parent, int64_t* count, f
     const int64_t rows = std::min<int64_t>(std::max<int64_t>(m->next_id_upper, 0), m->inst.cap);
     TableStage ts{};
     const size_t b_row4 = align256(4 * (size_t)rows), b_row8 = align256(8 * (size_t)rows);
-    const size_t need = 256 + b_row8 + 3 * b_row4 + (E ? align256(4 * (size_t)rows * m->D) : 0);
+    const size_t b_E = align256(4 * (size_t)rows * m->D);
+    const bool with_E = E && b_E <= kStageE;
+    const size_t need = 256 + b_row8 + 3 * b_row4 + (with_E ? b_E : 0);
     if (first || need > kStageBytes) return DISC_OK;
     if (need > m->stage_cap) {
         if (m->stage) cudaFreeHost(m->stage);
@@ -2732,7 +2736,7 @@ static disc_status export_staged(disc_map* m, int32_t* parent, int64_t* count, f
     ts.parent = (int*)(p + 256 + b_row8);
     ts.Q = (float*)(p + 256 + b_row8 + b_row4);
     ts.n_obs = (int*)(p + 256 + b_row8 + 2 * b_row4);
-    ts.E = E ? (float*)(p + 256 + b_row8 + 3 * b_row4) : nullptr;
+    ts.E = with_E ? (float*)(p + 256 + b_row8 + 3 * b_row4) : nullptr;
     launch_stage_table(m->inst, m->d_next_id, m->D, ts, m->stream);
     CK(cudaGetLastError());
     CK(cudaStreamSynchronize(m->stream));
@@ -2744,7 +2748,8 @@ static disc_status export_staged(disc_map* m, int32_t* parent, int64_t* count, f
     if (parent) std::memcpy(parent, ts.parent, sizeof(int32_t) * n);
     if (count) std::memcpy(count, ts.count, sizeof(int64_t) * n);
     if (Q) std::memcpy(Q, ts.Q, sizeof(float) * n);
-    if (E) std::memcpy(E, ts.E, sizeof(float) * (size_t)n * m->D);
+    if (E && with_E) std::memcpy(E, ts.E, sizeof(float) * (size_t)n * m->D);
+    else if (E) CK(cudaMemcpy(E, m->inst.E, sizeof(float) * (size_t)n * m->D, cudaMemcpyDeviceToHost));
     if (n_obs) std::memcpy(n_obs, ts.n_obs, sizeof(int32_t) * n);
     return DISC_OK;
 }
