@@ -32,15 +32,16 @@ constexpr int SER_THREADS = 1024;
 constexpr int OV_SLOTS = 2 * SER_THREADS;
 constexpr int OV_PROBES = 64;  // longest probe of the shared pair hash
 
-// label of a key in the voxel table, -1 if absent
-__device__ __forceinline__ int vt_label(const VoxelTable& vt, unsigned long long key)
+// label of a key in the voxel table, -1 if absent, from the n-th place h of
+// its probe sequence on
+__device__ __noinline__ int far_label(const VoxelTable& vt, unsigned long long key, unsigned long long h,
+                                      unsigned long long n)
 {
-    unsigned long long h = vt_home(key, vt.mask);
-    for (unsigned long long pr = 0; pr <= vt.mask; pr++) {
+    for (; n <= vt.mask; n++) {
         const unsigned long long kk = vt.keys[h];
         if (kk == key) return vt.labels[h];
         if (kk == EMPTY_KEY) return -1;
-        h = vt_next(h, pr + 1, vt.mask);
+        h = vt_next(h, n + 1, vt.mask);
     }
     return -1;
 }
@@ -69,60 +70,125 @@ __device__ void add_pair(const Scratch& sc, const SerialScratch& ss, unsigned lo
     atomicAdd(&ss.ocnt[t], cnt);
 }
 
+// key of a voxel from its biased coordinates
+__device__ __forceinline__ unsigned long long key_at(int x, int y, int z)
+{
+    return ((unsigned long long)(unsigned)x << (2 * KEY_BITS)) | ((unsigned long long)(unsigned)y << KEY_BITS) |
+           (unsigned long long)(unsigned)z;
+}
+
+// label l's root among the nr distinct roots; returns how many there are now.
+// (The rare steps of the neighbourhood are calls: inlined at each place they
+// made the loop too long for the instruction cache.)
+__device__ __noinline__ int add_root(const int32_t* parent, int l, int roots[27], int nr)
+{
+    const int root = parent[l];
+    for (int t = 0; t < nr; t++)
+        if (roots[t] == root) return nr;
+    roots[nr] = root;
+    return nr + 1;
+}
+
 // Neighbourhood overlap (overlap_dilation): segment voxel `key` (label lab,
 // -1 if absent) overlaps each distinct instance labelling it or one of its 26
-// neighbours, once: their roots into roots[27], returns how many.  Nine
-// neighbours at a time (one x offset), whose table slots, labels and parents
-// are each loaded together; they lie in four blocks of the table, hashed once
-// each.  Only a collision walks on.
-__device__ __forceinline__ int dilated_roots(const VoxelTable& vt, const Instances& inst, unsigned long long key,
+// neighbours, once: their roots into roots[27], returns how many.  The nine
+// neighbours of one x offset lie in four blocks of the table, and a block's
+// four voxels of one x in four consecutive slots (vt_place: x is the highest
+// of the place's three bits, which the block's hash permutes by an exclusive
+// or): one 32-byte load of keys and one 16-byte load of labels per block, two
+// blocks at a time.  Slots are compared as they lie (the exclusive or goes
+// into the expected key), and only a label other than the last three met
+// is looked up.  A place that another block's voxel holds is walked past at the
+// end, all lanes of a warp together.
+// Bound by latency and issue.  Room frames (134,000 segment voxels, the table
+// a quarter full): k_overlap 46.5 us per frame with a load of eight bytes, a
+// label and a parent per neighbour, 37.6 so (14.4 without the neighbours; 7 of
+// the rest for places held by other voxels, 5 for labels looked up).  All four
+// blocks' loads at once, with every step inlined, took 78.
+__device__ __forceinline__ int dilated_roots(const VoxelTable& vt, const int32_t* parent, unsigned long long key,
                                              int lab, int roots[27])
 {
-    int nr = 0;
-    if (lab >= 0) roots[nr++] = inst.parent[lab];
-    int k[3];
-    unpack_key(key, k);
+    constexpr int FIELD = (1 << KEY_BITS) - 1;
+    int nr = 0, c0 = lab, c1 = lab, c2 = lab;  // labels met last
+    if (lab >= 0) roots[nr++] = parent[lab];
+    const int xc = (int)(key >> (2 * KEY_BITS)) & FIELD, yc = (int)(key >> KEY_BITS) & FIELD, zc = (int)key & FIELD;
+    if (vt.mask < 7) {  // a table of less than a block
 #pragma unroll 1
-    for (int dx = -1; dx <= 1; dx++) {
-        const int x = k[0] + dx;
-        if (x < -KEY_BIAS || x > KEY_BIAS - 1) continue;
-        unsigned long long nk[9], h[9], cur[9], block[4];
-        int nl[9];
-        // blocks of the lower and upper y and z neighbours
-        const unsigned long long bx = (unsigned long long)((x + KEY_BIAS) & ~1) << (2 * KEY_BITS);
-        const int y0 = (k[1] - 1 + KEY_BIAS) >> 1, z0 = (k[2] - 1 + KEY_BIAS) >> 1;
+        for (int n = 0; n < 27; n++) {
+            const int x = xc + n / 9 - 1, y = yc + n / 3 % 3 - 1, z = zc + n % 3 - 1;
+            if (((x | y | z) & ~FIELD) != 0) continue;
+            const unsigned long long nk = key_at(x, y, z);
+            const int l = far_label(vt, nk, vt_home(nk, vt.mask), 0);
+            if (l >= 0) nr = add_root(parent, l, roots, nr);
+        }
+        return nr;
+    }
+    // the lower blocks, and which of a block's two y (z) are one of the three:
+    // bits for the lower block, then for the upper one
+    const int y0 = (yc - 1) >> 1, z0 = (zc - 1) >> 1;
+    const unsigned my = (yc == 0 ? 0u : (yc & 1) ? 3u : 2u) | (yc == FIELD ? 0u : (yc & 1) ? 1u : 3u) << 2;
+    const unsigned mz = (zc == 0 ? 0u : (zc & 1) ? 3u : 2u) | (zc == FIELD ? 0u : (zc & 1) ? 1u : 3u) << 2;
+    unsigned long long walk = 0;  // places held by another voxel: 16 (x offset) + 4 (block) + slot
+#pragma unroll 1
+    for (int n = 0; n < 6; n++) {
+        const int x = xc + (n >> 1) - 1, by = y0 + (n & 1);
+        const unsigned ym = my >> 2 * (n & 1);
+        if ((x & ~FIELD) != 0 || (ym & 3) == 0) continue;
+        unsigned long long kk[2][4], expect[2];
+        int4 l4[2];
+        unsigned want[2];
 #pragma unroll
-        for (int q = 0; q < 4; q++)
-            block[q] = mix64(bx | ((unsigned long long)(unsigned)(2 * (y0 + (q >> 1))) << KEY_BITS) |
-                             (unsigned long long)(unsigned)(2 * (z0 + (q & 1))));
-#pragma unroll
-        for (int j = 0; j < 9; j++) {
-            const int y = k[1] + j / 3 - 1, z = k[2] + j % 3 - 1;
-            const bool in = !(dx == 0 && j == 4) && y >= -KEY_BIAS && y <= KEY_BIAS - 1 && z >= -KEY_BIAS &&
-                            z <= KEY_BIAS - 1;
-            nk[j] = ((unsigned long long)(x + KEY_BIAS) << (2 * KEY_BITS)) |
-                    ((unsigned long long)(y + KEY_BIAS) << KEY_BITS) | (unsigned long long)(z + KEY_BIAS);
-            const bool uy = ((y + KEY_BIAS) >> 1) != y0, uz = ((z + KEY_BIAS) >> 1) != z0;
-            const unsigned long long b = uy ? (uz ? block[3] : block[2]) : (uz ? block[1] : block[0]);
-            h[j] = vt_place(b, nk[j], vt.mask);
-            cur[j] = in ? vt.keys[h[j]] : EMPTY_KEY;
+        for (int q = 0; q < 2; q++) {
+            const unsigned long long h = mix64(key_at(x & ~1, 2 * by, 2 * (z0 + q)));
+            const unsigned p = (unsigned)(h >> 61);
+            const unsigned long long at = ((h << 3) | (((x & 1) << 2) ^ (p & 4))) & vt.mask;
+            asm("ld.global.v4.b64 {%0, %1, %2, %3}, [%4];"
+                : "=l"(kk[q][0]), "=l"(kk[q][1]), "=l"(kk[q][2]), "=l"(kk[q][3])
+                : "l"(vt.keys + at));
+            l4[q] = *(const int4*)(vt.labels + at);
+            expect[q] = key_at(x, 2 * by, 2 * (z0 + q)) ^ ((unsigned long long)((p >> 1) & 1) << KEY_BITS | (p & 1));
+            const unsigned zm = mz >> (2 * q) & 3;
+            unsigned w = ((ym & 1) ? zm : 0) | ((ym & 2) ? zm << 2 : 0);
+            if (p & 1) w = (w & 5) << 1 | (w >> 1 & 5);
+            if (p & 2) w = (w & 3) << 2 | w >> 2;
+            want[q] = w;  // bit s: slot s is a neighbour's place
         }
 #pragma unroll
-        for (int j = 0; j < 9; j++) {
-            nl[j] = -1;
-            if (cur[j] == EMPTY_KEY) continue;
-            nl[j] = cur[j] == nk[j] ? vt.labels[h[j]] : vt_label(vt, nk[j]);
-        }
+        for (int q = 0; q < 2; q++) {
+            const int l[4] = {l4[q].x, l4[q].y, l4[q].z, l4[q].w};
+            unsigned far = 0;
+            unsigned other = 0;
 #pragma unroll
-        for (int j = 0; j < 9; j++)
-            if (nl[j] >= 0) nl[j] = inst.parent[nl[j]];
-#pragma unroll
-        for (int j = 0; j < 9; j++) {
-            if (nl[j] < 0 || (j > 0 && nl[j] == nl[j - 1])) continue;  // (neighbours mostly share their root)
-            bool seen = false;
-            for (int t = 0; t < nr; t++) seen |= roots[t] == nl[j];
-            if (!seen) roots[nr++] = nl[j];
+            for (int s = 0; s < 4; s++) {
+                const int hi = (int)(kk[q][s] >> 32);  // (negative only in an empty slot)
+                const bool hit = hi == (int)(expect[q] >> 32) &&
+                                 (unsigned)kk[q][s] == ((unsigned)expect[q] ^ ((unsigned)(s >> 1) << KEY_BITS | (s & 1)));
+                if (!hit && hi >= 0) far |= 1u << s;
+                if (hit && l[s] != c0 && l[s] != c1 && l[s] != c2) other |= 1u << s;
+            }
+            far &= want[q];
+            other &= want[q];
+            walk |= (unsigned long long)far << (16 * (n >> 1) + 8 * (n & 1) + 4 * q);
+            while (other) {
+                const int s = __ffs(other) - 1, x = s < 2 ? (s ? l[1] : l[0]) : s == 2 ? l[2] : l[3];
+                other &= other - 1;
+                if (x < 0 || x == c0) continue;
+                c2 = c1;
+                c1 = c0;
+                c0 = x;
+                nr = add_root(parent, x, roots, nr);
+            }
         }
+    }
+    while (walk) {
+        const int n = __ffsll((long long)walk) - 1;
+        walk &= walk - 1;
+        const int x = xc + (n >> 4) - 1, by = y0 + (n >> 3 & 1), bz = z0 + (n >> 2 & 1);
+        const unsigned long long h = mix64(key_at(x & ~1, 2 * by, 2 * bz));
+        const unsigned at = (n & 3) ^ ((unsigned)(h >> 61) & 3);
+        const unsigned long long nk = key_at(x, 2 * by + (int)(at >> 1), 2 * bz + (int)(at & 1));
+        const int l = far_label(vt, nk, vt_next(vt_place(h, nk, vt.mask), 1, vt.mask), 1);
+        if (l >= 0) nr = add_root(parent, l, roots, nr);
     }
     return nr;
 }
@@ -162,11 +228,11 @@ __device__ void phase_overlap(const Scratch& sc, const SerialScratch& ss, const 
             // an entry adds one pair, or up to 27 (then a pair that finds no
             // place in the shared hash goes straight to the frame's)
             int roots[27];
-            const int nr = dilate ? dilated_roots(vt, inst, key, lab, roots)
+            const int nr = dilate ? dilated_roots(vt, inst.parent, key, lab, roots)
                                   : lab >= 0 ? (roots[0] = inst.parent[lab], 1) : 0;
             for (int r = 0; r < nr; r++) {
                 const unsigned long long okey = ((unsigned long long)m << 32) | (unsigned)roots[r];
-                unsigned t = (unsigned)(mix64(okey) & (OV_SLOTS - 1));
+                unsigned t = ((unsigned)roots[r] * 0x9E3779B1u + (unsigned)m * 0x85EBCA77u) / (unsigned)(0x100000000ull / OV_SLOTS);
                 int pr = 0;
                 for (; pr < OV_PROBES; pr++) {
                     const unsigned long long prev = atomicCAS(&pkey[t], EMPTY_KEY, okey);
