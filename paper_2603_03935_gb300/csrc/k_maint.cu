@@ -32,16 +32,20 @@ __global__ void k_rehash(VoxelTable from, VoxelTable to, int* err)
 // each of its warps four instances, whose rows it reads once for all of them;
 // the norms are taken beside.  Every sum keeps its order (a lane its dimensions
 // in turn, then the lanes by halves), so scores do not depend on the tiling.
-// Bound by the shared-memory reads of the queries.  4000 instances x 64
-// queries of 768: 122 us with a warp per (query, instance), which read both
-// rows and took both norms each time; 45 us so.
-constexpr int QUERY_TILE = 8, QUERY_DIM = 1024, QUERY_INST = 4, QUERY_WARPS = 8;
+// Bound by instruction issue, and by the latency of the rows' loads (24 steps
+// of a lane at dimension 768): each row's next two values are on their way
+// while one is used, and four queries' values lie side by side for one 16-byte
+// read.  4000 instances x 64 queries of 768: 122 us with a warp per (query,
+// instance), which read both rows and took both norms each time; 45 us with
+// the tile, 33 with the loads ahead (three or four ahead, in more registers,
+// 44).
+constexpr int QUERY_TILE = 8, QUERY_DIM = 1024, QUERY_INST = 4, QUERY_WARPS = 8, QUERY_AHEAD = 2;
 static_assert(QUERY_TILE * QUERY_INST == 32 && QUERY_WARPS == QUERY_TILE, "a lane per product, a warp per query's norm");
 
 __global__ void __launch_bounds__(32 * QUERY_WARPS) k_query_scores(const float* q, int nq, int D, Instances inst,
                                                                    int nid, float* scores)
 {
-    __shared__ float qs[QUERY_TILE][QUERY_DIM];
+    __shared__ float4 qs[QUERY_TILE / 4][QUERY_DIM];  // four queries side by side
     __shared__ float s_na[QUERY_TILE];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int q0 = blockIdx.y * QUERY_TILE;
@@ -58,23 +62,45 @@ __global__ void __launch_bounds__(32 * QUERY_WARPS) k_query_scores(const float* 
     for (int c0 = 0; c0 < D; c0 += QUERY_DIM) {
         const int cn = min(QUERY_DIM, D - c0);
         __syncthreads();
-        for (int t = 0; t < QUERY_TILE; t++)
-            for (int d = threadIdx.x; d < cn; d += 32 * QUERY_WARPS)
-                qs[t][d] = q0 + t < nq ? q[(size_t)(q0 + t) * D + c0 + d] : 0.0f;
+        {  // a warp per query: its norm on the way
+            const float* src = q + (size_t)min(q0 + warp, nq - 1) * D + c0;
+#pragma unroll 8
+            for (int d = lane; d < cn; d += 32) {
+                const float a = src[d];
+                ((float*)&qs[warp / 4][d])[warp % 4] = a;
+                na += a * a;
+            }
+        }
+        float ahead[QUERY_INST][QUERY_AHEAD];  // the rows' next values, on their way
+#pragma unroll
+        for (int k = 0; k < QUERY_AHEAD; k++)
+#pragma unroll
+            for (int u = 0; u < QUERY_INST; u++)
+                ahead[u][k] = lane + 32 * k < cn ? row[u][c0 + lane + 32 * k] : 0.0f;
         __syncthreads();
-        for (int d = lane; d < cn; d += 32) na += qs[warp][d] * qs[warp][d];
-#pragma unroll 2
+#pragma unroll QUERY_AHEAD
         for (int d = lane; d < cn; d += 32) {
             float b[QUERY_INST];
 #pragma unroll
-            for (int u = 0; u < QUERY_INST; u++) b[u] = row[u][c0 + d];
+            for (int u = 0; u < QUERY_INST; u++) {
+                b[u] = ahead[u][0];
+#pragma unroll
+                for (int k = 0; k + 1 < QUERY_AHEAD; k++) ahead[u][k] = ahead[u][k + 1];
+                const int dn = d + 32 * QUERY_AHEAD;
+                ahead[u][QUERY_AHEAD - 1] = dn < cn ? row[u][c0 + dn] : 0.0f;
+            }
 #pragma unroll
             for (int u = 0; u < QUERY_INST; u++) nb[u] += b[u] * b[u];
 #pragma unroll
-            for (int t = 0; t < QUERY_TILE; t++) {
-                const float a = qs[t][d];
+            for (int h = 0; h < QUERY_TILE / 4; h++) {
+                const float4 a = qs[h][d];
 #pragma unroll
-                for (int u = 0; u < QUERY_INST; u++) dt[u * QUERY_TILE + t] += a * b[u];
+                for (int u = 0; u < QUERY_INST; u++) {
+                    dt[u * QUERY_TILE + 4 * h] += a.x * b[u];
+                    dt[u * QUERY_TILE + 4 * h + 1] += a.y * b[u];
+                    dt[u * QUERY_TILE + 4 * h + 2] += a.z * b[u];
+                    dt[u * QUERY_TILE + 4 * h + 3] += a.w * b[u];
+                }
             }
         }
     }
