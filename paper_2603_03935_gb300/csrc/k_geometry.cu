@@ -85,19 +85,26 @@ __global__ void k_slot_reset(BatchScratch bs, int B)
 // so neighbours' points (for the pixel normal) are read, not recomputed.
 // Each valid pixel becomes a record (its (mask, voxel) key and exact normal)
 // of the partition its key hashes to: one counter increment and one 32-byte
-// store, no probing and nothing that the frame's next use has to clear.  In
-// a tile whose neighbouring pixels mostly share voxels (near surfaces, coarse
-// voxels: fewer runs of equal keys along the rows than half the valid pixels)
-// the pixels first meet in a shared hash that sums their normals, and only
-// the tile's distinct keys become records, so many pixels of one voxel do not
-// pile up in one partition.
-// Bound by instruction issue (58 % active) and by the scattered record stores
+// store, no probing and nothing that the frame's next use has to clear.
+// Unless nearly every pixel of the tile starts a run of equal keys along its
+// row (more than 7/8 of the valid ones: far surfaces, fine voxels), the pixels
+// first meet in a shared hash that sums their normals, and only the tile's
+// distinct keys become records.  Depth noise breaks the runs of pixels whose
+// voxels repeat all over the tile, and a voxel's records pile up in one
+// partition, where k_entries sums them one after the other: Room frames with
+// 1 % noise had 231,000 records of 72,000 voxels, up to 86 of one, with the
+// line at half the valid pixels.  Back-projection and entries, us per frame,
+// with the line at 1/2 | 3/4 | 7/8 | 15/16 | every tile merged: those frames
+// 17.1 | 12.3 | 11.7 | 12.0 | 12.4; the same room drifting 14.2 | 13.4 | 12.7 |
+// 13.3 | 14.0; a building of 5 cm voxels 11.9 | 10.3 | 9.9 | 10.0 | 10.0; 16
+// uneven maps 9.4 | 9.1 | 8.8 | 9.1 | 9.3.
+// Bound by instruction issue (60 % active) and by the scattered record stores
 // and counter increments, one line per lane (L1 70 % busy).  Measured on Room
 // frames (640x480, 2.5 cm voxels, 8 frames per launch) in place of one global
 // (segment, voxel) hash per frame with 32-byte slots, whose probes and three
-// 64-bit atomics per key missed L2: 18.1 -> 6.9 us per frame, and 2.6 -> 0.3 us
-// for clearing the slot; with k_entries (4.5 -> 7.3 us, they now also sum the
-// pixels) 25.2 -> 14.5 us.  The partition counters lie a cache line apart: side
+// 64-bit atomics per key missed L2: 18.1 -> 7.2 us per frame, and 2.6 -> 0.3 us
+// for clearing the slot; with k_entries (4.5 -> 5.6 us, they now also sum the
+// pixels) 25.2 -> 13.1 us.  The partition counters lie a cache line apart: side
 // by side (8 to a sector) the kernel took 28.8 us.
 constexpr int BP_TX = 32, BP_TY = 16, BP_PER = 2;      // tile; pixels per thread (rows 2 ty and 2 ty + 1)
 constexpr int BP_ROWS = BP_TY / BP_PER, BP_THREADS = BP_TX * BP_ROWS;
@@ -268,7 +275,7 @@ __global__ void __launch_bounds__(BP_THREADS) k_backproject(const FrameParams* f
         if (same && (lane & 1)) hk[j] = 0ull;
     }
     const int parts = seg_parts((long long)W * H);
-    if (2 * s_runs > s_valid || s_valid == 0) {  // uniform per block
+    if (8 * s_runs > 7 * s_valid || s_valid == 0) {  // uniform per block
 #pragma unroll
         for (int j = 0; j < BP_PER; j++)
             if (hk[j]) seg_append(sc, parts, hk[j], nfix[j][0], nfix[j][1], nfix[j][2]);
