@@ -447,10 +447,10 @@ disc_status disc_debug_gemm_stall(int32_t device, int32_t on);
 /* ---- Launch schedule and autotuner -----------------------------------------
  * How a map's (or a group's) batches are cut into launches: the frames per
  * launch of the geometry kernels (back-projection, entries, DBSCAN), whose
- * per-frame hashes should stay in L2; the CTA counts of the four serial
+ * per-frame records should stay in L2; the CTA counts of the four serial
  * kernels per frame of maps with the neighbourhood overlap; how many lanes
  * look one voxel up in the table together (warp-cooperative probing: each
- * round a group of probe_width lanes reads that many consecutive slots of the
+ * round a group of probe_width lanes reads that many consecutive places of the
  * probe sequence); and into how many smaller batches a call whose frames fit
  * one batch is cut, so that each smaller batch's stateless kernels run beside
  * the frame chain of the one before it.  None changes any result. */
