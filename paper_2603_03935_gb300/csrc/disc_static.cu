@@ -58,11 +58,12 @@ __global__ void k_static_begin(unsigned char* base, FrameParams fp)
     if (blockIdx.x == 0 && threadIdx.x == 0) *(FrameParams*)(base + OFF_PARAMS) = fp;
 }
 
-// heat_p = D_p * cos(f_p, q), one fp32 rounding
-__global__ void k_heat(float* heat, const float* cosq, int P)
+// heat_p = D_p * cos(f_p, q), one fp32 rounding; a refused call's heat stays
+// as it was (its D_p and cosines were not written)
+__global__ void k_heat(float* heat, const float* cosq, int P, const FrameCounters* ctr)
 {
     const int p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p < P) heat[p] = __fmul_rn(heat[p], cosq[p]);
+    if (p < P && ctr->err == 0) heat[p] = __fmul_rn(heat[p], cosq[p]);
 }
 
 // Eq. 1 and the token cosines on the static working set; without cosg the
@@ -122,7 +123,7 @@ static disc_status static_stats(const void* tokens, int32_t token_dtype, int32_t
     k_static_begin<<<4, 256, 0, st>>>(base, fp);
     const bool bf16 = token_dtype == DISC_TOKENS_BF16;
     launch_token_stats(dfp, bs, 1, P, D, bf16, !bf16, st);
-    if (!cosg) k_heat<<<(P + 255) / 256, 256, 0, st>>>(Dp, sc.cosg, P);
+    if (!cosg) k_heat<<<(P + 255) / 256, 256, 0, st>>>(Dp, sc.cosg, P, sc.ctr);
     if (cudaGetLastError() != cudaSuccess) return DISC_ERR_CUDA;
     int err = 0;
     if (cudaMemcpyAsync(&err, &sc.ctr->err, sizeof(int), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
