@@ -531,7 +531,8 @@ __global__ void __launch_bounds__(SEG_THREADS) k_entries(const FrameParams* fps,
 
 // ---- Eq. 2-3: S_angle = mean of the voxel terms; Q per segment -------------------
 // Runs after both the token and the geometry kernels: a frame that either
-// failed takes its error here, and its geometry counters read zero.
+// failed takes its error here, and its geometry counters, voxel counts and
+// S_angle read zero.
 __global__ void k_quality(const FrameParams* fps, BatchScratch bs)
 {
     const FrameParams& fp = fps[blockIdx.x];
@@ -543,6 +544,10 @@ __global__ void k_quality(const FrameParams* fps, BatchScratch bs)
             FrameCounters* c = sc.ctr;
             c->err = err;
             c->n_entries = c->valid_pixels = c->dropped_pixels = c->max_probe = c->denoised = 0;
+        }
+        for (int m = threadIdx.x; m < fp.M; m += blockDim.x) {
+            sc.nvox[m] = 0;
+            sc.S[5 * m + 1] = sc.S[5 * m + 4] = 0.0f;
         }
         return;
     }

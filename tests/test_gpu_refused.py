@@ -19,3 +19,28 @@ def test_a_refused_heatmap_leaves_its_output_as_it_was(where):
                                           torch.cuda.current_stream().cuda_stream)
     assert binding.STATUS[rc] == "DISC_ERR_RANGE"
     assert torch.equal(heat, before)
+
+
+@pytest.mark.parametrize("dilation", [0, 1])
+def test_a_failed_frames_report_holds_no_voxels(dilation):
+    import synth
+    import torch
+    from paper_2603_03935_gb300 import DiscMap, device_frame
+    from tests import common
+    dev = torch.device("cuda:0")
+    sc = synth.tiny_scene(num_frames=2)
+    fr = sc.render(range(2))
+    gmap = DiscMap(**common.disc_cfg(sc, overlap_dilation=dilation))
+    fr.tokens[1][3, 5] = 2000.0  # out of the accepted range: the second frame fails
+    for i in range(2):
+        frame = device_frame(torch.from_numpy(fr.depth[i]).to(dev), torch.from_numpy(fr.labels[i].view("int16")).to(dev),
+                             torch.from_numpy(fr.tokens[i]).to(dev), fr.poses[i], (sc.fx, sc.fy, sc.cx, sc.cy),
+                             int(fr.num_masks[i]))
+        stats, done, rc = gmap.integrate_frames([frame], check=False)
+        rep = gmap.last_frame()
+        if i == 0:
+            assert rc == 0 and done == 1 and rep["nvox"].sum() > 0 and (rep["S"][:, 1] > 0).any()
+    assert rc != 0 and done == 0
+    assert all(stats[0][k] == 0 for k in ("valid_pixels", "unique_seg_voxels", "new_voxels", "live_segments"))
+    assert (rep["nvox"] == 0).all() and (rep["S"][:, [1, 4]] == 0).all() and (rep["rep"] == -1).all()
+    gmap.close()
