@@ -372,10 +372,16 @@ __global__ void k_weights(const FrameParams* fps, BatchScratch bs)
 {
     __shared__ long long red_ll[32];
     __shared__ float red_f[32];
+    __shared__ int s_err;
     const FrameParams& fp = fps[blockIdx.z];
     const Scratch sc = bs.frame(blockIdx.z);
     const int m = blockIdx.x;
-    if (m >= fp.M || sc.ctr->err) return;
+    if (m >= fp.M) return;  // uniform per block
+    // read once for the block: the other grid's token kernels, which share the
+    // frame's counters, may set it meanwhile
+    if (threadIdx.x == 0) s_err = *(volatile int32_t*)&sc.ctr->err;
+    __syncthreads();
+    if (s_err) return;
     const int npix = sc.npix[m];
     float* w = sc.W + (size_t)m * fp.Kpad;
     float* S = sc.S + 5 * m;

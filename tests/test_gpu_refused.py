@@ -44,3 +44,41 @@ def test_a_failed_frames_report_holds_no_voxels(dilation):
     assert all(stats[0][k] == 0 for k in ("valid_pixels", "unique_seg_voxels", "new_voxels", "live_segments"))
     assert (rep["nvox"] == 0).all() and (rep["S"][:, [1, 4]] == 0).all() and (rep["rep"] == -1).all()
     gmap.close()
+
+
+@pytest.mark.parametrize("bad_grid", ["second", "first", "both"])
+def test_a_token_out_of_range_in_either_grid_fails_its_frame_alone(bad_grid):
+    # the grids' kernels run side by side and share the frame's error word
+    import numpy as np
+    import oracle
+    import synth
+    import torch
+    from paper_2603_03935_gb300 import DiscMap, device_frame
+    from tests import common
+    dev = torch.device("cuda:0")
+    sc = synth.tiny_scene(num_frames=12)
+    fr = sc.render(range(12))
+    at = fr.assoc_tokens(5, 7, 96)
+    cfg = common.disc_cfg(sc, assoc_dim=96, assoc_patch_h=5, assoc_patch_w=7)
+    gmap, omap = DiscMap(**cfg), oracle.OracleMap(**common.to_oracle_cfg(cfg))
+
+    def frame(i, bad):
+        first, second = fr.tokens[i].copy(), at[i].copy()
+        if bad:
+            for g, t in (("first", first), ("second", second)):
+                if bad_grid in (g, "both"):
+                    t.reshape(-1)[i * 7 % t.size] = 1500.0
+        return device_frame(torch.from_numpy(fr.depth[i]).to(dev), torch.from_numpy(fr.labels[i].view(np.int16)).to(dev),
+                            torch.from_numpy(first).to(dev), fr.poses[i], (sc.fx, sc.fy, sc.cx, sc.cy),
+                            int(fr.num_masks[i]), assoc_tokens=torch.from_numpy(second).to(dev))
+
+    for i in range(0, 12, 4):
+        # the call stops at its third frame; the rest is given again without the bad token
+        stats, done, rc = gmap.integrate_frames([frame(i + j, j == 2) for j in range(4)], check=False)
+        assert rc != 0 and done == 2 and stats[2]["status"] == rc and stats[2]["new_voxels"] == 0
+        _, done, rc = gmap.integrate_frames([frame(i + j, False) for j in (2, 3)])
+        assert rc == 0 and done == 2
+        for j in range(4):
+            omap.integrate(*oracle.frame_args(fr, i + j), assoc_tokens=at[i + j])
+    common.compare_maps(gmap, omap, ctx=f"{bad_grid} grid out of range")
+    gmap.close()
