@@ -1039,7 +1039,7 @@ int enqueue_stateless(Runner& r, int k, int S, int combos, cudaStream_t st, int 
     if (geo) after(st, sg, r.ev_cover);
     run_phase(r, PH_WEIGHTS, st, [&] { return launch_weights(dfp, bs, S, Mmax, st); });
     run_phase(r, PH_POOL_EXACT, st, [&] { return launch_pool_exact(dfp, bs, S, P, D, Mmax, any_bf16, any_f32, st); });
-    run_phase(r, PH_POOL_GEMM, st, [&] { return launch_pool_gemm(dfp, bs, S, P, D, Mmax, any, st); });
+    run_phase(r, PH_POOL_GEMM, st, [&] { return launch_pool_gemm(dfp, bs, S, P, D, Mmax, any, !r.green[0], st); });
     if (grid2) {
         // the association features: the same kernels on the second grid's
         // view (pixel-mean weights; frames of maps without it are inert)
@@ -1052,7 +1052,7 @@ int enqueue_stateless(Runner& r, int k, int S, int combos, cudaStream_t st, int 
         run_phase(r, PH_WEIGHTS, sv, [&] { return launch_weights(dfa, va, S, Mmax, sv); });
         run_phase(r, PH_POOL_EXACT, sv,
                   [&] { return launch_pool_exact(dfa, va, S, r.Pa, r.Da, Mmax, any_bf16, any_f32, sv); });
-        run_phase(r, PH_POOL_GEMM, sv, [&] { return launch_pool_gemm(dfa, va, S, r.Pa, r.Da, Mmax, any, sv); });
+        run_phase(r, PH_POOL_GEMM, sv, [&] { return launch_pool_gemm(dfa, va, S, r.Pa, r.Da, Mmax, any, !r.green[0], sv); });
     }
     if (geo) {
         for (int f0 = 0; f0 < S; f0 += r.geo_chunk) {
@@ -1141,11 +1141,14 @@ disc_status part_graph(Runner& r, long long key, cudaStream_t st, F&& enqueue, B
     const int64_t before = r.launches;
     int64_t pl0[PH_COUNT];
     for (int i = 0; i < PH_COUNT; i++) pl0[i] = r.phase_launches[i];
+    const bool clean = cudaPeekAtLastError() == cudaSuccess;
     const int n = enqueue();
+    // (a launch the device refuses would only be missing from the graph)
+    const bool refused = clean && cudaPeekAtLastError() != cudaSuccess;
     r.launches = before;  // counted when the graph is launched
     for (int i = 0; i < PH_COUNT; i++) r.phase_launches[i] = pl0[i];
     cudaError_t e = cudaStreamEndCapture(st, &graph);
-    if (e != cudaSuccess) {
+    if (e != cudaSuccess || refused) {
         cudaGetLastError();
         if (graph) cudaGraphDestroy(graph);
         return DISC_ERR_CUDA;

@@ -497,7 +497,7 @@ static void launch_gemm_as(const FrameParams* fps, const BatchScratch& bs, int t
 }
 
 int launch_pool_gemm(const FrameParams* fps, const BatchScratch& bs, int B, int P, int D, int Mmax, const bool any[2][3],
-                     cudaStream_t st)
+                     bool clusters, cudaStream_t st)
 {
     if (Mmax <= 0) return 0;
     const int NT = std::max(16, (Mmax + 15) / 16 * 16);
@@ -505,9 +505,10 @@ int launch_pool_gemm(const FrameParams* fps, const BatchScratch& bs, int B, int 
     // As many CTAs per tile as leave every SM one, with two chunks each at
     // least: a single frame's 6 tiles of 18 chunks take 8 CTAs each (one CTA:
     // 59 us, all of it 18 chunks in a row); a batch that fills the SMs by
-    // itself takes one, without the exchange of partial sums.
+    // itself takes one, without the exchange of partial sums.  So does an SM
+    // partition, which may be too small or too scattered to hold a cluster.
     int KS = 1;
-    while (KS < 8 && 2 * KS * tiles * B <= 152 && 4 * KS <= chunks) KS *= 2;
+    while (clusters && KS < 8 && 2 * KS * tiles * B <= 152 && 4 * KS <= chunks) KS *= 2;
     int n = 0;
     if (any[0][0]) { launch_gemm_as<float, DISC_FP32>(fps, bs, tiles, B, NT, KS, st); n++; }
     if (any[1][0]) { launch_gemm_as<__nv_bfloat16, DISC_FP32>(fps, bs, tiles, B, NT, KS, st); n++; }

@@ -47,9 +47,10 @@ int launch_coverage(const FrameParams* fps, const BatchScratch& bs, int B, int P
 int launch_weights(const FrameParams* fps, const BatchScratch& bs, int B, int Mmax, cudaStream_t st);
 int launch_pool_exact(const FrameParams* fps, const BatchScratch& bs, int B, int P, int D, int Mmax, bool any_bf16,
                       bool any_f32, cudaStream_t st);
-// one launch per (token dtype, precision) present: any[tok_bf16][prec_bf16]
+// one launch per (token dtype, precision) present: any[tok_bf16][prec_bf16];
+// clusters: the stream reaches every SM, so a cluster of CTAs can be placed
 int launch_pool_gemm(const FrameParams* fps, const BatchScratch& bs, int B, int P, int D, int Mmax, const bool any[2][3],
-                     cudaStream_t st);
+                     bool clusters, cudaStream_t st);
 // back-projection and the per-entry pass (S_angle terms, |V_m|, labels at
 // batch start) on frames [f0, f0 + nb); then Q of every segment
 int launch_backproject(const FrameParams* fps, const BatchScratch& bs, int f0, int nb, int H, int W, cudaStream_t st);

@@ -1,6 +1,7 @@
 """The tensor-core pooled embedding at the edges of its tiles and of the split
 of the patches over a cluster: against the exact one, within 1e-5 of its norm
-per mask at FP32 precision and within the bound the gate uses at BF16 and FP8."""
+per mask at FP32 precision and within the bound the gate uses at BF16 and FP8;
+and on an SM partition too small for clusters."""
 import numpy as np
 import pytest
 
@@ -36,4 +37,40 @@ def test_pool_gemm_within_its_bound(masks, grid, dim, frames):
         if precision == 0:
             assert (err <= 1e-5 * np.linalg.norm(r["E"].astype(np.float64), axis=1)[live]).all()
         assert (err <= r["E_bound"][live]).all(), f"precision {precision}"
+        m.close()
+
+
+@pytest.mark.parametrize("precision", [0, 2])
+def test_calls_on_an_sm_partition_smaller_than_a_cluster_wants(precision):
+    # 128 of 152 SMs for the frame chain: the pooling GEMM of 250 masks (one
+    # CTA per SM at FP32) runs on what is left
+    import torch
+    from paper_2603_03935_gb300 import DiscMap, device_frame
+    dev = torch.device("cuda:0")
+    gen = torch.Generator(device=dev).manual_seed(3)
+    W, H, masks, dim = 160, 96, 250, 512
+    maps = []
+    for sms in (0, 128):
+        maps.append(DiscMap(voxel_size=0.05, embed_dim=dim, patch_h=32, patch_w=32, max_width=W, max_height=H,
+                            max_masks=masks, min_mask_pixels=1, voxel_capacity=1 << 18, max_load=0.5,
+                            instance_capacity=4096, precision=precision, serial_sms=sms, batch_frames=2))
+    frames = []
+    for i in range(8):
+        tokens = torch.randn(32 * 32, dim, device=dev, generator=gen)
+        labels = torch.randint(0, masks + 1, (H // 4, W // 4), device=dev, generator=gen).repeat_interleave(4, 0)
+        labels = labels.repeat_interleave(4, 1).to(torch.int16).contiguous()
+        depth = torch.rand(H, W, device=dev, generator=gen) * 0.2 + 2.0
+        frames.append(device_frame(depth, labels, tokens, np.eye(4), (50.0, 50.0, W / 2.0, H / 2.0), masks))
+    for lo, hi in ((0, 2), (2, 3), (3, 8)):  # one batch (asynchronous), one frame, three batches
+        for m in maps:
+            _, done, rc = m.integrate_frames_async(frames[lo:hi]).result()
+            assert rc == 0 and done == hi - lo
+        r = [m.last_frame() for m in maps]
+        live = r[0]["npix"] > 0
+        assert np.array_equal(r[0]["E"], r[1]["E"]) and np.array_equal(r[0]["rep"], r[1]["rep"])
+        for x in r:
+            err = np.linalg.norm(x["E_fast"].astype(np.float64) - x["E"], axis=1)[live]
+            assert (err <= x["E_bound"][live]).all()
+    assert all(np.array_equal(a, b) for a, b in zip(maps[0].voxels(), maps[1].voxels()))
+    for m in maps:
         m.close()
