@@ -18,18 +18,23 @@
 // kind::f8f6f4 MMA per 32-wide K step; the epilogue multiplies column m by
 // its row scale 2^b_m.
 //
-// A 128-row tile of D belongs to a cluster of KS CTAs, each of which takes a
-// KS-th of the patches (K); with KS > 1 the partial sums meet through
-// distributed shared memory, added in rank order.  One elected thread issues
-// the MMAs; a two-stage shared-memory ring is recycled through mbarriers that
+// The patches (K) fall into up to 8 groups of chunks, by their number alone.
+// Each group is accumulated by itself and the groups' sums are added in order,
+// so E does not depend on how many CTAs share the work.  A 128-row tile of D
+// belongs to a cluster of KS CTAs, each of which takes a KS-th of the groups;
+// with KS > 1 the groups' sums meet through distributed shared memory, with
+// one CTA they are added on the way.  One elected thread issues the MMAs; a
+// two-stage shared-memory ring is recycled through mbarriers that
 // tcgen05.commit arrives on.  Every wait is bounded by a global-timer limit
 // after which the kernel records DISC_ERR_TIMEOUT and returns.
 //
 // The contraction reads each token once for ~M/2 flop per byte, so it is bound
 // by how many token loads are in flight: 256 threads of 16 loads, one chunk
-// ahead, two CTAs or more per SM.  With 128 threads, one CTA per SM and one
-// CTA per tile whatever the batch, a 32-frame Room batch took 95 us (now 52) and a
-// single frame (6 CTAs) 59 us (now 13).
+// ahead, two CTAs per SM.  bf16 tokens stay as loaded until they are staged
+// (widened at the load, they made every chunk wait for the next one's: 32
+// building frames at BF16 63 us, 55 so).  With 128 threads, one CTA per SM and
+// one CTA per tile whatever the batch, a 32-frame Room batch took 95 us (now
+// 53) and a single frame (6 CTAs) 59 us (now 15).
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -146,15 +151,43 @@ __device__ __forceinline__ bool mbar_wait(uint32_t mbar, uint32_t parity)
     }
 }
 
+// 16 accumulator columns of the warp's 32 lanes; the registers hold them after
+// tcgen05.wait::ld, and tmem_use keeps their uses behind it
+__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16])
+{
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+          "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+        : "r"(taddr));
+}
+__device__ __forceinline__ void tmem_use(uint32_t (&r)[16])
+{
+#pragma unroll
+    for (int j = 0; j < 16; j++) asm volatile("" : "+r"(r[j]));
+}
+__device__ __forceinline__ void tmem_st16(uint32_t taddr, const float (&v)[16])
+{
+    asm volatile(
+        "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16};" ::"r"(
+            taddr),
+        "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]), "f"(v[4]), "f"(v[5]), "f"(v[6]), "f"(v[7]), "f"(v[8]), "f"(v[9]),
+        "f"(v[10]), "f"(v[11]), "f"(v[12]), "f"(v[13]), "f"(v[14]), "f"(v[15])
+        : "memory");
+}
+
 __device__ __forceinline__ void fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
-template <typename T>
-__device__ __forceinline__ float ldtok(const T* F, size_t i);
-template <>
-__device__ __forceinline__ float ldtok<float>(const float* F, size_t i) { return __ldg(F + i); }
-template <>
-__device__ __forceinline__ float ldtok<__nv_bfloat16>(const __nv_bfloat16* F, size_t i) { return __bfloat162float(F[i]); }
+// a token as it lies in memory (a chunk's loads stay in flight until they are
+// widened, where the chunk is staged) and its value
+__device__ __forceinline__ float ldtok(const float* F, size_t i) { return __ldg(F + i); }
+__device__ __forceinline__ unsigned short ldtok(const __nv_bfloat16* F, size_t i)
+{
+    return __ldg((const unsigned short*)F + i);
+}
+__device__ __forceinline__ float tok_f32(float x) { return x; }
+__device__ __forceinline__ float tok_f32(unsigned short x) { return __uint_as_float((unsigned)x << 16); }
 
 }  // namespace
 
@@ -162,15 +195,15 @@ constexpr uint32_t A_TILE_BYTES = GEMM_MT * GEMM_KC * 4;  // 16 KB (tf32); bf16 
 constexpr uint32_t A_LBO = (GEMM_MT / 8) * 128;           // 2048: next 16-byte K group (4 tf32 / 8 bf16 / 16 e4m3)
 
 constexpr int GEMM_THREADS = 256;
+constexpr int GEMM_GROUPS = 8;  // groups of chunks at most
 
-// The bytes of one CTA: two pipeline stages and the barriers; with a cluster
-// also room for the partial sums over the stages; and never less than its
-// share of the SM's shared memory by tensor-memory columns (512 columns over
-// 227 KB), so that the CTAs that fit an SM also fit its tensor memory and an
-// allocation never waits (a cluster's CTA that waited for columns held by
-// another cluster could wait for itself).
-constexpr size_t SMEM_MAX = 227 * 1024;
-__host__ __device__ constexpr uint32_t gemm_columns(int NT) { return NT <= 32 ? 32 : NT <= 64 ? 64 : NT <= 128 ? 128 : 256; }
+// Tensor memory: a CTA takes at most 256 of the SM's 512 columns, and its
+// registers let two CTAs onto an SM, not three (set_gemm_kernel_attrs checks
+// that), so an allocation never waits (a cluster's CTA that waited for columns
+// held by another cluster could wait for itself).
+constexpr int GEMM_COLS = 256;
+constexpr size_t SMEM_MAX = 227 * 1024, GEMM_SMEM = SMEM_MAX - 1024;  // (beside the kernel's static bytes)
+__host__ __device__ constexpr uint32_t columns_of(int n) { return n <= 32 ? 32 : n <= 64 ? 64 : n <= 128 ? 128 : 256; }
 // operand bytes of one stage: tf32 A hi | A lo (fp32 tokens only: bf16 ones are exact in tf32) | B hi | B lo, or
 // bf16 / e4m3 A | B
 __host__ __device__ constexpr uint32_t gemm_stage_bytes(int NT, int precision, bool bf16_tokens)
@@ -179,13 +212,16 @@ __host__ __device__ constexpr uint32_t gemm_stage_bytes(int NT, int precision, b
            : precision == DISC_BF16   ? A_TILE_BYTES / 2 + (uint32_t)NT * GEMM_KC * 2
                                       : A_TILE_BYTES * (bf16_tokens ? 1 : 2) + (uint32_t)NT * GEMM_KC * 8;
 }
-__host__ size_t gemm_smem_bytes(int NT, int precision, bool bf16_tokens, int KS)
+// The bytes of one CTA: two pipeline stages and the barriers; with a cluster
+// also room for the partial sums over the stages.
+__host__ size_t gemm_smem_bytes(int NT, int precision, bool bf16_tokens, int KS, int groups)
 {
     size_t b = 2 * (size_t)gemm_stage_bytes(NT, precision, bf16_tokens);
-    if (KS > 1) b = std::max(b, (size_t)NT * GEMM_MT * 4);
-    return std::max(b + 128, SMEM_MAX * gemm_columns(NT) / 512);
+    if (KS > 1) b = std::max(b, (size_t)(groups / KS) * NT * GEMM_MT * 4);
+    return b + 128;
 }
-static_assert(2 * gemm_stage_bytes(MAX_MASKS, DISC_FP32, false) + 128 <= SMEM_MAX, "the largest stage pair fits an SM");
+static_assert(2 * gemm_stage_bytes(MAX_MASKS, DISC_FP32, false) + 128 <= GEMM_SMEM, "the largest stage pair fits an SM");
+static_assert((size_t)GEMM_COLS * GEMM_MT * 4 + 128 <= GEMM_SMEM, "so do the partial sums of every column");
 
 // Test hook: when set, the kernel issues no MMA and no commit, so its bounded
 // waits run out and the frame fails with DISC_ERR_TIMEOUT (nothing is in
@@ -200,9 +236,10 @@ cudaError_t set_gemm_stall(bool on)
 
 // PR: the disc_precision of the frames this instance serves
 template <typename T, int PR>
-__global__ void __launch_bounds__(GEMM_THREADS, 2) k_pool_gemm(const FrameParams* fps, BatchScratch bs, int NT)
+__global__ void __launch_bounds__(GEMM_THREADS, 2) k_pool_gemm(const FrameParams* fps, BatchScratch bs, int NT,
+                                                               int groups)
 {
-    extern __shared__ __align__(1024) uint8_t smem[];
+    extern __shared__ __align__(128) uint8_t smem[];
     __shared__ int s_err;
     const FrameParams& fp = fps[blockIdx.z];
     const Scratch sc = bs.frame(blockIdx.z);
@@ -233,10 +270,15 @@ __global__ void __launch_bounds__(GEMM_THREADS, 2) k_pool_gemm(const FrameParams
     const uint32_t B_LBO = (uint32_t)NT * 16;
     const uint32_t STAGE = gemm_stage_bytes(NT, PR, !LO);
     // the barriers lie past the stages and past the partial sums over them
-    const size_t used = max(2 * (size_t)STAGE, KS > 1 ? (size_t)NT * GEMM_MT * 4 : (size_t)0);
+    const int gp = groups / (int)KS;  // groups of this CTA
+    const size_t used = max(2 * (size_t)STAGE, KS > 1 ? (size_t)gp * NT * GEMM_MT * 4 : (size_t)0);
     uint64_t* mbar = (uint64_t*)(smem + used);
     uint32_t* tmem_slot = (uint32_t*)(mbar + 2);
-    const uint32_t ncols = gemm_columns(NT);
+    // A cluster's CTA keeps an accumulator per group.  A CTA that takes a tile
+    // alone keeps one, and the sum of the groups before: in the columns past
+    // it, or (above 128 masks) in the result's place in memory.
+    const bool sums = KS == 1 && gp > 1, tsum = sums && 2 * NT <= GEMM_COLS;
+    const uint32_t ncols = columns_of(KS > 1 ? gp * NT : tsum ? 2 * NT : NT);
 
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
@@ -257,6 +299,8 @@ __global__ void __launch_bounds__(GEMM_THREADS, 2) k_pool_gemm(const FrameParams
     // this CTA's share of the 32-patch chunks
     const int all_chunks = (P + GEMM_KC - 1) / GEMM_KC;
     const int cb = (int)(all_chunks * rank / KS), nchunks = (int)(all_chunks * (rank + 1) / KS) - cb;
+    auto group_start = [&](int g) { return all_chunks * ((int)rank * gp + g) / groups - cb; };
+    int group = 0, group_at = 0, group_end = group_start(1);  // the group of the current chunk
     bool failed = false;
     int last_commit = -1;  // chunk of the most recent commit (same on all threads)
     const bool stall = g_gemm_stall != 0;  // uniform: read once
@@ -266,12 +310,13 @@ __global__ void __launch_bounds__(GEMM_THREADS, 2) k_pool_gemm(const FrameParams
     // multiplied, so loads stay in flight across the loop.
     constexpr int HALF = GEMM_KC / 2, WPRE = 2;
     const int row = tid & 127, half = tid >> 7;
-    auto load_chunk = [&](int c, float (&x)[HALF]) {
+    using Raw = decltype(ldtok((const T*)nullptr, 0));
+    auto load_chunk = [&](int c, Raw (&x)[HALF]) {
         const int d = d0 + row, p0 = (cb + c) * GEMM_KC + half * HALF;
 #pragma unroll
         for (int j = 0; j < HALF; j++) {
             const int p = p0 + j;
-            x[j] = (d < D && p < P) ? ldtok<T>(F, (size_t)p * D + d) : 0.0f;
+            x[j] = (d < D && p < P) ? ldtok(F, (size_t)p * D + d) : Raw(0);
         }
     };
     // granule g of the chunk's weight tile: 16 bytes of e4m3, or 16 bytes of
@@ -283,7 +328,7 @@ __global__ void __launch_bounds__(GEMM_THREADS, 2) k_pool_gemm(const FrameParams
         if constexpr (F8) return *(const float4*)(sc.W8 + (size_t)n * fp.Kpad + p0 + 16 * kq);
         else return *(const float4*)(sc.W + (size_t)n * fp.Kpad + p0 + 4 * kq);
     };
-    float xn[HALF];
+    Raw xn[HALF];
     float4 wn[WPRE];
     auto prefetch = [&](int c) {
         load_chunk(c, xn);
@@ -295,13 +340,39 @@ __global__ void __launch_bounds__(GEMM_THREADS, 2) k_pool_gemm(const FrameParams
     };
     if (nchunks > 0) prefetch(0);
 
+    // The accumulators in tensor memory: warp w reads lanes 32 (w & 3) .. + 31
+    // (rows of D), columns (masks) in 16s, alternating between the two warps
+    // of the same lanes.  add_group: 16 columns of the group's accumulator
+    // onto the sum of the groups before.
+    const uint32_t tlane = tmem + ((uint32_t)((warp & 3) * 32) << 16);
+    const int er = (warp & 3) * 32 + lane;
+    float* out = sc.Efast + d0 + er;  // of mask 0
+    const bool er_in = d0 + er < D;
+    auto add_group = [&](int c0, float (&v)[16]) {
+        uint32_t r[16], q[16];
+        tmem_ld16(tlane + (uint32_t)c0, r);
+        if (tsum) {
+            if (group > 0) tmem_ld16(tlane + (uint32_t)(NT + c0), q);
+        } else {
+#pragma unroll
+            for (int j = 0; j < 16; j++)
+                q[j] = group > 0 && er_in && c0 + j < M ? __float_as_uint(out[(size_t)(c0 + j) * D]) : 0u;
+        }
+        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+        tmem_use(r);
+        if (group > 0) tmem_use(q);
+#pragma unroll
+        for (int j = 0; j < 16; j++)
+            v[j] = __fadd_rn(group > 0 ? __uint_as_float(q[j]) : 0.0f, __uint_as_float(r[j]));
+    };
+
     for (int c = 0; c < nchunks && !failed; c++) {
         const int s = c & 1;
         uint8_t* st = smem + s * STAGE;
         float x[HALF];
         float4 w[WPRE];
 #pragma unroll
-        for (int j = 0; j < HALF; j++) x[j] = xn[j];
+        for (int j = 0; j < HALF; j++) x[j] = tok_f32(xn[j]);
 #pragma unroll
         for (int i = 0; i < WPRE; i++) w[i] = wn[i];
         if (c + 1 < nchunks) prefetch(c + 1);
@@ -309,6 +380,29 @@ __global__ void __launch_bounds__(GEMM_THREADS, 2) k_pool_gemm(const FrameParams
             // the MMAs of chunk c-2 read this stage: wait for their commit
             bool ok = mbar_wait(smem_u32(&mbar[s]), (uint32_t)(((c >> 1) - 1) & 1));
             if (__syncthreads_or(!ok)) { failed = true; break; }
+        }
+        if (c == group_end) {
+            if (sums) {  // the group is whole once its last chunk's MMAs are done
+                const bool ok = mbar_wait(smem_u32(&mbar[s ^ 1]), (uint32_t)(((c - 1) >> 1) & 1));
+                if (__syncthreads_or(!ok)) { failed = true; break; }
+                fence_after();
+                for (int c0 = 16 * (warp >> 2); c0 < NT; c0 += 32) {
+                    float v[16];
+                    add_group(c0, v);
+                    if (tsum) {
+                        tmem_st16(tlane + (uint32_t)(NT + c0), v);
+                    } else if (er_in) {
+#pragma unroll
+                        for (int j = 0; j < 16; j++)
+                            if (c0 + j < M) out[(size_t)(c0 + j) * D] = v[j];
+                    }
+                }
+                asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+                fence_before();  // (the next MMAs overwrite the accumulator after the barrier below)
+            }
+            group_at = c;
+            group++;
+            group_end = group_start(group + 1);
         }
         // A: the F^T tile
         if constexpr (F8) {
@@ -381,18 +475,19 @@ __global__ void __launch_bounds__(GEMM_THREADS, 2) k_pool_gemm(const FrameParams
         __syncthreads();
         if (tid == 0 && !stall) {
             fence_after();
+            const uint32_t acc = tmem + (KS > 1 ? (uint32_t)(group * NT) : 0u);
             if constexpr (F8) {
                 // one K step of 32 = two 16-byte core-matrix columns of e4m3
                 const uint32_t a0 = smem_u32(st), b0 = a0 + A_BYTES;
-                mma_e4m3(tmem, smem_desc(a0, A_LBO, 128), smem_desc(b0, B_LBO, 128), idesc, c > 0 ? 1u : 0u);
+                mma_e4m3(acc, smem_desc(a0, A_LBO, 128), smem_desc(b0, B_LBO, 128), idesc, c > group_at ? 1u : 0u);
             } else if constexpr (BF) {
                 // K step 16 = two 16-byte core-matrix columns of bf16
                 const uint32_t a0 = smem_u32(st), b0 = a0 + A_BYTES;
 #pragma unroll
                 for (int ks = 0; ks < GEMM_KC / 16; ks++) {
                     const uint32_t ao = ks * 2 * A_LBO, bo = ks * 2 * B_LBO;
-                    mma_bf16(tmem, smem_desc(a0 + ao, A_LBO, 128), smem_desc(b0 + bo, B_LBO, 128), idesc,
-                             (c > 0 || ks > 0) ? 1u : 0u);
+                    mma_bf16(acc, smem_desc(a0 + ao, A_LBO, 128), smem_desc(b0 + bo, B_LBO, 128), idesc,
+                             (c > group_at || ks > 0) ? 1u : 0u);
                 }
             } else {
                 const uint32_t a_hi = smem_u32(st), a_lo = a_hi + A_BYTES;
@@ -402,52 +497,44 @@ __global__ void __launch_bounds__(GEMM_THREADS, 2) k_pool_gemm(const FrameParams
                     const uint32_t ao = ks * 2 * A_LBO, bo = ks * 2 * B_LBO;
                     const uint64_t dah = smem_desc(a_hi + ao, A_LBO, 128);
                     const uint64_t dbh = smem_desc(b_hi + bo, B_LBO, 128), dbl = smem_desc(b_lo + bo, B_LBO, 128);
-                    mma_tf32(tmem, dah, dbh, idesc, (c > 0 || ks > 0) ? 1u : 0u);
-                    mma_tf32(tmem, dah, dbl, idesc, 1u);
-                    if constexpr (LO) mma_tf32(tmem, smem_desc(a_lo + ao, A_LBO, 128), dbh, idesc, 1u);
+                    mma_tf32(acc, dah, dbh, idesc, (c > group_at || ks > 0) ? 1u : 0u);
+                    mma_tf32(acc, dah, dbl, idesc, 1u);
+                    if constexpr (LO) mma_tf32(acc, smem_desc(a_lo + ao, A_LBO, 128), dbh, idesc, 1u);
                 }
             }
             mma_commit(smem_u32(&mbar[s]));
         }
         if (!stall) last_commit = c;
     }
-    if (!failed && nchunks > 0) {
+    if (!failed) {
         const int c = nchunks - 1;
         bool ok = mbar_wait(smem_u32(&mbar[c & 1]), (uint32_t)((c >> 1) & 1));
         failed = __syncthreads_or(!ok);
     }
     fence_after();
-    // epilogue: warp w reads TMEM lanes 32 (w & 3) .. + 31 (rows of D), columns
-    // (masks) in 16s, alternating between the two warps of the same lanes
-    float* part = (float*)smem;  // [NT][128] this CTA's partial sums (KS > 1; every MMA is done)
+    // epilogue
+    float* part = (float*)smem;  // [gp][NT][128] this CTA's partial sums (KS > 1; every MMA is done)
     if (!failed) {
-        const int er = (warp & 3) * 32 + lane, d = d0 + er;
         for (int c0 = 16 * (warp >> 2); c0 < NT; c0 += 32) {
-            uint32_t r[16];
-            if (nchunks > 0) {
-                const uint32_t taddr = tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)c0;
-                asm volatile(
-                    "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, "
-                    "[%16];"
-                    : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-                      "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]),
-                      "=r"(r[15])
-                    : "r"(taddr));
-                asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-            } else {
+            if (KS > 1) {
+                for (int g = 0; g < gp; g++) {
+                    uint32_t r[16];
+                    tmem_ld16(tlane + (uint32_t)(g * NT + c0), r);
+                    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+                    tmem_use(r);
 #pragma unroll
-                for (int j = 0; j < 16; j++) r[j] = 0u;
+                    for (int j = 0; j < 16; j++) part[(g * NT + c0 + j) * GEMM_MT + er] = __uint_as_float(r[j]);
+                }
+                continue;
             }
+            float v[16];
+            add_group(c0, v);
 #pragma unroll
             for (int j = 0; j < 16; j++) {
                 const int m = c0 + j;
-                if (KS > 1) {
-                    part[m * GEMM_MT + er] = __uint_as_float(r[j]);
-                } else if (m < M && d < D) {
-                    float v = __uint_as_float(r[j]);
-                    if constexpr (F8) v = scale_pow2(v, sc.qexpm[m]);
-                    sc.Efast[(size_t)m * D + d] = v;
-                }
+                if (m >= M || !er_in) continue;
+                if constexpr (F8) v[j] = scale_pow2(v[j], sc.qexpm[m]);
+                out[(size_t)m * D] = v[j];
             }
         }
     } else {
@@ -457,15 +544,23 @@ __global__ void __launch_bounds__(GEMM_THREADS, 2) k_pool_gemm(const FrameParams
         if (tid == 0) atomicCAS(&sc.ctr->err, 0, DISC_ERR_TIMEOUT);
     }
     if (KS > 1) {
-        // the cluster's partial sums, in rank order (a CTA that failed leaves
-        // what it had staged: its frame has failed); each CTA takes every
-        // KS-th mask
+        // the cluster's partial sums, group after group (a CTA that failed
+        // leaves what it had staged: its frame has failed); each CTA takes
+        // every KS-th mask
         cluster_sync();
         const int d = d0 + row;
+        unsigned at[GEMM_GROUPS];  // the row's partial sums of mask 0 (groups and KS are powers of two)
+#pragma unroll
+        for (int g = 0; g < GEMM_GROUPS; g++)
+            if (g < groups) at[g] = dsm_map(part + (g & (gp - 1)) * NT * GEMM_MT + row, (unsigned)g >> (gp >> 1));
         for (int m = (int)rank + (int)KS * half; m < M; m += 2 * (int)KS) {
-            float v = 0.0f;
-            for (unsigned q = 0; q < KS; q++)
-                v += __int_as_float(dsm_ld32(dsm_map(part + m * GEMM_MT + row, q)));
+            float p[GEMM_GROUPS], v = 0.0f;
+#pragma unroll
+            for (int g = 0; g < GEMM_GROUPS; g++)  // all on their way before the first is added
+                if (g < groups) p[g] = __int_as_float(dsm_ld32(at[g] + (unsigned)(m * GEMM_MT * 4)));
+#pragma unroll
+            for (int g = 0; g < GEMM_GROUPS; g++)
+                if (g < groups) v = __fadd_rn(v, p[g]);
             if constexpr (F8) v = scale_pow2(v, sc.qexpm[m]);
             if (d < D) sc.Efast[(size_t)m * D + d] = v;
         }
@@ -479,7 +574,7 @@ __global__ void __launch_bounds__(GEMM_THREADS, 2) k_pool_gemm(const FrameParams
 
 template <typename T, int PR>
 static void launch_gemm_as(const FrameParams* fps, const BatchScratch& bs, int tiles, int B, int NT, int KS,
-                           cudaStream_t st)
+                           int groups, cudaStream_t st)
 {
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute at[1];
@@ -489,11 +584,11 @@ static void launch_gemm_as(const FrameParams* fps, const BatchScratch& bs, int t
     at[0].val.clusterDim.z = 1;
     cfg.gridDim = dim3(KS, tiles, B);
     cfg.blockDim = dim3(GEMM_THREADS);
-    cfg.dynamicSmemBytes = gemm_smem_bytes(NT, PR, sizeof(T) == 2, KS);
+    cfg.dynamicSmemBytes = gemm_smem_bytes(NT, PR, sizeof(T) == 2, KS, groups);
     cfg.stream = st;
     cfg.attrs = at;
     cfg.numAttrs = 1;
-    cudaLaunchKernelEx(&cfg, k_pool_gemm<T, PR>, fps, bs, NT);
+    cudaLaunchKernelEx(&cfg, k_pool_gemm<T, PR>, fps, bs, NT, groups);
 }
 
 int launch_pool_gemm(const FrameParams* fps, const BatchScratch& bs, int B, int P, int D, int Mmax, const bool any[2][3],
@@ -502,28 +597,42 @@ int launch_pool_gemm(const FrameParams* fps, const BatchScratch& bs, int B, int 
     if (Mmax <= 0) return 0;
     const int NT = std::max(16, (Mmax + 15) / 16 * 16);
     const int tiles = (D + GEMM_MT - 1) / GEMM_MT, chunks = (P + GEMM_KC - 1) / GEMM_KC;
-    // As many CTAs per tile as leave every SM one, with two chunks each at
-    // least: a single frame's 6 tiles of 18 chunks take 8 CTAs each (one CTA:
-    // 59 us, all of it 18 chunks in a row); a batch that fills the SMs by
-    // itself takes one, without the exchange of partial sums.  So does an SM
-    // partition, which may be too small or too scattered to hold a cluster.
+    // How the patches are grouped depends on their number alone: two chunks to
+    // a group at least, eight groups at most.
+    int groups = 1;
+    while (groups < GEMM_GROUPS && 4 * groups <= chunks) groups *= 2;
+    // A small batch takes a CTA per group, or one per two groups, a large one
+    // a CTA per tile, without the exchange of partial sums (below): us for 1 |
+    // 4 | 8 | 16 | 32 Room frames with 8 CTAs per tile 15.5 | 19.3 | 28.7 |
+    // 44.1 | 79, with 4 19.4 | 19.4 | 25.5 | 37.8 | 59, with one 39 | 39 | 40 |
+    // 40 | 53.  Above 128 masks two groups' accumulators do not fit, and 8 CTAs
+    // are faster than one up to 16 frames (200 masks: 63 and 78 us).  An SM
+    // partition may be too small or too scattered to hold a cluster.
     int KS = 1;
-    while (clusters && KS < 8 && 2 * KS * tiles * B <= 152 && 4 * KS <= chunks) KS *= 2;
+    if (clusters) {
+        const bool pairs = groups == 8 && 2 * NT <= GEMM_COLS;
+        if (groups * tiles * B <= (pairs ? 152 : 2 * NT <= GEMM_COLS ? 400 : 800)) KS = groups;
+        else if (pairs && 4 * tiles * B <= 400) KS = 4;
+    }
     int n = 0;
-    if (any[0][0]) { launch_gemm_as<float, DISC_FP32>(fps, bs, tiles, B, NT, KS, st); n++; }
-    if (any[1][0]) { launch_gemm_as<__nv_bfloat16, DISC_FP32>(fps, bs, tiles, B, NT, KS, st); n++; }
-    if (any[0][1]) { launch_gemm_as<float, DISC_BF16>(fps, bs, tiles, B, NT, KS, st); n++; }
-    if (any[1][1]) { launch_gemm_as<__nv_bfloat16, DISC_BF16>(fps, bs, tiles, B, NT, KS, st); n++; }
-    if (any[0][2]) { launch_gemm_as<float, DISC_FP8_E4M3>(fps, bs, tiles, B, NT, KS, st); n++; }
-    if (any[1][2]) { launch_gemm_as<__nv_bfloat16, DISC_FP8_E4M3>(fps, bs, tiles, B, NT, KS, st); n++; }
+    if (any[0][0]) { launch_gemm_as<float, DISC_FP32>(fps, bs, tiles, B, NT, KS, groups, st); n++; }
+    if (any[1][0]) { launch_gemm_as<__nv_bfloat16, DISC_FP32>(fps, bs, tiles, B, NT, KS, groups, st); n++; }
+    if (any[0][1]) { launch_gemm_as<float, DISC_BF16>(fps, bs, tiles, B, NT, KS, groups, st); n++; }
+    if (any[1][1]) { launch_gemm_as<__nv_bfloat16, DISC_BF16>(fps, bs, tiles, B, NT, KS, groups, st); n++; }
+    if (any[0][2]) { launch_gemm_as<float, DISC_FP8_E4M3>(fps, bs, tiles, B, NT, KS, groups, st); n++; }
+    if (any[1][2]) { launch_gemm_as<__nv_bfloat16, DISC_FP8_E4M3>(fps, bs, tiles, B, NT, KS, groups, st); n++; }
     return n;
 }
 
 template <typename T, int PR>
 static cudaError_t gemm_attr()
 {
+    cudaFuncAttributes a;
+    const cudaError_t e = cudaFuncGetAttributes(&a, k_pool_gemm<T, PR>);
+    if (e != cudaSuccess) return e;
+    if (3 * GEMM_THREADS * a.numRegs <= 65536) return cudaErrorInvalidConfiguration;  // see GEMM_COLS
     return cudaFuncSetAttribute(k_pool_gemm<T, PR>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)gemm_smem_bytes(MAX_MASKS, PR, sizeof(T) == 2, 8));
+                                (int)GEMM_SMEM);
 }
 
 cudaError_t set_gemm_kernel_attrs()

@@ -1,7 +1,7 @@
 """The tensor-core pooled embedding at the edges of its tiles and of the split
 of the patches over a cluster: against the exact one, within 1e-5 of its norm
 per mask at FP32 precision and within the bound the gate uses at BF16 and FP8;
-and on an SM partition too small for clusters."""
+on an SM partition too small for clusters; and the same bits in every batch."""
 import numpy as np
 import pytest
 
@@ -73,4 +73,39 @@ def test_calls_on_an_sm_partition_smaller_than_a_cluster_wants(precision):
             assert (err <= x["E_bound"][live]).all()
     assert all(np.array_equal(a, b) for a, b in zip(maps[0].voxels(), maps[1].voxels()))
     for m in maps:
+        m.close()
+
+
+# patches: 8, 5, 31 and 3 chunks (4, 2, 8 and 1 groups)
+@pytest.mark.parametrize("masks,precision,bf16", [(20, 0, False), (100, 1, True), (200, 0, False), (250, 2, True),
+                                                  (130, 1, False)])
+@pytest.mark.parametrize("grid,dim", [((16, 16), 200), ((12, 13), 128), ((32, 31), 700), ((9, 9), 64)])
+def test_the_pooled_embedding_does_not_depend_on_the_batch(grid, dim, masks, precision, bf16):
+    # the same frame last in batches of 1 to 64 frames, in smaller batches and
+    # on an SM partition: the same bits
+    import torch
+    from paper_2603_03935_gb300 import DiscMap, device_frame
+    dev = torch.device("cuda:0")
+    gen = torch.Generator(device=dev).manual_seed(masks)
+    W, H, P = 128, 96, grid[0] * grid[1]
+    frames = []
+    for i in range(2):
+        tokens = torch.randn(P, dim, device=dev, generator=gen)
+        labels = torch.randint(0, masks + 1, (H // 2, W // 2), device=dev, generator=gen).repeat_interleave(2, 0)
+        labels = labels.repeat_interleave(2, 1).to(torch.int16).contiguous()
+        depth = torch.full((H, W), 2.0, device=dev)
+        frames.append(device_frame(depth, labels, tokens.bfloat16() if bf16 else tokens, np.eye(4),
+                                   (50.0, 50.0, W / 2.0, H / 2.0), masks))
+    first = None
+    for n, split, sms in ((1, 0, 0), (3, 0, 0), (7, 0, 0), (14, 1, 0), (30, 1, 0), (64, 1, 0), (64, 8, 0), (16, 0, 64)):
+        m = DiscMap(voxel_size=0.05, embed_dim=dim, patch_h=grid[0], patch_w=grid[1], max_width=W, max_height=H,
+                    max_masks=masks, min_mask_pixels=1, voxel_capacity=1 << 16, max_load=0.5, instance_capacity=1024,
+                    precision=precision, batch_frames=64, serial_sms=sms)
+        m.set_schedule(batch_split=split)
+        m.integrate_frames([frames[0]] * (n - 1) + [frames[1]])
+        r = m.last_frame()
+        if first is None:
+            first = r["E_fast"], r["E_bound"]
+            assert np.abs(first[0]).max() > 0
+        assert np.array_equal(r["E_fast"], first[0]) and np.array_equal(r["E_bound"], first[1]), (n, split, sms)
         m.close()
