@@ -86,18 +86,21 @@ __global__ void k_slot_reset(BatchScratch bs, int B)
 // Each valid pixel becomes a record (its (mask, voxel) key and exact normal)
 // of the partition its key hashes to: one counter increment and one 32-byte
 // store, no probing and nothing that the frame's next use has to clear.
-// Unless nearly every pixel of the tile starts a run of equal keys along its
-// row (more than 7/8 of the valid ones: far surfaces, fine voxels), the pixels
-// first meet in a shared hash that sums their normals, and only the tile's
-// distinct keys become records.  Depth noise breaks the runs of pixels whose
-// voxels repeat all over the tile, and a voxel's records pile up in one
-// partition, where k_entries sums them one after the other: Room frames with
-// 1 % noise had 231,000 records of 72,000 voxels, up to 86 of one, with the
-// line at half the valid pixels.  Back-projection and entries, us per frame,
-// with the line at 1/2 | 3/4 | 7/8 | 15/16 | every tile merged: those frames
-// 17.1 | 12.3 | 11.7 | 12.0 | 12.4; the same room drifting 14.2 | 13.4 | 12.7 |
-// 13.3 | 14.0; a building of 5 cm voxels 11.9 | 10.3 | 9.9 | 10.0 | 10.0; 16
-// uneven maps 9.4 | 9.1 | 8.8 | 9.1 | 9.3.
+// Pixels that share a voxel first add up inside a thread and between two
+// neighbouring ones. Unless most of what is left is distinct (far surfaces,
+// fine voxels), the tile's pixels then meet in a shared hash that sums their
+// normals, and only its distinct keys become records: a voxel's records pile
+// up in one partition, where k_entries sums them one after the other. The
+// line is drawn on the keys themselves, a sample of one per thread counted in
+// a bitmap of their hashes, so holes, sparse depth and alternating labels do
+// not move it.  (Runs of equal keys along the rows, the line before, are broken
+// by a missing column: Room frames with every other column of depth missing
+// and 20 cm voxels took 31 us a frame, now 9, with 1 m voxels 201, now 8.)
+// Back-projection and entries, us per frame, tiles merged when fewer than 1/4 |
+// 1/2 | 5/8 | 3/4 | 7/8 of the sample are distinct: Room 13.3 | 12.6 | 12.7 |
+// 12.8 | 13.1 (by runs 12.5); a building of 5 cm voxels 10.7 | 10.1 | 10.0 |
+// 10.1 | 10.1 (9.9); Room without the depth noise 11.5 | 11.2 | 11.2 | 11.3 |
+// 11.6 (11.5); alternating labels 13.6 | 13.0 | 12.6 | 12.7 | 13.1 (13.7).
 // Bound by instruction issue (60 % active) and by the scattered record stores
 // and counter increments, one line per lane (L1 70 % busy).  Measured on Room
 // frames (640x480, 2.5 cm voxels, 8 frames per launch) in place of one global
@@ -110,6 +113,7 @@ constexpr int BP_TX = 32, BP_TY = 16, BP_PER = 2;      // tile; pixels per threa
 constexpr int BP_ROWS = BP_TY / BP_PER, BP_THREADS = BP_TX * BP_ROWS;
 constexpr int BP_HX = BP_TX + 2, BP_HY = BP_TY + 2, BP_HALO = BP_HX * BP_HY;
 constexpr int BP_SLOTS = 2 * BP_TX * BP_TY;
+constexpr int BP_LOG_BITS = 11, BP_BITS = 1 << BP_LOG_BITS;
 
 struct __align__(16) TilePoint {
     float p[3];
@@ -156,7 +160,8 @@ __global__ void __launch_bounds__(BP_THREADS) k_backproject(const FrameParams* f
     __shared__ __align__(16) unsigned char smem[HASH_BYTES];
     __shared__ unsigned short tlist[BP_TX * BP_TY];  // claimed tile slots
     __shared__ unsigned s_act[MAX_MASKS / 32];        // masks of at least min_px pixels
-    __shared__ int s_valid, s_runs, s_dropped, s_listed, s_err;
+    __shared__ uint4 s_bits[BP_BITS / 128];          // a bit per hash value of the tile's keys
+    __shared__ int s_valid, s_samples, s_dropped, s_listed, s_err;
     TilePoint* tp = (TilePoint*)smem;
     const FrameParams& fp = fps[f0 + blockIdx.z];
     const Scratch sc = bs.frame(f0 + blockIdx.z);
@@ -165,9 +170,10 @@ __global__ void __launch_bounds__(BP_THREADS) k_backproject(const FrameParams* f
     if (M <= 0 || u0 + 1 >= W || v0 + 1 >= H) return;  // uniform per block
     const int tid = threadIdx.y * BP_TX + threadIdx.x, lane = threadIdx.x;
     if (tid == 0) {
-        s_valid = s_runs = s_dropped = s_listed = 0;
+        s_valid = s_samples = s_dropped = s_listed = 0;
         s_err = sc.ctr->geo_err;
     }
+    if (tid < BP_BITS / 128) s_bits[tid] = make_uint4(0, 0, 0, 0);
     {
         const unsigned act = __ballot_sync(0xffffffffu, tid < M && sc.npix[tid] >= fp.min_px);
         if (lane == 0) s_act[threadIdx.y] = act;
@@ -223,7 +229,7 @@ __global__ void __launch_bounds__(BP_THREADS) k_backproject(const FrameParams* f
     if (s_err) return;
     unsigned long long hk[BP_PER];  // 0: no record
     long long nfix[BP_PER][3];
-    int nvalid = 0, ndrop = 0, nrun = 0;
+    int nvalid = 0, ndrop = 0;
 #pragma unroll
     for (int j = 0; j < BP_PER; j++) {
         const int at = at0 + j * BP_HX;
@@ -240,20 +246,6 @@ __global__ void __launch_bounds__(BP_THREADS) k_backproject(const FrameParams* f
         }
         nvalid += __popc(__ballot_sync(0xffffffffu, keyed));
         ndrop += __popc(__ballot_sync(0xffffffffu, active && !keyed));
-        const unsigned long long left = __shfl_up_sync(0xffffffffu, hk[j], 1);
-        nrun += __popc(__ballot_sync(0xffffffffu, keyed && (lane == 0 || left != hk[j])));
-    }
-    if (lane == 0) {
-        if (nvalid) {
-            atomicAdd(&s_valid, nvalid);
-            atomicAdd(&s_runs, nrun);
-        }
-        if (ndrop) atomicAdd(&s_dropped, ndrop);
-    }
-    __syncthreads();
-    if (tid == 0) {
-        if (s_valid) atomicAdd(&sc.ctr->valid_pixels, s_valid);
-        if (s_dropped) atomicAdd(&sc.ctr->dropped_pixels, s_dropped);
     }
     // the thread's two pixels, then the pixels of two neighbouring threads,
     // add up where they share a voxel
@@ -274,8 +266,31 @@ __global__ void __launch_bounds__(BP_THREADS) k_backproject(const FrameParams* f
         }
         if (same && (lane & 1)) hk[j] = 0ull;
     }
+    // a sum of every thread that has one, and how many distinct keys they have
+    // (nearly: a bit may stand for several)
+    unsigned* bits = (unsigned*)s_bits;
+    const unsigned long long sample = hk[0] ? hk[0] : hk[1];
+    const int nsample = __popc(__ballot_sync(0xffffffffu, sample != 0ull));
+    if (sample) {
+        const unsigned b = ((unsigned)sample * 0x9E3779B1u + (unsigned)(sample >> 32) * 0x85EBCA77u) >> (32 - BP_LOG_BITS);
+        atomicOr(&bits[b >> 5], 1u << (b & 31));
+    }
+    if (lane == 0) {
+        if (nvalid) atomicAdd(&s_valid, nvalid);
+        if (nsample) atomicAdd(&s_samples, nsample);
+        if (ndrop) atomicAdd(&s_dropped, ndrop);
+    }
+    __syncthreads();
+    if (tid == 0) {
+        if (s_valid) atomicAdd(&sc.ctr->valid_pixels, s_valid);
+        if (s_dropped) atomicAdd(&sc.ctr->dropped_pixels, s_dropped);
+    }
+    int distinct = 0;
+#pragma unroll
+    for (int i = 0; i < BP_BITS / 32; i += 32) distinct += __popc(bits[i + lane]);
+    distinct = __reduce_add_sync(0xffffffffu, distinct);
     const int parts = seg_parts((long long)W * H);
-    if (8 * s_runs > 7 * s_valid || s_valid == 0) {  // uniform per block
+    if (8 * distinct > 5 * s_samples || s_samples == 0) {  // uniform per block
 #pragma unroll
         for (int j = 0; j < BP_PER; j++)
             if (hk[j]) seg_append(sc, parts, hk[j], nfix[j][0], nfix[j][1], nfix[j][2]);

@@ -125,3 +125,70 @@ def test_skewed_voxel_tables_use_every_slot(probe_width):
     xyz = (np.stack(k, 1) + 0.5) * 0.02
     assert np.array_equal(gmap.query_points(xyz.astype(np.float32)), ids)
     gmap.close()
+
+
+def _sparse(kind, depth, labels):
+    """Every other column, a checkerboard, every other row, or every other column of every fourth row of depth, or two
+    labels in a checkerboard."""
+    v, u = np.meshgrid(np.arange(depth.shape[0]), np.arange(depth.shape[1]), indexing="ij")
+    if kind == "labels":
+        return depth, np.where((u + v) % 2 == 1, (labels - 1) // 2 * 2 + 1, (labels - 1) // 2 * 2 + 2).astype(np.uint16)
+    keep = {"columns": u % 2 == 0, "checker": (u + v) % 2 == 0, "rows": v % 2 == 1,
+            "beams": (u % 2 == 0) & (v % 4 == 0)}[kind]
+    return np.where(keep, depth, 0.0).astype(np.float32), labels
+
+
+@pytest.mark.parametrize("kind", ["columns", "checker", "rows", "beams", "labels"])
+@pytest.mark.parametrize("voxel", [0.01, 0.06, 0.9])
+def test_sparse_frames_equal_the_oracle(kind, voxel):
+    import torch
+    from paper_2603_03935_gb300 import DiscMap, device_frame
+    dev = torch.device("cuda:0")
+    rng = np.random.default_rng(9)
+    width, height, masks = 131, 75, 6
+    depth, _ = _wall(width, height, 1.5, 0.002, voxel)
+    labels = ((np.arange(height)[:, None] // 20 + np.arange(width)[None, :] // 30) % masks + 1).astype(np.uint16)
+    depth, labels = _sparse(kind, depth, labels)
+    tokens = rng.normal(size=(GRID[0] * GRID[1], DIM)).astype(np.float32)
+    cfg = dict(voxel_size=voxel, embed_dim=DIM, patch_h=GRID[0], patch_w=GRID[1], max_width=width, max_height=height,
+               max_masks=masks, min_mask_pixels=1, voxel_capacity=1 << 15, max_load=0.5, instance_capacity=256,
+               z_min=0.1, z_max=10.0, eps=1e-6, tau_cos=0.75, lambda_size=3.3, ov_num=1, ov_den=5)
+    gmap, omap = DiscMap(**cfg), oracle.OracleMap(**common.to_oracle_cfg(cfg))
+    intr = (50.0, 50.0, width / 2.0, height / 2.0)
+    st = gmap.integrate(device_frame(torch.from_numpy(depth).to(dev), torch.from_numpy(labels.view(np.int16)).to(dev),
+                                     torch.from_numpy(tokens).to(dev), np.eye(4), intr, masks))
+    o = omap.integrate(depth, labels, tokens, np.eye(4), intr, masks)
+    common.compare_frame(st, gmap.last_frame(), o, ctx=f"{kind}, voxels of {voxel}")
+    common.compare_maps(gmap, omap, ctx=kind)
+    gmap.close()
+
+
+@pytest.mark.parametrize("kind", ["columns", "checker", "labels"])
+def test_holes_do_not_cost_more_than_the_pixels_they_replace(kind):
+    # Coarse voxels: nearly every pixel shares its voxel with its tile's others, and has to be merged with them
+    # whatever lies between them. Half the pixels (or as many, under two labels) take no more than twice the time of
+    # all of them; unmerged, a voxel's records pile up in one partition (over ten times).
+    import torch
+    from paper_2603_03935_gb300 import DiscMap, device_frame
+    dev = torch.device("cuda:0")
+    width, height, masks, n = 640, 480, 8, 16
+    dense, _ = _wall(width, height, 2.0, 0.001, 0.5, f=525.0)
+    whole = ((np.arange(height)[:, None] // 240 + np.arange(width)[None, :] // 160 * 2) % masks + 1).astype(np.uint16)
+    tokens = torch.randn(GRID[0] * GRID[1], DIM, device=dev)
+    intr = (525.0, 525.0, width / 2.0, height / 2.0)
+    ms = []
+    for depth, labels in ((dense, whole), _sparse(kind, dense, whole)):
+        gmap = DiscMap(voxel_size=0.5, embed_dim=DIM, patch_h=GRID[0], patch_w=GRID[1], max_width=width,
+                       max_height=height, max_masks=masks, min_mask_pixels=1, voxel_capacity=1 << 14, max_load=0.5,
+                       instance_capacity=1024, z_min=0.1, z_max=10.0, batch_frames=n)
+        fr = device_frame(torch.from_numpy(depth).to(dev), torch.from_numpy(labels.view(np.int16)).to(dev), tokens,
+                          np.eye(4), intr, masks)
+        best = 1e9
+        for _ in range(4):
+            gmap.set_phase_timing(True)
+            gmap.integrate_frames([fr] * n)
+            ph = gmap.phase_times()
+            best = min(best, ph["backproject"]["ms"] + ph["entries"]["ms"])
+        ms.append(best)
+        gmap.close()
+    assert ms[1] < 2 * ms[0], ms
