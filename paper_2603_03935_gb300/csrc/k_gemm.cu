@@ -197,13 +197,17 @@ constexpr uint32_t A_LBO = (GEMM_MT / 8) * 128;           // 2048: next 16-byte 
 constexpr int GEMM_THREADS = 256;
 constexpr int GEMM_GROUPS = 8;  // groups of chunks at most
 
-// Tensor memory: a CTA takes at most 256 of the SM's 512 columns, and its
-// registers let two CTAs onto an SM, not three (set_gemm_kernel_attrs checks
-// that), so an allocation never waits (a cluster's CTA that waited for columns
-// held by another cluster could wait for itself).
+// Tensor memory: registers let two CTAs onto an SM, not three
+// (set_gemm_kernel_attrs checks that), and a CTA takes at most half of the SM's
+// 512 columns, or all of its shared memory as well. So an allocation never
+// waits (a cluster's CTA that waited for columns held by another cluster could
+// wait for itself).
 constexpr int GEMM_COLS = 256;
 constexpr size_t SMEM_MAX = 227 * 1024, GEMM_SMEM = SMEM_MAX - 1024;  // (beside the kernel's static bytes)
-__host__ __device__ constexpr uint32_t columns_of(int n) { return n <= 32 ? 32 : n <= 64 ? 64 : n <= 128 ? 128 : 256; }
+__host__ __device__ constexpr uint32_t columns_of(int n)
+{
+    return n <= 32 ? 32 : n <= 64 ? 64 : n <= 128 ? 128 : n <= 256 ? 256 : 512;
+}
 // operand bytes of one stage: tf32 A hi | A lo (fp32 tokens only: bf16 ones are exact in tf32) | B hi | B lo, or
 // bf16 / e4m3 A | B
 __host__ __device__ constexpr uint32_t gemm_stage_bytes(int NT, int precision, bool bf16_tokens)
@@ -212,16 +216,23 @@ __host__ __device__ constexpr uint32_t gemm_stage_bytes(int NT, int precision, b
            : precision == DISC_BF16   ? A_TILE_BYTES / 2 + (uint32_t)NT * GEMM_KC * 2
                                       : A_TILE_BYTES * (bf16_tokens ? 1 : 2) + (uint32_t)NT * GEMM_KC * 8;
 }
+// columns of one CTA's accumulators: with a cluster one per group, else one
+// and the sum of the groups before
+__host__ __device__ constexpr int gemm_columns(int NT, int KS, int groups)
+{
+    return KS > 1 ? groups / KS * NT : groups > 1 ? 2 * NT : NT;
+}
 // The bytes of one CTA: two pipeline stages and the barriers; with a cluster
 // also room for the partial sums over the stages.
 __host__ size_t gemm_smem_bytes(int NT, int precision, bool bf16_tokens, int KS, int groups)
 {
+    if (gemm_columns(NT, KS, groups) > GEMM_COLS) return GEMM_SMEM;
     size_t b = 2 * (size_t)gemm_stage_bytes(NT, precision, bf16_tokens);
     if (KS > 1) b = std::max(b, (size_t)(groups / KS) * NT * GEMM_MT * 4);
     return b + 128;
 }
 static_assert(2 * gemm_stage_bytes(MAX_MASKS, DISC_FP32, false) + 128 <= GEMM_SMEM, "the largest stage pair fits an SM");
-static_assert((size_t)GEMM_COLS * GEMM_MT * 4 + 128 <= GEMM_SMEM, "so do the partial sums of every column");
+static_assert((size_t)GEMM_COLS * GEMM_MT * 4 + 128 <= GEMM_SMEM, "so do the partial sums of a group");
 
 // Test hook: when set, the kernel issues no MMA and no commit, so its bounded
 // waits run out and the frame fails with DISC_ERR_TIMEOUT (nothing is in
@@ -274,11 +285,8 @@ __global__ void __launch_bounds__(GEMM_THREADS, 2) k_pool_gemm(const FrameParams
     const size_t used = max(2 * (size_t)STAGE, KS > 1 ? (size_t)gp * NT * GEMM_MT * 4 : (size_t)0);
     uint64_t* mbar = (uint64_t*)(smem + used);
     uint32_t* tmem_slot = (uint32_t*)(mbar + 2);
-    // A cluster's CTA keeps an accumulator per group.  A CTA that takes a tile
-    // alone keeps one, and the sum of the groups before: in the columns past
-    // it, or (above 128 masks) in the result's place in memory.
-    const bool sums = KS == 1 && gp > 1, tsum = sums && 2 * NT <= GEMM_COLS;
-    const uint32_t ncols = columns_of(KS > 1 ? gp * NT : tsum ? 2 * NT : NT);
+    const bool sums = KS == 1 && gp > 1;
+    const uint32_t ncols = columns_of(gemm_columns(NT, (int)KS, groups));
 
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
@@ -351,13 +359,7 @@ __global__ void __launch_bounds__(GEMM_THREADS, 2) k_pool_gemm(const FrameParams
     auto add_group = [&](int c0, float (&v)[16]) {
         uint32_t r[16], q[16];
         tmem_ld16(tlane + (uint32_t)c0, r);
-        if (tsum) {
-            if (group > 0) tmem_ld16(tlane + (uint32_t)(NT + c0), q);
-        } else {
-#pragma unroll
-            for (int j = 0; j < 16; j++)
-                q[j] = group > 0 && er_in && c0 + j < M ? __float_as_uint(out[(size_t)(c0 + j) * D]) : 0u;
-        }
+        if (group > 0) tmem_ld16(tlane + (uint32_t)(NT + c0), q);
         asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
         tmem_use(r);
         if (group > 0) tmem_use(q);
@@ -389,13 +391,7 @@ __global__ void __launch_bounds__(GEMM_THREADS, 2) k_pool_gemm(const FrameParams
                 for (int c0 = 16 * (warp >> 2); c0 < NT; c0 += 32) {
                     float v[16];
                     add_group(c0, v);
-                    if (tsum) {
-                        tmem_st16(tlane + (uint32_t)(NT + c0), v);
-                    } else if (er_in) {
-#pragma unroll
-                        for (int j = 0; j < 16; j++)
-                            if (c0 + j < M) out[(size_t)(c0 + j) * D] = v[j];
-                    }
+                    tmem_st16(tlane + (uint32_t)(NT + c0), v);
                 }
                 asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
                 fence_before();  // (the next MMAs overwrite the accumulator after the barrier below)
@@ -605,14 +601,16 @@ int launch_pool_gemm(const FrameParams* fps, const BatchScratch& bs, int B, int 
     // a CTA per tile, without the exchange of partial sums (below): us for 1 |
     // 4 | 8 | 16 | 32 Room frames with 8 CTAs per tile 15.5 | 19.3 | 28.7 |
     // 44.1 | 79, with 4 19.4 | 19.4 | 25.5 | 37.8 | 59, with one 39 | 39 | 40 |
-    // 40 | 53.  Above 128 masks two groups' accumulators do not fit, and 8 CTAs
-    // are faster than one up to 16 frames (200 masks: 63 and 78 us).  An SM
-    // partition may be too small or too scattered to hold a cluster.
+    // 40 | 54.  Above 128 masks a CTA of two groups or of a whole tile has an
+    // SM to itself: 200 masks in fp32, 8 | 12 | 16 frames, with 4 CTAs 64 | 65 |
+    // 94, with one 78 | 79 | 79.  An SM partition may be too small or too
+    // scattered to hold a cluster.
     int KS = 1;
     if (clusters) {
-        const bool pairs = groups == 8 && 2 * NT <= GEMM_COLS;
-        if (groups * tiles * B <= (pairs ? 152 : 2 * NT <= GEMM_COLS ? 400 : 800)) KS = groups;
-        else if (pairs && 4 * tiles * B <= 400) KS = 4;
+        const int most = 2 * NT <= GEMM_COLS ? 400 : 304;
+        const bool two = groups == 8 && 2 * (size_t)NT * GEMM_MT * 4 + 128 <= GEMM_SMEM;  // two groups to a CTA
+        if (groups * tiles * B <= (two ? 152 : most)) KS = groups;
+        else if (two && 4 * tiles * B <= most) KS = 4;
     }
     int n = 0;
     if (any[0][0]) { launch_gemm_as<float, DISC_FP32>(fps, bs, tiles, B, NT, KS, groups, st); n++; }
