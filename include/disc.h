@@ -451,15 +451,19 @@ disc_status disc_debug_gemm_stall(int32_t device, int32_t on);
  * kernels per frame of maps with the neighbourhood overlap; how many lanes
  * look one voxel up in the table together (warp-cooperative probing: each
  * round a group of probe_width lanes reads that many consecutive places of the
- * probe sequence); and into how many smaller batches a call whose frames fit
- * one batch is cut, so that each smaller batch's stateless kernels run beside
- * the frame chain of the one before it.  None changes any result. */
+ * probe sequence); how many CTAs (a thread-block cluster) carry one map's
+ * frames in the association kernel; and into how many smaller batches a call
+ * whose frames fit one batch is cut, so that each smaller batch's stateless
+ * kernels run beside the frame chain of the one before it.  None changes any
+ * result. */
 typedef struct {
     int32_t geometry_chunk;  /* frames per geometry launch, 1..32 (default 8) */
     int32_t serial_ctas;     /* serial kernels' CTAs in quarters of the default count, 1..32 (default 4) */
     int32_t probe_width;     /* lanes per key of the voxel-table lookup: 1, 2, 4 or 8 (0 or 1: one lane) */
-    int32_t assoc_cluster;   /* 0, 1, 2, 4 or 8; without effect: one CTA carries a map's frames in the
-                                association kernel (clusters of CTAs measured slower) */
+    int32_t assoc_cluster;   /* CTAs per map in the association kernel, 1, 2, 4 or 8 (capped by what the batch's
+                                maps leave and the device co-schedules): one carries the map's frames, the
+                                others help with frames of many pairs; 0: 8 for batches with a frame of more
+                                than 32 masks (48 when it is alone), else 1; always 1 with serial_sms */
     int32_t batch_split;     /* smaller batches per call that fits one batch: 0 (2 for one map's synchronous
                                 calls of 16 frames or more, else 1: an asynchronous call's frame chain
                                 already overlaps the next call), or 1, 2, 4, 8; each keeps at least 4 frames */
@@ -476,7 +480,7 @@ disc_status disc_map_set_schedule(disc_map* map, const disc_schedule* schedule);
 disc_status disc_group_set_schedule(disc_group* group, const disc_schedule* schedule);
 
 /* Autotuner: times each candidate schedule (geometry_chunk in {2, 4, 8} x
- * probe_width in {1, 2, 4} x assoc_cluster automatic or half of it, then the
+ * probe_width in {1, 2, 4} x assoc_cluster automatic or 4, then the
  * fastest of these with batch_split at each of {1, 2, 4} other than the
  * automatic one) on the sample frames, integrated into fresh maps
  * with the given maps' configurations (created and destroyed here; the given

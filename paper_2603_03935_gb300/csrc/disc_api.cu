@@ -186,7 +186,7 @@ struct Runner {
     int geo_chunk = GEOMETRY_CHUNK;   // frames per back-projection / entries / DBSCAN launch
     int cta_scale = 4;                // serial kernels' CTAs in quarters of the default count
     int probe_width = 1;              // lanes per key of the batch's voxel-table lookup
-    int assoc_cluster = 0;            // accepted, without effect (one CTA per map associates)
+    int assoc_cluster = 0;            // CTAs per map of the association kernel (0: automatic)
     int batch_split = 0;              // smaller batches per call that fits one (0: automatic)
     bool graphs_off = false;
     std::map<long long, BatchGraph> graphs;
@@ -1001,6 +1001,13 @@ constexpr int COMBO_DBSCAN = 1 << 6;
 constexpr int COMBO_ASSOC = 1 << 7;   // some frame's map has a second token grid
 constexpr int COMBO_DILATE = 1 << 8;  // some frame's map takes the neighbourhood overlap: the batch's
                                       // frames run as four kernels each (overlap, score, union, apply)
+constexpr int COMBO_CROWD = 1 << 9;   // some frame may have enough pairs or copies for a cluster to associate
+// Such frames: a cluster's other CTAs take 48 pairs or copies and more. Pairs
+// are left to score once instances changed in the batch, and a frame has a
+// pair or two per mask, so from 33 masks on; a frame alone in its batch only
+// has copies, one per mask at most. (Smaller frames: 8 CTAs are no faster, and
+// 7 of them idle.)
+constexpr int CROWD_MASKS = 32, CROWD_MASKS_ALONE = 48;
 
 // slots [base, base + S) of set k (base > 0: the second half of a batch whose
 // halves wait for their own input copies).  The token kernels (st) and the
@@ -1094,7 +1101,9 @@ int enqueue_serial(Runner& r, int k, int S, int G, int J, int combos, cudaStream
         step.j = 0;
         run_phase(r, PH_LOOKUP, st,
                   [&] { return launch_lookup(dfp, bs, step.view, step.refs, r.ah, S, r.probe_width, st); });
-        run_phase(r, PH_ASSOCIATE, st, [&] { return launch_associate(dfp, bs, step, G, st); });
+        // (on an SM partition, serial_sms, a cluster may have no place)
+        const int cluster = r.green[0] ? 1 : r.assoc_cluster ? r.assoc_cluster : (combos & COMBO_CROWD) ? 8 : 1;
+        run_phase(r, PH_ASSOCIATE, st, [&] { return launch_associate(dfp, bs, step, G, cluster, st); });
         run_phase(r, PH_COMMIT, st, [&] {
             const int n = launch_commit(bs, step, r.ah, G, st);
             cudaMemsetAsync(r.ah.n, 0, sizeof(int32_t), st);  // the hash is empty again
@@ -1113,7 +1122,7 @@ int enqueue_serial(Runner& r, int k, int S, int G, int J, int combos, cudaStream
 
 long long graph_key(int part, int k, int S, int G, int J, int combos)
 {
-    return (((((((long long)S << 11) | G) << 9) | J) << 9 | combos) << 3) | (part << 1) | k;
+    return (((((((long long)S << 11) | G) << 9) | J) << 10 | combos) << 3) | (part << 1) | k;
 }
 
 // A part's kernel sequence captured once per shape and replayed.  A shape
@@ -1525,7 +1534,7 @@ disc_status run_call(Runner& r, std::vector<Work>& w, const AsyncCall* async = n
     if (s != DISC_OK) return s;
     const bool one_graph = r.timing && !r.graphs_off;
     // Batch b + 1's stateless part is enqueued after batch b's serial part:
-    // the serial kernel (one cluster of large-shared-memory CTAs per map)
+    // the serial kernel (a CTA or a cluster per map, each filling an SM)
     // then takes its SMs first and the stateless part fills the rest.
     // (Enqueued before it, the stateless kernels hold every SM and the
     // serial kernel waits for them to drain: measured slower.)
@@ -1571,6 +1580,7 @@ disc_status run_call(Runner& r, std::vector<Work>& w, const AsyncCall* async = n
                 const disc_frame& f = wk.frames[lo + j];
                 px += (uint64_t)f.width * f.height;
                 masks += f.num_masks;
+                if (f.num_masks > (cnt > 1 ? CROWD_MASKS : CROWD_MASKS_ALONE)) combos |= COMBO_CROWD;
                 combos |= 1 << (3 * (f.token_dtype == DISC_TOKENS_BF16) + wk.m->cfg.precision);
                 if (wk.m->cfg.dbscan_eps > 0.0f) combos |= COMBO_DBSCAN;
                 if (wk.m->cfg.assoc_dim > 0) combos |= COMBO_ASSOC;
@@ -1657,14 +1667,14 @@ disc_status run_call(Runner& r, std::vector<Work>& w, const AsyncCall* async = n
             return st;
         }
         if (halves) {
-            st = run_part(r, graph_key(2, k, Sh, 0, 0, combos), ss,
+            st = run_part(r, graph_key(2, k, Sh, 0, 0, combos & ~COMBO_CROWD), ss,
                           [&] { return enqueue_stateless(r, k, Sh, combos, ss); });
             if (st == DISC_OK) st = cuda_status(cudaStreamWaitEvent(ss, r.ev_in_half[k], 0));
             if (st == DISC_OK)
-                st = run_part(r, graph_key(3, k, S - Sh, Sh, 0, combos), ss,  // keyed by its first slot too
+                st = run_part(r, graph_key(3, k, S - Sh, Sh, 0, combos & ~COMBO_CROWD), ss,  // keyed by its first slot too
                               [&] { return enqueue_stateless(r, k, S - Sh, combos, ss, Sh); });
         } else {
-            st = run_part(r, graph_key(0, k, S, 0, 0, combos), ss,
+            st = run_part(r, graph_key(0, k, S, 0, 0, combos & ~COMBO_CROWD), ss,
                           [&] { return enqueue_stateless(r, k, S, combos, ss); });
         }
         if (st == DISC_OK && copied) st = cuda_status(cudaEventRecord(r.ev_in_free[k], ss));
@@ -1724,7 +1734,7 @@ disc_status run_call(Runner& r, std::vector<Work>& w, const AsyncCall* async = n
                 st = room_check(r, k, G, J, w, P.gl, hrefs, sr);
             }
             if (st == DISC_OK)
-                st = run_part(r, graph_key(1, k, S, G, J, P.combos & COMBO_DILATE), sr,
+                st = run_part(r, graph_key(1, k, S, G, J, P.combos & (COMBO_DILATE | COMBO_CROWD)), sr,
                               [&] { return enqueue_serial(r, k, S, G, J, P.combos, sr); });
         }
         // the batch's counters, in slot order, to the call's history
@@ -2460,18 +2470,13 @@ disc_status autotune(Runner& r, const std::vector<const disc_map_config*>& cfgs,
         return best;
     };
     // frames per geometry launch x lanes per key of the lookup x CTAs per
-    // map of the association kernel (automatic, or the next smaller cluster),
-    // the automatic batch split
+    // map of the association kernel (automatic, or 4 where the maps leave room
+    // for more than one), the automatic batch split
     for (int geo : {4, 2, 8})  // the default first
         for (int pw : {1, 2, 4})
-            for (int ac : {0, -1}) {
-                disc_schedule cand{geo, r.cta_scale, pw, ac, 0};
-                if (ac < 0) {  // half the automatic cluster of these maps
-                    int c = 1;
-                    while (c * 2 <= 8 && (c * 2) * (int)cfgs.size() <= 152) c *= 2;
-                    if (c == 1) continue;
-                    cand.assoc_cluster = c / 2;
-                }
+            for (int ac : {0, 4}) {
+                if (ac > 0 && cfgs.size() > 32) continue;
+                const disc_schedule cand{geo, r.cta_scale, pw, ac, 0};
                 const double ms = time_schedule(cand);
                 if (geo == 4 && pw == 1 && ac == 0) rep.default_ms = ms;
             }

@@ -602,6 +602,10 @@ __device__ __forceinline__ int dsm_ld32(unsigned a)
     asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(a) : "memory");
     return v;
 }
+__device__ __forceinline__ void dsm_st32(unsigned a, int v)
+{
+    asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(a), "r"(v) : "memory");
+}
 // every thread of every CTA of the cluster; shared-memory and global writes
 // before it are visible to the cluster after it (release / acquire)
 __device__ __forceinline__ void cluster_sync()

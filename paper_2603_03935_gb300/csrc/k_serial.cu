@@ -1507,6 +1507,7 @@ struct __align__(16) AssocShared {
     unsigned want[MAX_MASKS / 32];          // segments that open an instance
     int err, ncopies;                       // the frame's status and embedding copies
     int4 meta[ASSOC_FRAMES];                // the first frames' slot, n_pre, own error and masks
+    int4 job;                               // for the cluster's other CTAs: kind, items, frame slot
     int ne, nlive, nloc, nroots, np, nsc, border, ovf, multi, ncopy, merges, next, merged_any, all_changed;
 };
 constexpr size_t ASSOC_SMEM = sizeof(AssocShared);
@@ -1565,6 +1566,72 @@ __global__ void __launch_bounds__(256) k_gates(const FrameParams* fps, BatchScra
     }
 }
 
+// ---- what the other CTAs of a map's cluster do for its leader ---------------------
+// They wait at the cluster's barrier for a job, read it and its items from the
+// leader's shared memory, and meet the leader at the barrier again when it is
+// done.
+constexpr int JOB_END = 0, JOB_SCORE = 1, JOB_COPY = 2, JOB_PAIRS = 3;
+constexpr int JOB_MIN = 48;  // items that are worth one: three rounds of the leader's warps
+constexpr int LIVE_EDGE = 1 << 30, LIVE_BORDER = 1 << 29;  // what became of a pair, in its live word
+
+// Pairs w, w + nw, ... of the leader's n live pairs through the cosine gate.
+__device__ __noinline__ void job_score(const AssocShared& A, const FrameParams& fp, const GateFeatures& gf,
+                                       const Instances& inst, int n, int w, int nw)
+{
+    const unsigned live = dsm_map(A.live, 0);
+    for (int q = w; q < n; q += nw) {
+        const int x = dsm_ld32(live + 8u * q), k = dsm_ld32(live + 8u * q + 4u);
+        int border = 0;
+        const bool edge = warp_cosine_gate(fp, gf, inst, x & 511, k, &border);
+        if ((threadIdx.x & 31) == 0)
+            dsm_st32(live + 8u * q, x | (edge ? LIVE_EDGE : 0) | (border ? LIVE_BORDER : 0));
+    }
+}
+
+// One warp writes the embedding (and, with a second grid, the association
+// feature) that copy c of the frame names, and its scoring copy.
+__device__ __forceinline__ void copy_embedding(const MapRefs& R, const Scratch& sc, const Scratch& va, int D, int c)
+{
+    const Instances& inst = R.inst;
+    const int lane = threadIdx.x & 31;
+    const int src = R.ss.copy_src[c], dst = R.ss.copy_dst[c];
+    const float* from = src >= 0 ? inst.E + (size_t)src * D : sc.Ecan + (size_t)(-src - 1) * D;
+    if (inst.A) {
+        const int Da = inst.Da;
+        const float* fa = src >= 0 ? inst.A + (size_t)src * Da : va.Ecan + (size_t)(-src - 1) * Da;
+        copy_row(from, inst.E + (size_t)dst * D, nullptr, D, lane);
+        copy_row(fa, inst.A + (size_t)dst * Da, inst.Eb ? inst.Eb + (size_t)dst * Da : nullptr, Da, lane);
+        if (inst.E8) e4m3_copy_row(fa, Da, inst.E8 + (size_t)dst * Da, inst.Er + dst);
+    } else {
+        copy_row(from, inst.E + (size_t)dst * D, inst.Eb ? inst.Eb + (size_t)dst * D : nullptr, D, lane);
+        if (inst.E8) e4m3_copy_row(from, D, inst.E8 + (size_t)dst * D, inst.Er + dst);
+    }
+}
+
+__device__ __noinline__ void assoc_help(const AssocShared& A, const MapRefs& R, const FrameParams* fps,
+                                        const BatchScratch& bs, const BatchScratch& view, int rank, int nranks)
+{
+    const int wid = threadIdx.x >> 5, nw = ASSOC_THREADS >> 5;
+    const unsigned job = dsm_map(&A.job, 0);
+    while (true) {
+        cluster_sync();  // the leader has a job
+        const int kind = dsm_ld32(job), n = dsm_ld32(job + 4), slot = dsm_ld32(job + 8);
+        if (kind != JOB_END) {
+            const FrameParams& fp = fps[slot];
+            const Scratch sc = bs.frame(slot), va = view.frame(slot);
+            if (kind == JOB_PAIRS) {  // (past the shared capacities: the pairs of the map's global hash)
+                phase_score(fp, sc, va, R.ss, R.inst, rank * nw + wid, nranks * nw);
+            } else if (kind == JOB_SCORE) {
+                job_score(A, fp, gate_features(fp, sc, va, R.inst), R.inst, n, rank * nw + wid, nranks * nw);
+            } else {  // (the leader goes on to the next frame meanwhile)
+                for (int c = (rank - 1) * nw + wid; c < n; c += (nranks - 1) * nw) copy_embedding(R, sc, va, fp.D, c);
+            }
+        }
+        cluster_sync();  // it is done, and the leader's shared memory read
+        if (kind == JOB_END) return;
+    }
+}
+
 // One CTA per map of the batch walks the map's frames in order.  Per frame:
 //   (1) every item (its label resolved to the root as of now) adds to its
 //       (segment, root) pair in the shared pair hash;
@@ -1587,13 +1654,20 @@ __global__ void __launch_bounds__(256) k_gates(const FrameParams* fps, BatchScra
 // passing pair scored between two cluster barriers, the union in fourteen
 // block barriers) and 11.8 with k_gates and this union: a cluster barrier that
 // orders global memory costs 1.2 us and empties the L1, a block barrier 0.03
-// us, and with the gates taken beforehand few pairs are left to share.
+// us.  So one CTA, the leader, walks the frames, and the others of a cluster
+// only wait for jobs: the pairs left to score and the embeddings to copy where
+// a frame has more than JOB_MIN of them (the copies while the leader goes on to
+// the next frame's steps (1) and (2)).  Frames of 240 masks, us per frame, one
+// CTA | 8 with jobs: views that stay alike 42 | 18, views that improve 72 | 25,
+// masks that drift over the instances 88 | 26; 100 masks 23 | 14, 32 | 19,
+// 41 | 18; 40 masks 14.8 | 14.6, 17.2 | 17.1, 19.5 | 14.6.  Spills about 500
+// bytes a thread at 128 registers, the most that 512 threads can have.
 __global__ void __launch_bounds__(ASSOC_THREADS, 1) k_associate(const FrameParams* fps, BatchScratch bs,
                                                                 SerialStep st)
 {
     extern __shared__ __align__(16) unsigned char assoc_smem[];
     AssocShared& A = *(AssocShared*)assoc_smem;
-    const int g = blockIdx.x;
+    const int g = blockIdx.y, rank = blockIdx.x, nranks = gridDim.x;  // a cluster spans the grid's x
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     constexpr int NT = ASSOC_THREADS;
     // the map's table pointers, in shared memory: read there, they are never
@@ -1602,6 +1676,23 @@ __global__ void __launch_bounds__(ASSOC_THREADS, 1) k_associate(const FrameParam
     static_assert(sizeof(MapRefs) % 8 == 0, "copied in 8-byte words");
     for (int i = tid; i < (int)(sizeof(MapRefs) / 8); i += NT)
         ((unsigned long long*)&s_refs)[i] = ((const unsigned long long*)&st.refs[g])[i];
+    if (rank > 0) {  // uniform per block
+        __syncthreads();
+        assoc_help(A, s_refs, fps, bs, st.view, rank, nranks);
+        return;
+    }
+    // a job for the cluster's other CTAs, and the wait until the last one is done
+    bool helping = false;
+    auto finish = [&] {
+        if (helping) cluster_sync();
+        helping = false;
+    };
+    auto give = [&](int kind, int n, int slot) {
+        finish();
+        if (tid == 0) A.job = make_int4(kind, n, slot, 0);
+        cluster_sync();
+        helping = true;
+    };
     for (int j = tid; j < min(st.J, ASSOC_FRAMES); j += NT) {
         const int slot = st.slot_of[g * st.J + j];
         A.meta[j] = slot < 0 ? make_int4(-1, 0, 0, 0)
@@ -1757,8 +1848,33 @@ __global__ void __launch_bounds__(ASSOC_THREADS, 1) k_associate(const FrameParam
                     if (border) atomicAdd(&A.border, border);
                 }
                 __syncthreads();
+            }
+            // the copies of the frame before, where the other CTAs make them:
+            // the gates read embeddings, step (3) writes the copy lists
+            finish();
+            if (!global_pairs) {
                 const int nlive = A.nlive;
-                if (nlive > 0) {
+                if (nranks > 1 && nlive > JOB_MIN) {
+                    give(JOB_SCORE, nlive, slot);
+                    job_score(A, fp, gate_features(fp, sc, st.view.frame(slot), inst), inst, nlive, wid,
+                              nranks * (NT >> 5));
+                    finish();
+                    int border = 0;
+                    for (int q = tid; q < nlive; q += NT) {
+                        const int x = A.live[q].x, k = A.live[q].y, h = (x >> 9) & (ARH - 1);
+                        if (x & LIVE_BORDER) border++;
+                        if (!(x & LIVE_EDGE)) continue;
+                        const int e = atomicAdd(&A.ne, 1);
+                        if (e < ASSOC_EDGES) {
+                            A.em[e] = x & 511;
+                            A.eh[e] = h;
+                        }
+                        claim_root(A, h, k, inst.count[k], inst.Q[k], inst.n_obs[k]);
+                    }
+                    border = warp_sum(border);
+                    if (lane == 0 && border) atomicAdd(&A.border, border);
+                    __syncthreads();
+                } else if (nlive > 0) {
                     const GateFeatures gf = gate_features(fp, sc, st.view.frame(slot), inst);
                     int rescored = 0;
                     for (int q = wid; q < nlive; q += NT >> 5) {
@@ -1908,8 +2024,11 @@ __global__ void __launch_bounds__(ASSOC_THREADS, 1) k_associate(const FrameParam
                         add_pair(sc, R.ss, ((key >> 33) << 32) | (unsigned)find_root(inst.parent, lab),
                                  sc.icnt[i] & ITEM_COUNT);
                 }
-                if (!block_read(&sc.ctr->err))
-                    phase_score(fp, sc, st.view.frame(slot), R.ss, inst, wid, NT >> 5);
+                if (!block_read(&sc.ctr->err)) {
+                    if (nranks > 1) give(JOB_PAIRS, 0, slot);
+                    phase_score(fp, sc, st.view.frame(slot), R.ss, inst, wid, nranks * (NT >> 5));
+                    finish();
+                }
                 if (!block_read(&sc.ctr->err)) phase_union(fp, sc, R.ss, inst, R.next_id, R.ss.ureg);
                 // empty the global pair hash
                 __syncthreads();
@@ -1949,24 +2068,14 @@ __global__ void __launch_bounds__(ASSOC_THREADS, 1) k_associate(const FrameParam
         // (4) the winners' embeddings; on the global path also the new voxels
         //     into the counts
         if (!A.err) {
-            const int D = fp.D;
             const int nc = A.ncopies;
-            // from the last warp down: the first warps take the next frame's
-            // items, so the two run side by side
-            for (int c = (NT >> 5) - 1 - wid; c < nc; c += NT >> 5) {
-                const int src = R.ss.copy_src[c], dst = R.ss.copy_dst[c];
-                const float* from = src >= 0 ? inst.E + (size_t)src * D : sc.Ecan + (size_t)(-src - 1) * D;
-                if (inst.A) {
-                    const Scratch va = st.view.frame(slot);
-                    const int Da = inst.Da;
-                    const float* fa = src >= 0 ? inst.A + (size_t)src * Da : va.Ecan + (size_t)(-src - 1) * Da;
-                    copy_row(from, inst.E + (size_t)dst * D, nullptr, D, lane);
-                    copy_row(fa, inst.A + (size_t)dst * Da, inst.Eb ? inst.Eb + (size_t)dst * Da : nullptr, Da, lane);
-                    if (inst.E8) e4m3_copy_row(fa, Da, inst.E8 + (size_t)dst * Da, inst.Er + dst);
-                } else {
-                    copy_row(from, inst.E + (size_t)dst * D, inst.Eb ? inst.Eb + (size_t)dst * D : nullptr, D, lane);
-                    if (inst.E8) e4m3_copy_row(from, D, inst.E8 + (size_t)dst * D, inst.Er + dst);
-                }
+            if (nranks > 1 && nc > JOB_MIN) {
+                give(JOB_COPY, nc, slot);
+            } else {
+                // from the last warp down: the first warps take the next
+                // frame's items, so the two run side by side
+                const Scratch va = st.view.frame(slot);
+                for (int c = (NT >> 5) - 1 - wid; c < nc; c += NT >> 5) copy_embedding(R, sc, va, fp.D, c);
             }
             if (!united && !blocked)
                 for (int m = tid; m < M; m += NT) {
@@ -1980,6 +2089,10 @@ __global__ void __launch_bounds__(ASSOC_THREADS, 1) k_associate(const FrameParam
         }
     }
     if (tid == 0) st.merged[g] = A.merged_any;
+    if (nranks > 1) {
+        give(JOB_END, 0, 0);
+        finish();
+    }
 }
 
 // After the batch's frames: every voxel of the absent-voxel hash whose first
@@ -2129,13 +2242,41 @@ int launch_lookup(const FrameParams* fps, const BatchScratch& bs, const BatchScr
 
 size_t union_region_bytes_full() { return UNION_SMEM; }
 
-int launch_associate(const FrameParams* fps, const BatchScratch& bs, const SerialStep& st, int G, cudaStream_t s)
+// A CTA of this kernel fills an SM's registers, so the clusters of a batch's
+// maps together leave most SMs to the kernels beside them. 16 maps of 240
+// masks, us per frame of the call (association alone): one CTA per map 25.1
+// (2.8), clusters of 8, 128 CTAs, 25.3 (2.2), of 4 24.5 (1.5), of 2 24.9 (2.1).
+constexpr int ASSOC_CTAS = 64;
+// CTAs per map of the association kernel that the device can place together
+static int g_assoc_max_cluster = 1;  // set once by set_serial_kernel_attrs
+
+static cudaLaunchConfig_t assoc_config(int G, int cluster, size_t smem, cudaLaunchAttribute* at, cudaStream_t s)
 {
+    cudaLaunchConfig_t cfg = {};
+    at->id = cudaLaunchAttributeClusterDimension;
+    at->val.clusterDim.x = cluster;
+    at->val.clusterDim.y = 1;
+    at->val.clusterDim.z = 1;
+    cfg.gridDim = dim3(cluster, G);
+    cfg.blockDim = dim3(ASSOC_THREADS);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cfg;
+}
+
+int launch_associate(const FrameParams* fps, const BatchScratch& bs, const SerialStep& st, int G, int cluster,
+                     cudaStream_t s)
+{
+    int c = 1;
+    while (2 * c <= std::min(cluster, g_assoc_max_cluster) && 2 * c * G <= ASSOC_CTAS) c *= 2;
     // A CTA of few maps keeps its SM to itself (a row of dependent steps that
     // shares its issue slots with stateless blocks runs 1.4 times as long):
     // it asks for all of the SM's shared memory.
-    const size_t smem = G <= 4 ? ASSOC_SMEM_ALONE : ASSOC_SMEM;
-    k_associate<<<G, ASSOC_THREADS, smem, s>>>(fps, bs, st);
+    cudaLaunchAttribute at;
+    const cudaLaunchConfig_t cfg = assoc_config(G, c, G <= 4 ? ASSOC_SMEM_ALONE : ASSOC_SMEM, &at, s);
+    cudaLaunchKernelEx(&cfg, k_associate, fps, bs, st);
     return 1;
 }
 
@@ -2151,6 +2292,16 @@ cudaError_t set_serial_kernel_attrs()
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(k_associate, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ASSOC_SMEM_ALONE);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k_overlap, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)OV_SMEM);
+    for (int c = 8; e == cudaSuccess && c > 1; c /= 2) {
+        cudaLaunchAttribute at;
+        const cudaLaunchConfig_t cfg = assoc_config(1, c, ASSOC_SMEM_ALONE, &at, nullptr);
+        int n = 0;
+        if (cudaOccupancyMaxActiveClusters(&n, k_associate, &cfg) == cudaSuccess && n > 0) {
+            g_assoc_max_cluster = c;
+            break;
+        }
+        cudaGetLastError();
+    }
     return e;
 }
 

@@ -83,7 +83,9 @@ int launch_serial_step(const FrameParams* fps, const BatchScratch& bs, const Ser
 // as the batch starts)
 int launch_lookup(const FrameParams* fps, const BatchScratch& bs, const BatchScratch& view, const MapRefs* refs,
                   const AbsentHash& ah, int S, int probe_width, cudaStream_t st);
-int launch_associate(const FrameParams* fps, const BatchScratch& bs, const SerialStep& st, int G, cudaStream_t s);
+// cluster: CTAs per map at most (1, 2, 4 or 8)
+int launch_associate(const FrameParams* fps, const BatchScratch& bs, const SerialStep& st, int G, int cluster,
+                     cudaStream_t s);
 int launch_commit(const BatchScratch& bs, const SerialStep& st, const AbsentHash& ah, int G, cudaStream_t s);
 // bytes of the union region a map keeps in global memory (SerialScratch::ureg)
 size_t union_region_bytes_full();
