@@ -894,7 +894,7 @@ disc_status ensure_instance_room(disc_map* m, int64_t incoming, cudaStream_t st)
     return DISC_OK;
 }
 
-constexpr size_t kKeepQueryBytes = 64 << 20;  // query scratch a map keeps between calls
+constexpr size_t kKeepQueryBytes = 64 << 20;  // query scratch that an export may leave with the map
 
 // device scratch of at least `bytes` for query calls (no allocation once it
 // is large enough: a freed buffer would synchronise the device each call)
@@ -2618,6 +2618,36 @@ static disc_status export_voxels_host(disc_map* m, uint64_t* keys, int32_t* ids,
     return DISC_OK;
 }
 
+// An export's device buffer: the map's query scratch up to what that keeps
+// between calls (or holds anyway), a buffer of its own above, which goes back
+// however the call ends.
+struct ExportBuffer {
+    disc_map* m;
+    unsigned char* own = nullptr;
+    size_t cap = 0;
+    unsigned char* get(size_t bytes)
+    {
+        drop();
+        unsigned char* p;
+        if (bytes <= m->qcap || std::max(bytes, 2 * m->qcap) <= kKeepQueryBytes) {  // (it doubles as it grows)
+            p = query_scratch(m, bytes);
+            cap = m->qcap;
+        } else {
+            p = own = m->mem.get<unsigned char>(bytes);
+            cap = own ? bytes : 0;
+            if (!own) m->mem.failed = false;
+        }
+        return p;
+    }
+    void drop()
+    {
+        if (own) m->mem.release(own, cap);
+        own = nullptr;
+        cap = 0;
+    }
+    ~ExportBuffer() { drop(); }
+};
+
 disc_status disc_map_export_voxels(disc_map* m, uint64_t* keys, int32_t* ids, int64_t cap)
 {
     if (!m || (cap > 0 && (!keys || !ids))) return DISC_ERR_INVALID_ARG;
@@ -2627,16 +2657,20 @@ disc_status disc_map_export_voxels(disc_map* m, uint64_t* keys, int32_t* ids, in
     const uint64_t n = read_used(m, m->stream);
     if ((int64_t)n > cap) return DISC_ERR_INVALID_ARG;
     if (n == 0) return DISC_OK;
-    // The bitmap over the voxels' box pays up to 512 MB, and while it has no
-    // more than 4096 bits per voxel (its passes then move no more than a few
-    // times what the table holds).
+    // The bitmap over the voxels' box takes up to 512 MB, and no more than 4096
+    // bits per voxel: up to there its passes cost little beside the host sort,
+    // and the bound keeps a small map from asking for much memory.  785,000
+    // voxels at 82 | 640 | 1,500 | 5,100 bits each: 0.5 | 0.9 | 1.0 | 1.5 ms
+    // (4.9 the first time, with its allocation), by the host sort 48; 6 million
+    // at 82 | 640: 3.6 | 3.8 (14, with an allocation), by the host sort 425.
     constexpr uint64_t kMaxBits = 1ull << 32;
     if (n >= (1ull << 31) || m->vt.mask >= (1ull << 32)) return export_voxels_host(m, keys, ids, cap);
     cudaStream_t st = m->stream;
     ExportScratch es{};
     const size_t b_head = 256, b_list = align256(sizeof(unsigned) * n);
     const size_t b_keys = align256(sizeof(unsigned long long) * n), b_ids = align256(sizeof(int32_t) * n);
-    unsigned char* base = query_scratch(m, b_head + b_list);
+    ExportBuffer buf{m};
+    unsigned char* base = buf.get(b_head + b_list);
     if (!base) return export_voxels_host(m, keys, ids, cap);
     es.head = (int*)base;
     es.list = (unsigned*)(base + b_head);
@@ -2662,8 +2696,8 @@ disc_status disc_map_export_voxels(disc_map* m, uint64_t* keys, int32_t* ids, in
     const size_t b_bits = align256(128 * (size_t)es.groups), b_before = align256(sizeof(int) * (size_t)es.groups);
     const size_t b_spans = align256(sizeof(int) * (size_t)spans);
     const size_t all = b_head + b_list + b_keys + b_ids + b_bits + b_before + b_spans;
-    if (all > m->qcap) {  // a larger buffer: the list is made again in it
-        base = query_scratch(m, all);
+    if (all > buf.cap) {  // a larger buffer: the list is made again in it
+        base = buf.get(all);
         if (!base) return export_voxels_host(m, keys, ids, cap);
         es.head = (int*)base;
         es.list = (unsigned*)(base + b_head);
@@ -2681,13 +2715,7 @@ disc_status disc_map_export_voxels(disc_map* m, uint64_t* keys, int32_t* ids, in
     CK(cudaMemcpyAsync(keys, es.keys, sizeof(uint64_t) * n, cudaMemcpyDeviceToHost, st));
     CK(cudaMemcpyAsync(ids, es.ids, sizeof(int32_t) * n, cudaMemcpyDeviceToHost, st));
     CK(cudaGetLastError());
-    const disc_status s = cuda_status(cudaStreamSynchronize(st));
-    if (m->qcap > kKeepQueryBytes) {  // a large map's scratch goes back
-        m->mem.release(m->qscratch, m->qcap);
-        m->qscratch = nullptr;
-        m->qcap = 0;
-    }
-    return s;
+    return cuda_status(cudaStreamSynchronize(st));
 }
 
 disc_status disc_map_export_assoc(disc_map* m, float* A, int32_t cap)

@@ -127,3 +127,40 @@ def test_instance_table_read_again_and_again(dim, per):
         once.close()
     again.close()
     empty.close()
+
+
+def test_a_large_export_gives_its_memory_back():
+    # 17 million voxels too far apart for the bitmap (the host sorts them): the list of their slots goes back; and an
+    # export beside a large query scratch leaves that as it is
+    import torch
+    from paper_2603_03935_gb300 import DiscMap, device_frame
+    dev = torch.device("cuda:0")
+    gen = torch.Generator(device=dev).manual_seed(2)
+    width, height = 2048, 1536
+    gmap = DiscMap(voxel_size=0.02, embed_dim=16, patch_h=4, patch_w=4, max_width=width, max_height=height, max_masks=2,
+                   min_mask_pixels=1, voxel_capacity=1 << 26, max_load=0.5, instance_capacity=64, z_min=0.1, z_max=1e4,
+                   batch_frames=1)
+    labels = torch.ones(height, width, dtype=torch.int16, device=dev)
+    tokens = torch.randn(16, 16, device=dev)
+    intr = (1000.0, 1000.0, width / 2.0, height / 2.0)
+
+    def frame():
+        depth = 500.0 * (0.2 + torch.rand(height, width, device=dev, generator=gen))
+        gmap.integrate(device_frame(depth, labels, tokens, np.eye(4), intr, 1))
+
+    def export():
+        n, _ = gmap.counts()
+        keys, ids = gmap.voxels()
+        assert len(keys) == n and (np.diff(keys.astype(np.int64)) > 0).all() and (ids >= 0).all()
+
+    for _ in range(6):
+        frame()
+    assert gmap.counts()[0] > 17e6
+    before = gmap.device_bytes()  # no query scratch yet; an export may leave 64 MB of it
+    export()
+    assert gmap.device_bytes() <= before + (64 << 20)
+    gmap.query_points(np.zeros((9_000_000, 3), np.float32))  # 144 MB of query scratch
+    held = gmap.device_bytes()
+    export()
+    assert gmap.device_bytes() == held
+    gmap.close()
