@@ -463,7 +463,7 @@ typedef struct {
     int32_t assoc_cluster;   /* CTAs per map in the association kernel, 1, 2, 4 or 8 (capped by what the batch's
                                 maps leave and the device co-schedules): one carries the map's frames, the
                                 others help with frames of many pairs; 0: 8 for batches with a frame of more
-                                than 32 masks (48 when it is alone), else 1; always 1 with serial_sms */
+                                than 48 masks, else 1; always 1 with serial_sms */
     int32_t batch_split;     /* smaller batches per call that fits one batch: 0 (2 for one map's synchronous
                                 calls of 16 frames or more, else 1: an asynchronous call's frame chain
                                 already overlaps the next call), or 1, 2, 4, 8; each keeps at least 4 frames */

@@ -1002,12 +1002,11 @@ constexpr int COMBO_ASSOC = 1 << 7;   // some frame's map has a second token gri
 constexpr int COMBO_DILATE = 1 << 8;  // some frame's map takes the neighbourhood overlap: the batch's
                                       // frames run as four kernels each (overlap, score, union, apply)
 constexpr int COMBO_CROWD = 1 << 9;   // some frame may have enough pairs or copies for a cluster to associate
-// Such frames: a cluster's other CTAs take 48 pairs or copies and more. Pairs
-// are left to score once instances changed in the batch, and a frame has a
-// pair or two per mask, so from 33 masks on; a frame alone in its batch only
-// has copies, one per mask at most. (Smaller frames: 8 CTAs are no faster, and
-// 7 of them idle.)
-constexpr int CROWD_MASKS = 32, CROWD_MASKS_ALONE = 48;
+// Such frames: a cluster's other CTAs take 48 pairs or copies and more, and a
+// frame has one or two of them per mask. (The 40 masks of Room frames: 8 CTAs
+// associate drifting views faster, 14.6 us a frame for 19.5, views that stay
+// alike no faster, and their 7 SMs cost the stateless kernels beside them 2 %.)
+constexpr int CROWD_MASKS = 48;
 
 // slots [base, base + S) of set k (base > 0: the second half of a batch whose
 // halves wait for their own input copies).  The token kernels (st) and the
@@ -1580,7 +1579,7 @@ disc_status run_call(Runner& r, std::vector<Work>& w, const AsyncCall* async = n
                 const disc_frame& f = wk.frames[lo + j];
                 px += (uint64_t)f.width * f.height;
                 masks += f.num_masks;
-                if (f.num_masks > (cnt > 1 ? CROWD_MASKS : CROWD_MASKS_ALONE)) combos |= COMBO_CROWD;
+                if (f.num_masks > CROWD_MASKS) combos |= COMBO_CROWD;
                 combos |= 1 << (3 * (f.token_dtype == DISC_TOKENS_BF16) + wk.m->cfg.precision);
                 if (wk.m->cfg.dbscan_eps > 0.0f) combos |= COMBO_DBSCAN;
                 if (wk.m->cfg.assoc_dim > 0) combos |= COMBO_ASSOC;
