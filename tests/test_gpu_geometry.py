@@ -1,6 +1,8 @@
 """Back-projection records and their gathering into (segment, voxel) entries,
 at the edges of the partitions: every frame's voxel sets, normals (S_angle)
 and counters equal the oracle's bit for bit."""
+import ctypes
+
 import numpy as np
 import pytest
 
@@ -192,3 +194,55 @@ def test_holes_do_not_cost_more_than_the_pixels_they_replace(kind):
         ms.append(best)
         gmap.close()
     assert ms[1] < 2 * ms[0], ms
+
+
+@pytest.mark.parametrize("probe_width", [1, 2, 4, 8])
+@pytest.mark.parametrize("capacity,first,more,place", [(64, 20, 12, 5), (256, 100, 60, 0), (512, 250, 90, 7)])
+def test_more_voxels_of_one_place_than_groups(capacity, first, more, place, probe_width):
+    """Voxels picked by the table's own hash: more of them have their home in one place of their groups of eight than
+    there are groups, so the probe sequence has to go once round and on to the next place; then the table grows."""
+    import torch
+    from paper_2603_03935_gb300 import DiscMap, binding, device_frame
+    dev = torch.device("cuda:0")
+    rng = np.random.default_rng(capacity)
+    cfg = dict(voxel_size=0.02, embed_dim=DIM, patch_h=GRID[0], patch_w=GRID[1], max_width=W, max_height=H, max_masks=8,
+               min_mask_pixels=1, voxel_capacity=capacity, max_load=0.7, instance_capacity=64, z_min=0.1, z_max=10.0,
+               eps=1e-6, tau_cos=0.75, lambda_size=3.3, ov_num=1, ov_den=5)
+    gmap, omap = DiscMap(**cfg), oracle.OracleMap(**common.to_oracle_cfg(cfg))
+    gmap.set_schedule(probe_width=probe_width)
+    cx, cy = W / 2 - 0.25, H / 2 - 0.25  # 0.04 m from pixel to pixel, each in the middle of its voxel
+    u, v = np.meshgrid(np.arange(W), np.arange(H))
+    kx, ky = (np.floor((a + 0.5 - c) * 0.04 / 0.02).astype(np.int64) + (1 << 17) for a, c in ((u, cx), (v, cy)))
+    keys = (kx << 36) | (ky << 18) | (int(2.01 / 0.02) + (1 << 17))
+    low = (1 << 36) | (1 << 18) | 1
+
+    def home(key):  # the key's place in its group: parities, permuted by the block's hash
+        local = ((key >> 34) & 4) | ((key >> 17) & 2) | (key & 1)
+        return local ^ (_mix64(key & ~low) >> 61)
+
+    same = np.array([home(int(k)) == place for k in keys.reshape(-1)])
+    pick = rng.permutation(np.where(same)[0])
+    assert len(pick) > first and first > capacity // 8
+    labels = (np.arange(H)[:, None] // 24 * 4 + np.arange(W)[None, :] // 16 + 1).astype(np.uint16)
+    tokens = rng.normal(size=(GRID[0] * GRID[1], DIM)).astype(np.float32)
+    pose = np.eye(4)
+    pose[2, 3] = 0.01
+    probes = []
+    for take in (pick[:first], pick[first // 2:first], pick[first // 3:first + more]):
+        depth = np.zeros(H * W, np.float32)
+        depth[take] = 2.0
+        depth = depth.reshape(H, W)
+        st = gmap.integrate(device_frame(torch.from_numpy(depth).to(dev), torch.from_numpy(labels.view(np.int16)).to(dev),
+                                         torch.from_numpy(tokens).to(dev), pose, (50.0, 50.0, cx, cy), 8))
+        o = omap.integrate(depth, labels, tokens, pose, (50.0, 50.0, cx, cy), 8)
+        common.compare_frame(st, gmap.last_frame(), o, ctx=f"{len(take)} voxels of {capacity} slots")
+        probes.append(st["max_probe"])
+    got, ids = gmap.voxels()
+    assert set(got.tolist()) == set(keys.reshape(-1)[pick[:first + more]].tolist())
+    assert probes[1] >= capacity // 8  # found past a whole round
+    now = binding.Config()
+    assert binding.lib().disc_map_get_config(gmap._h, ctypes.byref(now)) == 0 and now.voxel_capacity > capacity
+    common.compare_maps(gmap, omap, ctx="one place")
+    k = [((got >> np.uint64(s)).astype(np.int64) & 0x3ffff) - (1 << 17) for s in (36, 18, 0)]
+    assert np.array_equal(gmap.query_points(((np.stack(k, 1) + 0.5) * 0.02).astype(np.float32)), ids)
+    gmap.close()
