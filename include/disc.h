@@ -422,7 +422,7 @@ disc_status disc_map_load(const char* path, const disc_map_config* cfg_override,
  *   Dp, cosg     [P] device memory, written;
  *   cuda_stream  cudaStream_t of the current device (NULL = default stream).
  * Limits: P <= 16384, D <= 4096; larger sizes return DISC_ERR_INVALID_ARG.
- * Its working set (~450 KB) is a file-scope __device__ array that every GPU
+ * Its working set (~260 KB) is a file-scope __device__ array that every GPU
  * loading the library holds until the process exits; every call on a GPU
  * shares it, so calls whose GPU work overlaps race.  The first call on each
  * device looks up that array's device address (the current device must be

@@ -174,7 +174,7 @@ __device__ __forceinline__ T warp_sum(T v)
 // ---------------------------------------------------------------------------
 // Device state.  Plain structs of device pointers, passed to kernels by value.
 
-struct VoxelTable {              // open addressing, linear probing
+struct VoxelTable {              // open addressing by groups of eight slots (vt_home, vt_next)
     unsigned long long* keys;    // EMPTY_KEY = free
     int32_t* labels;             // instance id at insertion (resolve via parent)
     unsigned long long mask;     // capacity - 1 (capacity is a power of two)

@@ -45,7 +45,7 @@ unsigned char* g_addr[MAX_DEVICES] = {};
 
 }  // namespace
 
-// The working set: ~450 KB, one copy per GPU that loads the library.
+// The working set: ~260 KB, one copy per GPU that loads the library.
 static __device__ __align__(256) unsigned char g_token_scratch[STATIC_BYTES];
 
 // The working set's counters and sums to zero and the call's parameters

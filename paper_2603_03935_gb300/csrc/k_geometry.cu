@@ -1,7 +1,8 @@
 // Geometry kernels of the integration step, batched over the frames of a batch
 // (they only read the map):
 //   Sec. III-A  masked depth -> world points -> voxel keys and pixel normals;
-//               per-segment voxel sets V_m in the frame slot's hash
+//               per-segment voxel sets V_m as records by key partition, each
+//               partition gathered into distinct entries
 //   Eq. 3       per voxel max(0, -r_v . n_v), summed exactly per segment
 //   Sec. III-B  label of every voxel in the map as it stood at the start of
 //               the batch (voxels absent then are re-probed by the serial
@@ -105,9 +106,9 @@ __global__ void k_slot_reset(BatchScratch bs, int B)
 // and counter increments, one line per lane (L1 70 % busy).  Measured on Room
 // frames (640x480, 2.5 cm voxels, 8 frames per launch) in place of one global
 // (segment, voxel) hash per frame with 32-byte slots, whose probes and three
-// 64-bit atomics per key missed L2: 18.1 -> 7.2 us per frame, and 2.6 -> 0.3 us
-// for clearing the slot; with k_entries (4.5 -> 5.6 us, they now also sum the
-// pixels) 25.2 -> 13.1 us.  The partition counters lie a cache line apart: side
+// 64-bit atomics per key missed L2: 18.1 -> 7.3 us per frame, and 2.6 -> 0.3 us
+// for clearing the slot; with k_entries (4.5 -> 5.3 us, they now also sum the
+// pixels) 25.2 -> 12.9 us.  The partition counters lie a cache line apart: side
 // by side (8 to a sector) the kernel took 28.8 us.
 constexpr int BP_TX = 32, BP_TY = 16, BP_PER = 2;      // tile; pixels per thread (rows 2 ty and 2 ty + 1)
 constexpr int BP_ROWS = BP_TY / BP_PER, BP_THREADS = BP_TX * BP_ROWS;
