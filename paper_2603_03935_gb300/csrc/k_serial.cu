@@ -1120,7 +1120,8 @@ __global__ void k_serial_begin(const MapRefs* refs, int G)
 // absent entries into (b) and (c).  Each frame is left with a few hundred
 // to a few thousand items, (m, label) and (m, j0, m0), with voxel counts.
 // k_associate then runs each map's frames in order in one CTA (overlap pairs
-// from the items, the gates, the union, fusion and the voxel counts), and
+// from the items, the gates, the union, fusion and the voxel counts; a
+// cluster's other CTAs take crowded frames' pairs and copies), and
 // k_commit inserts the batch's new voxels with their first frame's labels and
 // flattens the parent tables.  A frame that fails inserts nothing, and the
 // frames after it in its map are blocked.
