@@ -232,7 +232,7 @@ __host__ size_t gemm_smem_bytes(int NT, int precision, bool bf16_tokens, int KS,
     return b + 128;
 }
 static_assert(2 * gemm_stage_bytes(MAX_MASKS, DISC_FP32, false) + 128 <= GEMM_SMEM, "the largest stage pair fits an SM");
-static_assert((size_t)GEMM_COLS * GEMM_MT * 4 + 128 <= GEMM_SMEM, "so do the partial sums of a group");
+static_assert((size_t)MAX_MASKS * GEMM_MT * 4 + 128 <= GEMM_SMEM, "so do the partial sums of a group");
 
 // Test hook: when set, the kernel issues no MMA and no commit, so its bounded
 // waits run out and the frame fails with DISC_ERR_TIMEOUT (nothing is in
@@ -568,10 +568,42 @@ __global__ void __launch_bounds__(GEMM_THREADS, 2) k_pool_gemm(const FrameParams
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(ncols) : "memory");
 }
 
-template <typename T, int PR>
-static void launch_gemm_as(const FrameParams* fps, const BatchScratch& bs, int tiles, int B, int NT, int KS,
-                           int groups, cudaStream_t st)
+// CTAs per tile. A CTA costs its chunks and as much as four more (set-up, the
+// exchange of partial sums, the result), and the CTAs run in waves: one per SM,
+// or two where their shared memory lets them, which take 1.4 times as long. That
+// orders what was measured, us for 1 | 4 | 8 | 12 | 16 | 32 frames: Room with 8
+// CTAs per tile 15.5 | 19.3 | 28.7 | 35.9 | 44.1 | 79, with 4 19.4 | 19.4 | 25.5 |
+// 25.5 | 37.8 | 59, with 2 27 | 27 | 27.5 | 29.7 | 37.4 | 54, with one 39 | 39 |
+// 40 | 40 | 40 | 54; 200 masks in fp32 (a CTA per SM) with 8 25 | 44 | 79 | 99 |
+// 136 | -, with 4 36 | 36 | 64 | 65 | 94 | 159, with one 77 | 77 | 78 | 79 | 79 |
+// 158. An SM partition may be too small or too scattered to hold a cluster.
+static int gemm_split(int NT, int precision, bool bf16_tokens, int groups, int chunks, int tiles, int B, bool clusters)
 {
+    int best = 1, least = 0;
+    for (int KS = 1; KS <= (clusters ? groups : 1); KS *= 2) {
+        const int cols = gemm_columns(NT, KS, groups);
+        if (cols > 2 * GEMM_COLS || (KS > 1 && (size_t)(groups / KS) * NT * GEMM_MT * 4 + 128 > GEMM_SMEM)) continue;
+        const bool two = 2 * (gemm_smem_bytes(NT, precision, bf16_tokens, KS, groups) + 128 + 1024) <= SMEM_MAX + 1024;
+        const int ctas = KS * tiles * B, left = ctas % 304;
+        const int waves = two ? ctas / 304 * 7 + (left > 152 ? 7 : left > 0 ? 5 : 0) : (ctas + 151) / 152 * 5;  // in fifths
+        const int cost = waves * ((chunks + KS - 1) / KS + 4);
+        if (KS == 1 || cost < least) {
+            best = KS;
+            least = cost;
+        }
+    }
+    return best;
+}
+
+template <typename T, int PR>
+static void launch_gemm_as(const FrameParams* fps, const BatchScratch& bs, int tiles, int B, int NT, int chunks,
+                           bool clusters, cudaStream_t st)
+{
+    // How the patches are grouped depends on their number alone: two chunks to
+    // a group at least, eight groups at most.
+    int groups = 1;
+    while (groups < GEMM_GROUPS && 4 * groups <= chunks) groups *= 2;
+    const int KS = gemm_split(NT, PR, sizeof(T) == 2, groups, chunks, tiles, B, clusters);
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeClusterDimension;
@@ -593,32 +625,13 @@ int launch_pool_gemm(const FrameParams* fps, const BatchScratch& bs, int B, int 
     if (Mmax <= 0) return 0;
     const int NT = std::max(16, (Mmax + 15) / 16 * 16);
     const int tiles = (D + GEMM_MT - 1) / GEMM_MT, chunks = (P + GEMM_KC - 1) / GEMM_KC;
-    // How the patches are grouped depends on their number alone: two chunks to
-    // a group at least, eight groups at most.
-    int groups = 1;
-    while (groups < GEMM_GROUPS && 4 * groups <= chunks) groups *= 2;
-    // A small batch takes a CTA per group, or one per two groups, a large one
-    // a CTA per tile, without the exchange of partial sums (below): us for 1 |
-    // 4 | 8 | 16 | 32 Room frames with 8 CTAs per tile 15.5 | 19.3 | 28.7 |
-    // 44.1 | 79, with 4 19.4 | 19.4 | 25.5 | 37.8 | 59, with one 39 | 39 | 40 |
-    // 40 | 54.  Above 128 masks a CTA of two groups or of a whole tile has an
-    // SM to itself: 200 masks in fp32, 8 | 12 | 16 frames, with 4 CTAs 64 | 65 |
-    // 94, with one 78 | 79 | 79.  An SM partition may be too small or too
-    // scattered to hold a cluster.
-    int KS = 1;
-    if (clusters) {
-        const int most = 2 * NT <= GEMM_COLS ? 400 : 304;
-        const bool two = groups == 8 && 2 * (size_t)NT * GEMM_MT * 4 + 128 <= GEMM_SMEM;  // two groups to a CTA
-        if (groups * tiles * B <= (two ? 152 : most)) KS = groups;
-        else if (two && 4 * tiles * B <= most) KS = 4;
-    }
     int n = 0;
-    if (any[0][0]) { launch_gemm_as<float, DISC_FP32>(fps, bs, tiles, B, NT, KS, groups, st); n++; }
-    if (any[1][0]) { launch_gemm_as<__nv_bfloat16, DISC_FP32>(fps, bs, tiles, B, NT, KS, groups, st); n++; }
-    if (any[0][1]) { launch_gemm_as<float, DISC_BF16>(fps, bs, tiles, B, NT, KS, groups, st); n++; }
-    if (any[1][1]) { launch_gemm_as<__nv_bfloat16, DISC_BF16>(fps, bs, tiles, B, NT, KS, groups, st); n++; }
-    if (any[0][2]) { launch_gemm_as<float, DISC_FP8_E4M3>(fps, bs, tiles, B, NT, KS, groups, st); n++; }
-    if (any[1][2]) { launch_gemm_as<__nv_bfloat16, DISC_FP8_E4M3>(fps, bs, tiles, B, NT, KS, groups, st); n++; }
+    if (any[0][0]) { launch_gemm_as<float, DISC_FP32>(fps, bs, tiles, B, NT, chunks, clusters, st); n++; }
+    if (any[1][0]) { launch_gemm_as<__nv_bfloat16, DISC_FP32>(fps, bs, tiles, B, NT, chunks, clusters, st); n++; }
+    if (any[0][1]) { launch_gemm_as<float, DISC_BF16>(fps, bs, tiles, B, NT, chunks, clusters, st); n++; }
+    if (any[1][1]) { launch_gemm_as<__nv_bfloat16, DISC_BF16>(fps, bs, tiles, B, NT, chunks, clusters, st); n++; }
+    if (any[0][2]) { launch_gemm_as<float, DISC_FP8_E4M3>(fps, bs, tiles, B, NT, chunks, clusters, st); n++; }
+    if (any[1][2]) { launch_gemm_as<__nv_bfloat16, DISC_FP8_E4M3>(fps, bs, tiles, B, NT, chunks, clusters, st); n++; }
     return n;
 }
 
