@@ -1,7 +1,6 @@
 """The tensor-core pooled embedding at the edges of its tiles and of the split
 of the patches over a cluster: against the exact one, within 1e-5 of its norm
-per mask at FP32 precision and within the bound the gate uses at BF16 and FP8;
-on an SM partition too small for clusters; and the same bits in every batch."""
+per mask at FP32 precision and within the bound the gate uses at BF16 and FP8."""
 import numpy as np
 import pytest
 
